@@ -41,8 +41,9 @@ __device__ __forceinline__ vec<T, V> ldv_if(bool ok, const T* p) {
 // any memory, until the predecessor has completed and its writes are
 // visible, and at once allows its own successor to be scheduled (which in
 // turn waits).  Both are no-ops for an ordinary launch.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_enter() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  pdl_wait();
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 

@@ -529,6 +529,16 @@ void set_gemm_wait_limit(long long polls);
 // tensor map; CMG_GEMM_TMA=0).
 cudaError_t launch_conv3x3_bf16(const void* X, int B, int H, int W, int C, const void* Wt, int Cout,
                                 const float* bias, int relu, void* Y16, int* status, cudaStream_t s);
+// The same convolution for C = 8, 32 or 64 and Cout <= 64 with the input patch
+// of each tile in shared memory (cmg_nn_conv.cu; the same bits).  turned: Wt is
+// the forward weights [C][9 Cout] of the layer whose data gradient this is
+// (taps turned by 180 degrees, channels exchanged, as cmg_nn_flip3x3 would;
+// C = 32 or 64, Cout % 8 == 0).  early: Wt and bias were not written by a
+// kernel that lets its successors start early (pdl_enter), so they may be read
+// while the stream's preceding kernel runs.  cudaErrorNotSupported outside that.
+cudaError_t launch_conv3x3_patch(const void* X, int B, int H, int W, int C, const void* Wt, int Cout,
+                                 const float* bias, int relu, int turned, void* Y16, int* status, cudaStream_t s,
+                                 int early = 0);
 cudaError_t launch_gemm_bf16_tn(const void* A, long lda, const void* B, long ldb, int M, int N, int K,
                                 const float* bias, int relu, float* C32, void* C16, int ldc, int* status,
                                 cudaStream_t s, int ksplit = 1);

@@ -54,7 +54,7 @@
 #include <cstdlib>
 #include <mutex>
 
-#include "cmg_internal.h"
+#include "cmg_nn_mma.cuh"
 
 namespace cmg {
 namespace nn {
@@ -63,88 +63,7 @@ constexpr int kBM = 128, kBN = 64, kBK = 64;
 constexpr int kThreads = 128;
 constexpr int kStages = 4;
 constexpr uint32_t kTmemCols = 64;                 // FP32 accumulator columns (= kBN)
-constexpr long kSpinLimit = 1L << 22;              // mbarrier polls before giving up
 constexpr int kSmemBytes = kStages * (kBM + kBN) * kBK * 2;   // 96 KiB of operand tiles
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-// tcgen05 shared-memory matrix descriptor: start address, leading (K
-// direction) and stride (M/N direction) byte offsets, descriptor version 1,
-// no swizzle.
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
-  uint64_t d = 0;
-  d |= (uint64_t)((addr & 0x3FFFF) >> 4);
-  d |= (uint64_t)((lbo >> 4) & 0x3FFF) << 16;
-  d |= (uint64_t)((sbo >> 4) & 0x3FFF) << 32;
-  d |= (uint64_t)1 << 46;
-  return d;
-}
-
-// K-major tile written by TMA with the 64-byte swizzle: rows of 64 bytes
-// (32 BF16 of K), 8-row groups 512 bytes apart, layout type 4 (64-byte
-// swizzle); the tile base is 512-byte aligned, so a K step of 16 inside the
-// 64-byte row advances the start address by 32 bytes.
-__device__ __forceinline__ uint64_t smem_desc_sw64(uint32_t addr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((addr & 0x3FFFF) >> 4);
-  d |= (uint64_t)1 << 16;
-  d |= (uint64_t)(512 >> 4) << 32;
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)4 << 61;
-  return d;
-}
-
-// The same descriptor for a K-major tile written by TMA with the 128-byte
-// swizzle: rows of 128 bytes (64 BF16 of K), 8-row groups 1024 bytes apart
-// (stride byte offset), layout type 2 (128-byte swizzle) in bits 61-63; the
-// leading byte offset is unused for this layout.  The tile base is 1024-byte
-// aligned, so a K step of 16 inside the 128-byte row advances the start
-// address by 32 bytes.
-__device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((addr & 0x3FFFF) >> 4);
-  d |= (uint64_t)1 << 16;
-  d |= (uint64_t)(1024 >> 4) << 32;
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)2 << 61;
-  return d;
-}
-
-// Instruction descriptor, kind::f16: FP32 accumulate, A and B BF16, both
-// K-major, N and M of the MMA.
-__host__ __device__ constexpr uint32_t instr_desc(int M, int N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
-}
-
-// Wait for phase `parity` of the mbarrier; false if the poll limit expires
-// or, when `abort` is given, once another thread has set it.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, const volatile int* abort = nullptr,
-                                          long long limit = kSpinLimit) {
-  const uint32_t a = smem_u32(bar);
-  for (long long i = 0; i < limit; ++i) {
-    uint32_t done;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(done)
-        : "r"(a), "r"(parity)
-        : "memory");
-    if (done) return true;
-    if (abort && *abort) return false;
-  }
-  return false;
-}
-
-// Arrive on the barrier and add `bytes` to the transaction count its phase
-// waits for (the TMA loads of one stage).
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
 
 // TMA load of one box of a 3-D tensor map at coordinates (c0, c1, c2),
 // completing on `bar` with the box's byte count.  c0 (the K coordinate) is
@@ -172,20 +91,6 @@ __device__ __forceinline__ void tma_load_im2col(void* dst, const CUtensorMap* ma
       : "memory");
 }
 
-__device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                         uint32_t accumulate) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-
-__device__ __forceinline__ void mma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-               : "memory");
-}
-
 // Asynchronous copy of a rows x 64 BF16 tile (row stride ld elements) into
 // the core-matrix layout; rows beyond `valid` and columns beyond K are
 // zero-filled (K % 8 == 0).  The source of a zero-filled chunk is the
@@ -201,10 +106,6 @@ __device__ __forceinline__ void load_tile_async(__nv_bfloat16* dst, const __nv_b
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(g), "r"(ok ? 16 : 0) : "memory");
   }
 }
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
 // Epilogue of one warp: rows m0 + 32 warp + lane of C, `chunks` blocks of
 // 32 accumulator columns (TMEM columns 32c.., C columns n0 + 32c..), bias,
 // ReLU, FP32 and/or BF16 stores.  Called by all 32 lanes together.
@@ -823,6 +724,10 @@ int pick_bn(int M, int N) {
 // Poll limit of the TMA kernel's work waits (0: kSpinLimit); see
 // cmg_nn_set_wait_limit.
 std::atomic<long long> g_wait_limit{0};
+long long wait_limit() {
+  const long long w = g_wait_limit.load(std::memory_order_relaxed);
+  return w > 0 ? w : (long long)kSpinLimit;
+}
 
 template <int BN, int S, int AM = 0>
 cudaError_t launch_tma(const CUtensorMap& mA, const CUtensorMap& mB, int M, int N, int K, const float* bias, int relu,
@@ -840,10 +745,9 @@ cudaError_t launch_tma(const CUtensorMap& mA, const CUtensorMap& mB, int M, int 
   if (tiles > 0x7fffffffL) return cudaErrorInvalidValue;
   const int sms = sm_count();
   const unsigned grid = (unsigned)(tiles < sms ? tiles : (sms > 0 ? sms : 1));   // persistent: one CTA per SM
-  const long long wl = g_wait_limit.load(std::memory_order_relaxed);
   gemm_bf16_tn_tma_kernel<BN, S, AM><<<grid, kTmaThreads, TmaTile<BN, S>::kSmem, s>>>(
       mA, mB, M, N, K, bias, relu, C32, C16, ldc, status, vec16, vec32, mtiles, ntiles, (int)tiles,
-      wl > 0 ? wl : (long long)kSpinLimit, geo);
+      wait_limit(), geo);
   return cudaGetLastError();
 }
 
@@ -861,6 +765,10 @@ cudaError_t launch_conv3x3_bf16(const void* X, int B, int H, int W, int C, const
   const int cpp = C % 64 == 0 ? 64 : C % 32 == 0 ? 32 : (C % 8 == 0 && C < 32) ? 8 : 0;
   if (!cpp || Cout < 1 || Cout > 64 || P < 1 || P > 0x7fffffffL || 9L * C > 0x7fffffffL)
     return cudaErrorNotSupported;
+  // the network's channel counts: the patch kernel, which reads each pixel 1.4
+  // times instead of nine
+  const cudaError_t pe = launch_conv3x3_patch(X, B, H, W, C, Wt, Cout, bias, relu, 0, Y16, status, s);
+  if (pe != cudaErrorNotSupported) return pe;
   const int K = 9 * C;
   CUtensorMap mA, mB;
   if (!nn::im2col_map(&mA, X, B, H, W, C, cpp) || !nn::operand_map(&mB, Wt, K, Cout, K, 1, 64))

@@ -167,10 +167,8 @@ cmg_status conv_forward(cmg_unet* u, int layer, const void* X, void* Y, int B) {
   const int H = u->S >> c.level;
   const long P = pixels(u, B, c.level);
   const Param& p = u->prm[layer];
-  // implicit GEMM (the tensor cores read X through an im2col tensor map);
-  // im2col + GEMM where it does not apply (same results)
-  const cmg_status st = cmg_nn_conv3x3_bf16(X, B, H, H, c.ci, p.w16, c.co, p.b, 1, Y, u->status, u->stream);
-  if (st != CMG_ERR_UNSUPPORTED) return st == CMG_OK ? CMG_OK : fail(u, st, "layer call: cmg_nn_conv3x3_bf16");
+  const cudaError_t e = launch_conv3x3_patch(X, B, H, H, c.ci, p.w16, c.co, p.b, 1, 0, Y, u->status, u->stream, 1);
+  if (e != cudaErrorNotSupported) return e == cudaSuccess ? CMG_OK : cuda_fail(u, e, "convolution");
   NN(cmg_nn_im2col(X, u->col, B, H, H, c.ci, 0, u->stream));
   NN(cmg_nn_gemm_bf16(u->col, 9 * c.ci, p.w16, 9 * c.ci, (int)P, c.co, 9 * c.ci, p.b, 1, nullptr, Y, c.co, u->status,
                       u->stream));
@@ -194,11 +192,10 @@ cmg_status conv_backward(cmg_unet* u, int layer, const void* X, const void* Y, c
                              u->stream));
   NN(cmg_nn_sum_slices(u->part, nsl, p.gw, (long long)c.co * 9 * c.ci, u->stream));
   if (!dX) return CMG_OK;
-  // dX as a 3x3 convolution of dZ with the turned weights (implicit GEMM, no
-  // patch-gradient matrix); else dZ W into patches and col2im
-  NN(cmg_nn_flip3x3(p.w16, u->WT, c.co, c.ci, u->stream));
-  const cmg_status st = cmg_nn_conv3x3_bf16(u->dZ, B, H, H, c.co, u->WT, c.ci, nullptr, 0, dX, u->status, u->stream);
-  if (st != CMG_ERR_UNSUPPORTED) return st == CMG_OK ? CMG_OK : fail(u, st, "layer call: cmg_nn_conv3x3_bf16");
+  // dX as a 3x3 convolution of dZ with the turned weights
+  const cudaError_t e = launch_conv3x3_patch(u->dZ, B, H, H, c.co, p.w16, c.ci, nullptr, 0, 1, dX, u->status,
+                                             u->stream, 1);
+  if (e != cudaErrorNotSupported) return e == cudaSuccess ? CMG_OK : cuda_fail(u, e, "data-gradient convolution");
   NN(cmg_nn_transpose(p.w16, u->WT, c.co, 9 * c.ci, u->stream));
   NN(cmg_nn_gemm_bf16(u->dZ, c.co, u->WT, c.co, (int)P, 9 * c.ci, c.co, nullptr, 0, u->dcol, nullptr, 9 * c.ci,
                       u->status, u->stream));

@@ -1,0 +1,36 @@
+"""The patch convolution (cmg_nn_conv.cu) where its 8 x 16 pixel tiles, its
+channel padding and its stores can go wrong: images smaller than a tile,
+ragged in both directions, exactly one tile, single rows and columns, output
+counts that leave 16-byte chunks, sectors or the MMA width unfilled, no bias.
+The same products are summed in the same order as by im2col + GEMM, so the
+results are the same bits; rows past the output stay untouched."""
+import ctypes
+
+import pytest
+import torch
+
+from test_gpu_nn_conv import data, lib, ptr  # noqa: F401  (module fixture)
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("C", [8, 32, 64])
+@pytest.mark.parametrize("B,H,W,Cout", [(1, 1, 1, 5), (3, 16, 8, 32), (2, 17, 9, 64), (1, 15, 23, 24), (2, 33, 7, 40),
+                                        (1, 2, 50, 1), (1, 129, 65, 48), (40, 48, 24, 33)])
+def test_patch_conv_edges(lib, B, H, W, C, Cout):  # noqa: F811
+    X, Wt, bias = data(B, H, W, C, Cout, seed=H * 100 + W + C + Cout)
+    P = B * H * W
+    Xd, Wd, bd = X.cuda(), Wt.cuda(), (bias.cuda() if Cout % 3 else None)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    s = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    Y = torch.full((P + 4, Cout), 7.0, dtype=torch.bfloat16, device="cuda")
+    assert lib.cmg_nn_conv3x3_bf16(ptr(Xd), B, H, W, C, ptr(Wd), Cout, ptr(bd), 1, ptr(Y), ptr(status), s) == 0
+    col = torch.empty(P, 9 * C, dtype=torch.bfloat16, device="cuda")
+    Y2 = torch.empty(P, Cout, dtype=torch.bfloat16, device="cuda")
+    assert lib.cmg_nn_im2col(ptr(Xd), ptr(col), B, H, W, C, 0, s) == 0
+    assert lib.cmg_nn_gemm_bf16(ptr(col), 9 * C, ptr(Wd), 9 * C, P, Cout, 9 * C, ptr(bd), 1, None, ptr(Y2), Cout,
+                                ptr(status), s) == 0
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    assert torch.equal(Y[:P], Y2)
+    assert bool((Y[P:] == 7.0).all())
