@@ -539,6 +539,36 @@ cudaError_t launch_conv3x3_bf16(const void* X, int B, int H, int W, int C, const
 cudaError_t launch_conv3x3_patch(const void* X, int B, int H, int W, int C, const void* Wt, int Cout,
                                  const float* bias, int relu, int turned, void* Y16, int* status, cudaStream_t s,
                                  int early = 0);
+// Weight gradient of the 3x3 layer C -> Cout (C = 8, 32, 64, Cout = 32, 64) as
+// per-slice partial sums part[slices][Cout][9 C] (at most wgrad_max_slices
+// of them), added by launch_finish_layer.
+long wgrad_max_slices(int B, int H, int W);
+cudaError_t launch_conv3x3_wgrad(const void* X, const void* dZ, int B, int H, int W, int C, int Cout, float* part,
+                                 int* slices, int* status, cudaStream_t s);
+
+// Gradient dZ of a layer's sums before its ReLU, from the gradient of its
+// output y [B][H][W][C] (C = 32 or 64): dZ = v where y > 0, else 0, with v
+//   kGradDirect    dA
+//   kGradUpsample  the 2 x 2 sums of dA [B][2H][2W][C] (nearest upsampling's gradient)
+//   kGradPoolSkip  dA [B][H/2][W/2][C] / 4 (average pooling's gradient) + dB (the skip's)
+//   kGradHead      dA[p] w[c], dA [B][H][W] the gradient of the 1x1 head's output
+// each step rounded to BF16 as the separate layers are, and the column sums:
+// rows[block][width] partials of the sum of dZ over the pixels (the bias
+// gradient), for the head followed by sums of dA y (its weight gradient)
+// and dA.  Returns the rows in *nrows (<= kGradRows).
+enum GradMode { kGradDirect = 0, kGradUpsample = 1, kGradPoolSkip = 2, kGradHead = 3 };
+constexpr int kGradRows = 152 * 4;
+cudaError_t launch_grad_act(int mode, const void* y, const void* dA, const void* dB, const float* w, void* dZ, int B,
+                            int H, int W, int C, float* rows, int* nrows, cudaStream_t s);
+// gw[n] = sum of part[slices][n], gb[c] = sum of rows[nrows][width] for c < C
+// (and, given hw / hb, the head's weight and bias gradients from the columns
+// after that), fixed order.
+cudaError_t launch_finish_layer(const float* part, int slices, float* gw, int n, const float* rows, int nrows, int width,
+                                float* gb, int C, float* hw, float* hb, cudaStream_t s);
+// out[p] = sum_c X[p][c] w16[c] + b[0] over 32 channels (the 1x1 head), FP32; also
+// to out2 when given.
+cudaError_t launch_head(const void* X, const void* w16, const float* b, long P, float* out, float* out2, int* status,
+                        cudaStream_t s);
 cudaError_t launch_gemm_bf16_tn(const void* A, long lda, const void* B, long ldb, int M, int N, int K,
                                 const float* bias, int relu, float* C32, void* C16, int ldc, int* status,
                                 cudaStream_t s, int ksplit = 1);

@@ -32,6 +32,7 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "cmg_common.cuh"
@@ -135,6 +136,22 @@ __device__ __forceinline__ void st32(void* p, const uint32_t* v) {
   asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]),
                "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
                : "memory");
+}
+
+// One warp brings 128 pixels of C8 channel groups into planes of pitch
+// `pitch`; where(px, src) gives pixel px's address, or false for zeros.
+template <int C8, typename Where>
+__device__ __forceinline__ void load_pixels(uint32_t dst, uint32_t pitch, const __nv_bfloat16* __restrict__ X, int lane,
+                                            Where where) {
+  constexpr int kStep = 32 / C8;
+  const int c8 = lane % C8, px0 = lane / C8;
+#pragma unroll 4
+  for (int i = 0; i < 128 / kStep; ++i) {
+    const int px = px0 + i * kStep;
+    long p;
+    const bool ok = where(px, p);
+    cp16(dst + c8 * pitch + px * 16, ok ? X + p * (C8 * 8) + c8 * 8 : X, ok);
+  }
 }
 
 template <int C, int NP>
@@ -377,8 +394,334 @@ cudaError_t launch_patch(const __nv_bfloat16* X, const Tiles& g, const __nv_bflo
   return e;
 }
 
+// ---- weight gradient -------------------------------------------------------
+//
+// gw[co][t C + c] = sum over pixels p of dZ[p][co] X[p shifted by tap t][c].
+// The contraction runs over pixels, so both operands are MN-major: dZ of a
+// tile as planes of 16-byte chunks (8 output channels of a pixel), X as the
+// forward kernel's patch, eight pixels of an image row being a core matrix;
+// a tap again is a start address.  An MMA of 64 x C x 16 takes two image rows
+// of the tile; a CTA sums a slice of at most 32 tiles (4096 pixels, the depth
+// of the FP32 accumulation) into one accumulator of C columns per tap, and the
+// slices are added in a fixed order by finish_layer (cmg_nn_ops.cu).
+//
+// Why: the GEMM form needed dZ transposed and the patch matrix transposed
+// ([9 C][pixels], 302 MB at 256^2, batch 8), which took ten times the
+// multiplications' time: 320 us of transposing per layer on average and 63 us
+// of GEMM.  Here X and dZ are read once (twice for C = 64, whose nine
+// accumulators exceed the 512 TMEM columns: five taps in one CTA, four in
+// another).  256^2 32->32, batch 8: 67 us in all; 128^2 64->64 31 us.  Bound by
+// the tensor cores' operand reads (3 to 4 KB per MMA of 64 x C x 16).
+template <int C, int CO>
+struct WgradTile {
+  static constexpr int C8 = C / 8, CO8 = CO / 8;
+  static constexpr int kTaps = C == 64 ? 5 : 9;              // taps of a CTA
+  static constexpr int kGroups = (9 + kTaps - 1) / kTaps;
+  static constexpr uint32_t kPitch = patch_pitch(C8);
+  static constexpr uint32_t kPitchZ = (CO8 == 8 ? 129u : 130u) * 16u;   // 128 pixels
+  static constexpr uint32_t kZ = CO8 * kPitchZ;
+  static constexpr uint32_t kStage = kZ + C8 * kPitch;
+  static constexpr int S = 4;
+  // the MMA's 64 rows read eight planes of dZ; with CO = 32 the last four are whatever follows (rows not stored)
+  static constexpr uint32_t kSlack = CO8 < 8 ? 4 * kPitchZ : 0;
+  static constexpr int kUse = (int)(S * kStage + kSlack);
+  static constexpr int kSmem = kUse > 116 * 1024 ? kUse : 116 * 1024;   // one CTA per SM (TMEM)
+  static constexpr uint32_t kCols = kTaps * C <= 128 ? 128 : 512;
+  static_assert(kTaps * C <= (int)kCols && kSmem <= 227 * 1024, "TMEM and shared memory");
+};
+constexpr int kWgThreads = kProd + 32 + 128;
+
+template <int C, int CO>
+__global__ void __launch_bounds__(kWgThreads, 1)
+    conv3x3_wgrad_kernel(const __nv_bfloat16* __restrict__ X, const __nv_bfloat16* __restrict__ dZ, Tiles g, int per,
+                         float* __restrict__ part, int* __restrict__ status, long long wlimit) {
+  using T = WgradTile<C, CO>;
+  constexpr int C8 = T::C8, CO8 = T::CO8, S = T::S;
+  extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ __align__(8) uint64_t full[S], done[S], fin;
+  __shared__ uint32_t tmem_base;
+  __shared__ volatile int failed;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t s0 = smem_u32(smem);
+  const int z = blockIdx.x, tap0 = blockIdx.y * T::kTaps, taps = tap0 + T::kTaps < 9 ? T::kTaps : 9 - tap0;
+  const int first = z * per, last = first + per < g.count ? first + per : g.count;
+
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
+                 "r"(T::kCols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  if (threadIdx.x == 32) {
+    for (int s = 0; s < S; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&done[s], 1);
+    }
+    mbar_init(&fin, 1);
+    failed = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = tmem_base;
+  pdl_enter();
+
+  if (warp < kProd / 32) {
+    for (int it = warp, t = first + warp; t < last; it += 4, t += 4) {
+      const int s = it % S;
+      int b, y0, x0;
+      tile_pos(g, t, b, y0, x0);
+      if (it >= S && !mbar_wait(&done[s], (uint32_t)((it / S - 1) & 1), &failed, wlimit)) failed = 1;
+      if (__any_sync(0xffffffffu, failed)) break;
+      const uint32_t dz = s0 + s * T::kStage;
+      load_pixels<CO8>(dz, T::kPitchZ, dZ, lane, [&](int px, long& p) {
+        const int gy = y0 + px / kPW, gx = x0 + px % kPW;
+        p = ((long)b * g.H + gy) * g.W + gx;
+        return gy < g.H && gx < g.W;
+      });
+      load_patch<C8>(dz + T::kZ, T::kPitch, X, g, b, y0, x0, lane);
+      cp_commit();
+      cp_wait<0>();
+      fence_async();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&full[s]);
+    }
+  } else if (warp == kProd / 32) {
+    const uint32_t idesc = instr_desc(64, C) | 1u << 15 | 1u << 16;   // both operands MN-major
+    const uint32_t ahi = desc_hi(T::kPitchZ), bhi = desc_hi(T::kPitch);
+    if (lane == 0) {
+      int it = 0;
+      for (int t = first; t < last && !failed; ++t, ++it) {
+        const int s = it % S;
+        if (!mbar_wait(&full[s], (uint32_t)((it / S) & 1), &failed, wlimit)) {
+          failed = 1;
+          break;
+        }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t al = desc_lo(s0 + s * T::kStage, 128), bl = desc_lo(s0 + s * T::kStage + T::kZ, kIW * 16);
+#pragma unroll 1
+        for (int k = 0; k < taps; ++k) {
+          const int t9 = tap0 + k, toff = t9 + (kIW - 3) * (t9 / 3);   // 10 dy + dx
+#pragma unroll
+          for (int j = 0; j < kPH / 2; ++j)
+            mma_bf16(tmem + k * C, al + j * 16, ahi, bl + toff + j * 2 * kIW, bhi, idesc, it > 0 || j > 0);
+        }
+        mma_commit(&done[s]);
+      }
+      mma_commit(&fin);   // completes once every MMA issued above has completed
+      if (!mbar_wait(&fin, 0)) failed = 1;
+    }
+  } else {
+    const int q = warp & 3;
+    const bool ok = __all_sync(0xffffffffu, mbar_wait(&fin, 0, &failed, wlimit > kSpinLimit ? wlimit : kSpinLimit));
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (ok && !failed) {
+      // M = 64: row 16 q + l of the product in lane l < 16 of quadrant q
+      const int co = q * 16 + lane;
+      float* row = part + ((long)z * CO + co) * (9 * C) + tap0 * C;
+#pragma unroll 1
+      for (int c0 = 0; c0 < taps * C; c0 += 8) {
+        uint32_t r[8];
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                     : "r"(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0)
+                     : "memory");
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        if (lane < 16 && co < CO) st32(row + c0, r);
+      }
+    }
+  }
+  __syncwarp();
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(T::kCols) : "memory");
+  if (failed && threadIdx.x == 0) atomicExch(status, 1);
+}
+
+// ---- 1x1 head ---------------------------------------------------------------
+//
+// out[p] = sum_c X[p][c] w[c] + bias over C = 32 channels, one output: two MMAs
+// of 128 x 16 x 16 per 128 pixels (the sums of the 64-wide GEMM, bit for bit),
+// bound by reading X.  The GEMM (cmg_nn_gemm.cu) took 34 us for 256^2, batch 8,
+// moving 32 output columns through its transposing epilogue for one.
+constexpr int kHeadN = 16, kHeadS = 4;
+constexpr uint32_t kHeadPitch = 130 * 16, kHeadStage = 4 * kHeadPitch;
+constexpr int kHeadSmem = (int)(kHeadS * kHeadStage + 4 * kHeadN * 16);
+
+__global__ void __launch_bounds__(kWgThreads)
+    head1x1_kernel(const __nv_bfloat16* __restrict__ X, const __nv_bfloat16* __restrict__ w,
+                   const float* __restrict__ bias, long P, long tiles, float* __restrict__ out, float* __restrict__ out2,
+                   int* __restrict__ status, long long wlimit) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ __align__(8) uint64_t full[kHeadS], done[kHeadS], acc_empty[kHeadS];
+  __shared__ uint32_t tmem_base;
+  __shared__ volatile int failed;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t sA = smem_u32(smem), sB = sA + kHeadS * kHeadStage;
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
+                 "r"(kHeadS * kHeadN)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  if (threadIdx.x == 32) {
+    for (int s = 0; s < kHeadS; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&done[s], 1);
+      mbar_init(&acc_empty[s], 4);
+    }
+    failed = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  pdl_wait();
+  // weight plane k8: row 0 the weights, rows 1 .. 15 zero
+  if (threadIdx.x < 4 * kHeadN) {
+    const int k8 = threadIdx.x / kHeadN, n = threadIdx.x % kHeadN;
+    *reinterpret_cast<uint4*>(smem + kHeadS * kHeadStage + threadIdx.x * 16) =
+        n == 0 ? *reinterpret_cast<const uint4*>(w + k8 * 8) : make_uint4(0, 0, 0, 0);
+  }
+  fence_async();
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = tmem_base;
+  pdl_enter();
+
+  if (warp < kProd / 32) {
+    long t = (long)blockIdx.x + (long)warp * gridDim.x;
+    for (int it = warp; t < tiles; it += 4, t += 4L * gridDim.x) {
+      const int s = it % kHeadS;
+      if (it >= kHeadS && !mbar_wait(&done[s], (uint32_t)((it / kHeadS - 1) & 1), &failed, wlimit)) failed = 1;
+      if (__any_sync(0xffffffffu, failed)) break;
+      load_pixels<4>(sA + s * kHeadStage, kHeadPitch, X, lane, [&](int px, long& p) {
+        p = t * 128 + px;
+        return p < P;
+      });
+      cp_commit();
+      cp_wait<0>();
+      fence_async();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&full[s]);
+    }
+  } else if (warp == kProd / 32) {
+    if (lane == 0) {
+      const uint32_t idesc = instr_desc(128, kHeadN), hi = desc_hi(128);
+      int it = 0;
+      for (long t = blockIdx.x; t < tiles && !failed; t += gridDim.x, ++it) {
+        const int s = it % kHeadS;
+        if ((it >= kHeadS && !mbar_wait(&acc_empty[s], (uint32_t)((it / kHeadS - 1) & 1), &failed, wlimit)) ||
+            !mbar_wait(&full[s], (uint32_t)((it / kHeadS) & 1), &failed, wlimit)) {
+          failed = 1;
+          break;
+        }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t al = desc_lo(sA + s * kHeadStage, kHeadPitch), bl = desc_lo(sB, kHeadN * 16);
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+          mma_bf16(tmem + s * kHeadN, al + 2 * j * kHeadPitch / 16, hi, bl + 2 * j * kHeadN, hi, idesc, j > 0);
+        mma_commit(&done[s]);
+      }
+      for (int j = it > kHeadS ? it - kHeadS : 0; j < it; ++j)
+        if (!mbar_wait(&done[j % kHeadS], (uint32_t)((j / kHeadS) & 1))) failed = 1;
+    }
+  } else {
+    const int q = warp & 3;
+    const float bv = bias[0];
+    int it = 0;
+    for (long t = blockIdx.x; t < tiles; t += gridDim.x, ++it) {
+      const int s = it % kHeadS;
+      if (!__all_sync(0xffffffffu, mbar_wait(&done[s], (uint32_t)((it / kHeadS) & 1), &failed, wlimit))) {
+        failed = 1;
+        break;
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      uint32_t r;
+      asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];"
+                   : "=r"(r)
+                   : "r"(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(s * kHeadN))
+                   : "memory");
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&acc_empty[s]);
+      const long p = t * 128 + q * 32 + lane;
+      if (p < P) {
+        out[p] = __uint_as_float(r) + bv;
+        if (out2) out2[p] = __uint_as_float(r) + bv;
+      }
+    }
+  }
+  __syncwarp();
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kHeadS * kHeadN) : "memory");
+  if (failed && threadIdx.x == 0) atomicExch(status, 1);
+}
+
+// Tiles per slice: an even share of the SMs, at most 32 tiles.
+int wgrad_per(long tiles, int groups) {
+  const long sms = sm_count() > 0 ? sm_count() : 1;
+  const long per = (tiles * groups + sms - 1) / sms;
+  return (int)(per < 1 ? 1 : per > 32 ? 32 : per);
+}
+
+template <int C, int CO>
+cudaError_t launch_wgrad(const __nv_bfloat16* X, const __nv_bfloat16* dZ, const Tiles& g, float* part, int* slices,
+                         int* status, cudaStream_t s) {
+  using T = WgradTile<C, CO>;
+  static std::once_flag once;
+  static cudaError_t attr = cudaSuccess;
+  std::call_once(once, [] {
+    attr = cudaFuncSetAttribute(conv3x3_wgrad_kernel<C, CO>, cudaFuncAttributeMaxDynamicSharedMemorySize, T::kSmem);
+  });
+  if (attr != cudaSuccess) return attr;
+  const int per = wgrad_per(g.count, T::kGroups);
+  *slices = (g.count + per - 1) / per;
+  const cudaError_t e = launch_k(conv3x3_wgrad_kernel<C, CO>, dim3((unsigned)*slices, T::kGroups), dim3(kWgThreads),
+                                 T::kSmem, s, X, dZ, g, per, part, status, wait_limit());
+  count_launches(1);
+  return e;
+}
+
 }  // namespace
 }  // namespace nn
+
+cudaError_t launch_head(const void* X, const void* w16, const float* b, long P, float* out, float* out2, int* status,
+                        cudaStream_t s) {
+  using namespace nn;
+  const long tiles = (P + 127) / 128, sms = sm_count() > 0 ? sm_count() : 1;
+  const unsigned grid = (unsigned)(tiles < 4 * sms ? tiles : 4 * sms);
+  const cudaError_t e = launch_k(head1x1_kernel, dim3(grid), dim3(kWgThreads), kHeadSmem, s,
+                                 static_cast<const __nv_bfloat16*>(X), static_cast<const __nv_bfloat16*>(w16), b, P,
+                                 tiles, out, out2, status, wait_limit());
+  count_launches(1);
+  return e;
+}
+
+long wgrad_max_slices(int B, int H, int W) {
+  const long tiles = (long)B * ((W + nn::kPW - 1) / nn::kPW) * ((H + nn::kPH - 1) / nn::kPH);
+  const long sms = nn::sm_count() > 0 ? nn::sm_count() : 1;
+  return std::max(sms, (tiles + 31) / 32) + 1;
+}
+
+cudaError_t launch_conv3x3_wgrad(const void* X, const void* dZ, int B, int H, int W, int C, int Cout, float* part,
+                                 int* slices, int* status, cudaStream_t s) {
+  using namespace nn;
+  Tiles g{B, H, W, (W + kPW - 1) / kPW, (H + kPH - 1) / kPH, 0};
+  const long tiles = (long)B * g.tx * g.ty;
+  if (tiles > 0x7fffffffL) return cudaErrorNotSupported;
+  g.count = (int)tiles;
+  const __nv_bfloat16 *x = static_cast<const __nv_bfloat16*>(X), *d = static_cast<const __nv_bfloat16*>(dZ);
+  if (C == 8 && Cout == 32) return launch_wgrad<8, 32>(x, d, g, part, slices, status, s);
+  if (C == 32 && Cout == 32) return launch_wgrad<32, 32>(x, d, g, part, slices, status, s);
+  if (C == 32 && Cout == 64) return launch_wgrad<32, 64>(x, d, g, part, slices, status, s);
+  if (C == 64 && Cout == 32) return launch_wgrad<64, 32>(x, d, g, part, slices, status, s);
+  if (C == 64 && Cout == 64) return launch_wgrad<64, 64>(x, d, g, part, slices, status, s);
+  return cudaErrorNotSupported;
+}
 
 cudaError_t launch_conv3x3_patch(const void* X, int B, int H, int W, int C, const void* Wt, int Cout,
                                  const float* bias, int relu, int turned, void* Y16, int* status, cudaStream_t s, int early) {

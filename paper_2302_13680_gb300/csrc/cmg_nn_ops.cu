@@ -12,7 +12,7 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
-#include "cmg_internal.h"
+#include "cmg_common.cuh"
 
 using bf16 = __nv_bfloat16;
 
@@ -243,6 +243,220 @@ __global__ void adamw_kernel(float* __restrict__ w, const float* __restrict__ g,
   }
 }
 
+// ---- eight channels (16 bytes) per thread -------------------------------------
+// The layer kernels between the convolutions move activations once, so they
+// are bound by memory; a thread takes one 16-byte chunk (8 channels of a
+// pixel) with 32-bit index arithmetic.  One channel per thread with 64-bit
+// divisions took 50 us where the bytes take 10 (upsampling to 256^2 x 32,
+// batch 8).
+struct alignas(16) B8 {
+  __nv_bfloat162 v[4];
+};
+__device__ __forceinline__ B8 ldb(const bf16* p) { return *reinterpret_cast<const B8*>(p); }
+__device__ __forceinline__ void stb(bf16* p, const B8& x) { *reinterpret_cast<B8*>(p) = x; }
+__device__ __forceinline__ void widen(const B8& x, float (&f)[8]) {
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const float2 t = __bfloat1622float2(x.v[k]);
+    f[2 * k] = t.x;
+    f[2 * k + 1] = t.y;
+  }
+}
+__device__ __forceinline__ B8 narrow(const float (&f)[8]) {
+  B8 x;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) x.v[k] = __floats2bfloat162_rn(f[2 * k], f[2 * k + 1]);
+  return x;
+}
+// Chunk i of [B][H][W][C8]: its pixel and channel group.
+struct Chunk {
+  unsigned c8, x, y, b;
+  __device__ __forceinline__ Chunk(unsigned i, unsigned H, unsigned W, unsigned C8) {
+    c8 = i % C8;
+    const unsigned p = i / C8, r = p / W;
+    x = p - r * W;
+    b = r / H;
+    y = r - b * H;
+  }
+};
+__device__ __forceinline__ size_t at(unsigned b, unsigned y, unsigned x, unsigned c8, unsigned H, unsigned W,
+                                     unsigned C8) {
+  return ((((size_t)b * H + y) * W + x) * C8 + c8) * 8;
+}
+// Sum of the 2 x 2 block at (2 y, 2 x), in the order of the scalar kernels.
+__device__ __forceinline__ void block_sum(const bf16* X, const Chunk& c, unsigned H2, unsigned W2, unsigned C8,
+                                          float (&v)[8]) {
+  const bf16* s = X + at(c.b, 2 * c.y, 2 * c.x, c.c8, H2, W2, C8);
+  float f0[8], f1[8], f2[8], f3[8];
+  widen(ldb(s), f0);
+  widen(ldb(s + C8 * 8), f1);
+  widen(ldb(s + (size_t)W2 * C8 * 8), f2);
+  widen(ldb(s + ((size_t)W2 + 1) * C8 * 8), f3);
+#pragma unroll
+  for (int k = 0; k < 8; ++k) v[k] = f0[k] + f1[k] + f2[k] + f3[k];
+}
+
+__global__ void __launch_bounds__(kT) avgpool8_kernel(const bf16* __restrict__ X, bf16* __restrict__ Y, unsigned Ho,
+                                                      unsigned Wo, unsigned C8, unsigned total) {
+  pdl_enter();
+  const unsigned i = blockIdx.x * kT + threadIdx.x;
+  if (i >= total) return;
+  const Chunk c(i, Ho, Wo, C8);
+  float v[8];
+  block_sum(X, c, 2 * Ho, 2 * Wo, C8, v);
+#pragma unroll
+  for (int k = 0; k < 8; ++k) v[k] *= 0.25f;
+  stb(Y + (size_t)i * 8, narrow(v));
+}
+
+__global__ void __launch_bounds__(kT) upsample_add8_kernel(const bf16* __restrict__ X, const bf16* __restrict__ S,
+                                                           bf16* __restrict__ Y, unsigned H, unsigned W, unsigned C8,
+                                                           unsigned total) {
+  pdl_enter();
+  const unsigned i = blockIdx.x * kT + threadIdx.x;
+  if (i >= total) return;
+  const Chunk c(i, H, W, C8);
+  float a[8], v[8];
+  widen(ldb(X + at(c.b, c.y / 2, c.x / 2, c.c8, H / 2, W / 2, C8)), a);
+  widen(ldb(S + (size_t)i * 8), v);
+#pragma unroll
+  for (int k = 0; k < 8; ++k) v[k] = a[k] + v[k];
+  stb(Y + (size_t)i * 8, narrow(v));
+}
+
+// launch_grad_act (cmg_internal.h).  A thread's chunks share their channel
+// group (the stride is a multiple of C8), so the column sums are eight
+// running FP32 sums per thread, then the CTA's in a fixed order.  One pass
+// instead of four or five (the gradient of the resampling, the skip's sum, the ReLU mask,
+// the bias gradient, whose column sums took one CTA per channel: 242 us at
+// 256^2 x 32).
+template <int MODE>
+__global__ void __launch_bounds__(kT) grad_act_kernel(const bf16* __restrict__ y, const bf16* __restrict__ dA,
+                                                      const bf16* __restrict__ dB, const float* __restrict__ w,
+                                                      bf16* __restrict__ dZ, unsigned H, unsigned W, unsigned C8,
+                                                      unsigned total, float* __restrict__ rows, int width) {
+  pdl_enter();
+  __shared__ float sh[kT][9];
+  float sum[8] = {}, hsum[8] = {}, dsum = 0.f, wc[8];
+  const unsigned c8 = threadIdx.x % C8;
+  if (MODE == kGradHead) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) wc[k] = w[c8 * 8 + k];
+  }
+  for (unsigned i = blockIdx.x * kT + threadIdx.x; i < total; i += gridDim.x * kT) {
+    float v[8], yv[8];
+    widen(ldb(y + (size_t)i * 8), yv);
+    if (MODE == kGradDirect) {
+      widen(ldb(dA + (size_t)i * 8), v);
+    } else if (MODE == kGradHead) {
+      const float d = __bfloat162float(dA[i / C8]);
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        v[k] = d * wc[k];
+        hsum[k] = fmaf(d, yv[k], hsum[k]);
+      }
+      if (c8 == 0) dsum += d;
+    } else {
+      const Chunk c(i, H, W, C8);
+      if (MODE == kGradUpsample) {
+        block_sum(dA, c, 2 * H, 2 * W, C8, v);
+      } else {
+        float a[8];
+        widen(ldb(dA + at(c.b, c.y / 2, c.x / 2, c.c8, H / 2, W / 2, C8)), a);
+        widen(ldb(dB + (size_t)i * 8), v);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = __bfloat162float(__float2bfloat16_rn(0.25f * a[k])) + v[k];
+      }
+    }
+    B8 o = narrow(v);
+    widen(o, v);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = yv[k] > 0.f ? v[k] : 0.f;
+    stb(dZ + (size_t)i * 8, narrow(v));
+#pragma unroll
+    for (int k = 0; k < 8; ++k) sum[k] += v[k];
+  }
+  // CTA sums: thread t < 8 C8 adds channel t over the threads of its group
+  const auto reduce = [&](const float (&a)[8], int col) {
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 8; ++k) sh[threadIdx.x][k] = a[k];
+    __syncthreads();
+    if (threadIdx.x < 8 * C8) {
+      const unsigned g = threadIdx.x / 8, k = threadIdx.x % 8;
+      float t = 0.f;
+      for (unsigned r = g; r < kT; r += C8) t += sh[r][k];
+      rows[(size_t)blockIdx.x * width + col + threadIdx.x] = t;
+    }
+  };
+  reduce(sum, 0);
+  if (MODE == kGradHead) {
+    reduce(hsum, 8 * C8);
+    const float one[8] = {dsum};
+    __syncthreads();
+    sh[threadIdx.x][8] = one[0];
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      float t = 0.f;
+      for (unsigned r = 0; r < kT; r += C8) t += sh[r][8];
+      rows[(size_t)blockIdx.x * width + 16 * C8] = t;
+    }
+  }
+}
+
+// launch_finish_layer.  CTAs 0 .. : 32 entries of gw each, eight threads per
+// entry over the slices; the last CTA: the columns of rows, a warp per column.
+__global__ void __launch_bounds__(kT) finish_layer_kernel(const float* __restrict__ part, int slices,
+                                                          float* __restrict__ gw, int n, int gblocks,
+                                                          const float* __restrict__ rows, int nrows, int width,
+                                                          float* __restrict__ gb, int C, float* __restrict__ hw,
+                                                          float* __restrict__ hb) {
+  pdl_enter();
+  const int lane = threadIdx.x & 31, wy = threadIdx.x >> 5;
+  if ((int)blockIdx.x < gblocks) {
+    __shared__ float sh[8][33];
+    const int e = blockIdx.x * 32 + lane;
+    float t = 0.f;
+    if (e < n) {
+#pragma unroll 4
+      for (int z = wy; z < slices; z += 8) t += part[(size_t)z * n + e];
+    }
+    sh[wy][lane] = t;
+    __syncthreads();
+    if (wy == 0 && e < n) {
+      for (int k = 1; k < 8; ++k) t += sh[k][lane];
+      gw[e] = t;
+    }
+    return;
+  }
+  const int col = ((int)blockIdx.x - gblocks) * 8 + wy;
+  if (col >= width) return;
+  float t = 0.f;
+  for (int r = lane; r < nrows; r += 32) t += rows[(size_t)r * width + col];
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  if (lane == 0) {
+    if (col < C) gb[col] = t;
+    else if (col < 2 * C) hw[col - C] = t;
+    else hb[col - 2 * C] = t;
+  }
+}
+
+// Network input with eight channels: one 16-byte store per pixel.
+__global__ void __launch_bounds__(kT) pack_input8_kernel(const double* __restrict__ f0, const double* __restrict__ f1,
+                                                         unsigned n, unsigned S, float s0, float s1,
+                                                         bf16* __restrict__ X, unsigned total) {
+  const unsigned i = blockIdx.x * kT + threadIdx.x;
+  if (i >= total) return;
+  const Chunk c(i, S, S, 1);
+  float v[8] = {};
+  if (c.x < n && c.y < n) {
+    const size_t node = ((size_t)c.b * n + c.y) * n + c.x;
+    v[0] = s0 * (float)f0[node];
+    v[1] = s1 * (float)f1[node];
+  }
+  stb(X + (size_t)i * 8, narrow(v));
+}
+
 // Network input [B][S][S][Cp] from two n x n FP64 fields per image (channel 0
 // and 1, scaled), zero elsewhere (channels >= 2 and pixels beyond n).
 __global__ void pack_input_kernel(const double* __restrict__ f0, const double* __restrict__ f1, int B, int n, int S,
@@ -293,7 +507,52 @@ inline cmg_status done(int launches) {
   return e == cudaSuccess ? CMG_OK : CMG_ERR_CUDA;
 }
 inline cudaStream_t st(void* s) { return static_cast<cudaStream_t>(s); }
+// 16-byte chunks of 8 channels, 32-bit chunk indices (also past the last CTA)
+inline bool chunked(long long n, int C, const void* a, const void* b, const void* c) {
+  return C % 8 == 0 && n / 8 < (1LL << 31) &&
+         ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b) | reinterpret_cast<uintptr_t>(c)) & 15) == 0;
+}
+inline cmg_status launched(cudaError_t e) {
+  count_launches(1);
+  if (e == cudaSuccess) e = cudaGetLastError();
+  return e == cudaSuccess ? CMG_OK : CMG_ERR_CUDA;
+}
+inline dim3 ctas(long long n) { return dim3((unsigned)((n + kT - 1) / kT)); }
 }  // namespace
+
+namespace cmg {
+
+cudaError_t launch_grad_act(int mode, const void* y, const void* dA, const void* dB, const float* w, void* dZ, int B,
+                            int H, int W, int C, float* rows, int* nrows, cudaStream_t s) {
+  const long total = (long)B * H * W * (C / 8);
+  if ((C != 32 && C != 64) || total >= (1L << 31)) return cudaErrorNotSupported;
+  const long want = (total + kT - 1) / kT;
+  const unsigned grid = (unsigned)(want < kGradRows ? want : kGradRows);
+  *nrows = (int)grid;
+  const int width = mode == kGradHead ? 2 * C + 1 : C;
+  const auto go = [&](auto* k) {
+    return launch_k(k, dim3(grid), dim3(kT), 0, s, (const bf16*)y, (const bf16*)dA, (const bf16*)dB, w, (bf16*)dZ,
+                    (unsigned)H, (unsigned)W, (unsigned)(C / 8), (unsigned)total, rows, width);
+  };
+  count_launches(1);
+  switch (mode) {
+    case kGradDirect: return go(grad_act_kernel<kGradDirect>);
+    case kGradUpsample: return go(grad_act_kernel<kGradUpsample>);
+    case kGradPoolSkip: return go(grad_act_kernel<kGradPoolSkip>);
+    case kGradHead: return go(grad_act_kernel<kGradHead>);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+cudaError_t launch_finish_layer(const float* part, int slices, float* gw, int n, const float* rows, int nrows, int width,
+                                float* gb, int C, float* hw, float* hb, cudaStream_t s) {
+  const int gblocks = (n + 31) / 32, cblocks = (width + 7) / 8;
+  count_launches(1);
+  return launch_k(finish_layer_kernel, dim3((unsigned)(gblocks + cblocks)), dim3(kT), 0, s, part, slices, gw, n, gblocks,
+                  rows, nrows, width, gb, C, hw, hb);
+}
+
+}  // namespace cmg
 
 extern "C" {
 
@@ -334,6 +593,10 @@ cmg_status cmg_nn_avgpool(const void* X, void* Y, int B, int H, int W, int C, in
   if (!X || !Y || B < 1 || H < 2 || W < 2 || (H | W) & 1 || C < 1) return CMG_ERR_INVALID_ARG;
   if (backward)   // X = dY [B][H/2][W/2][C], Y = dX [B][H][W][C]
     avgpool_bwd_kernel<<<blocks((long)B * H * W * C), kT, 0, st(stream)>>>((const bf16*)X, (bf16*)Y, B, H, W, C);
+  else if (chunked((long long)B * H * W * C / 4, C, X, Y, Y))
+    return launched(launch_k(avgpool8_kernel, ctas((long long)B * H * W * C / 32), dim3(kT), 0, st(stream),
+                             (const bf16*)X, (bf16*)Y, (unsigned)(H / 2), (unsigned)(W / 2), (unsigned)(C / 8),
+                             (unsigned)((long long)B * H * W * C / 32)));
   else
     avgpool_kernel<<<blocks((long)B * H * W * C / 4), kT, 0, st(stream)>>>((const bf16*)X, (bf16*)Y, B, H, W, C);
   return done(1);
@@ -341,6 +604,10 @@ cmg_status cmg_nn_avgpool(const void* X, void* Y, int B, int H, int W, int C, in
 
 cmg_status cmg_nn_upsample_add(const void* X, const void* S, void* Y, int B, int H, int W, int C, void* stream) {
   if (!X || !S || !Y || B < 1 || H < 2 || W < 2 || (H | W) & 1 || C < 1) return CMG_ERR_INVALID_ARG;
+  if (chunked((long long)B * H * W * C, C, X, S, Y))
+    return launched(launch_k(upsample_add8_kernel, ctas((long long)B * H * W * C / 8), dim3(kT), 0, st(stream),
+                             (const bf16*)X, (const bf16*)S, (bf16*)Y, (unsigned)H, (unsigned)W, (unsigned)(C / 8),
+                             (unsigned)((long long)B * H * W * C / 8)));
   upsample_add_kernel<<<blocks((long)B * H * W * C), kT, 0, st(stream)>>>((const bf16*)X, (const bf16*)S, (bf16*)Y, B,
                                                                           H, W, C);
   return done(1);
@@ -404,6 +671,12 @@ cmg_status cmg_nn_adamw(float* w, const float* g, float* m1, float* m2, void* w1
 cmg_status cmg_nn_pack_input(const double* f0, const double* f1, int B, int n, int S, int Cp, float s0, float s1,
                              void* X, void* stream) {
   if (!f0 || !f1 || !X || B < 1 || n < 1 || S < n || Cp < 2) return CMG_ERR_INVALID_ARG;
+  if (chunked((long long)B * S * S * Cp, Cp, X, X, X) && Cp == 8) {
+    const long long total = (long long)B * S * S;
+    pack_input8_kernel<<<ctas(total), kT, 0, st(stream)>>>(f0, f1, (unsigned)n, (unsigned)S, s0, s1, (bf16*)X,
+                                                           (unsigned)total);
+    return done(1);
+  }
   pack_input_kernel<<<blocks((long)B * S * S * Cp), kT, 0, st(stream)>>>(f0, f1, B, n, S, Cp, s0, s1, (bf16*)X);
   return done(1);
 }

@@ -11,9 +11,9 @@
 // S/4, S/8 with 32, 64, 64, 64 channels; two 3x3 convolutions + ReLU per
 // encoder level, 2x2 average pooling, nearest upsampling with additive
 // skips, one 3x3 convolution + ReLU per decoder level, a 1x1 linear head.
-// A 3x3 convolution is im2col + GEMM (weights [Cout][9 Cin], column
-// t*Cin + c for tap t = 3 dy + dx); its weight gradient a split-K GEMM over
-// the pixels, its data gradient a GEMM and a col2im gather.
+// The 3x3 convolutions (weights [Cout][9 Cin], column t*Cin + c for tap
+// t = 3 dy + dx), their data and their weight gradients are cmg_nn_conv.cu's
+// tensor-core kernels.
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
@@ -86,11 +86,21 @@ struct HostNormal {
   }
 };
 
-// loss = (sum of the CTA partials) / count, one thread, fixed order.
-__global__ void loss_sum_kernel(const float* __restrict__ part, int n, double inv_count, double* __restrict__ out) {
+// loss = (sum of the CTA partials) / count, one CTA, fixed order (one thread
+// took 160 us for the 4864 partials of a 256^2 batch).
+__global__ void __launch_bounds__(1024) loss_sum_kernel(const float* __restrict__ part, int n, double inv_count,
+                                                        double* __restrict__ out) {
+  __shared__ double sh[32];
   double s = 0.0;
-  for (int i = 0; i < n; ++i) s += (double)part[i];
-  *out = s * inv_count;
+  for (int i = threadIdx.x; i < n; i += 1024) s += (double)part[i];
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    s = sh[threadIdx.x];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (threadIdx.x == 0) *out = s * inv_count;
+  }
 }
 
 }  // namespace
@@ -106,14 +116,13 @@ struct cmg_unet {
   const void* x0 = nullptr;         // input of the last forward pass (caller's)
   void* act[kActs] = {};
   void* grad[kActs] = {};
-  void* pool_tmp = nullptr;         // 2x2 pooling gradient before the skip sum
   float* pred = nullptr;            // [Bmax][S][S] last prediction (internal)
   void* dpred = nullptr;            // [Bmax][S][S] BF16 loss gradient
   float* mse_part = nullptr;
   int mse_cap = 0;
   // per-layer work buffers sized for the largest layer
-  void *col = nullptr, *dZ = nullptr, *dZT = nullptr, *colT = nullptr, *WT = nullptr;
-  float *part = nullptr, *dcol = nullptr;
+  void* dZ = nullptr;               // gradient before a layer's ReLU
+  float *part = nullptr, *rows = nullptr;   // weight-gradient slices, column sums (launch_finish_layer)
   std::vector<void*> allocs;
   std::string err;
 };
@@ -153,54 +162,34 @@ long pixels(const cmg_unet* u, int B, int level) {
   return (long)B * H * H;
 }
 
-// Pixel slice of the split-K weight gradient: the largest multiple of 8 up
-// to 4096 that divides the pixel count P (P = B H^2 with H a multiple of 4,
-// so 8 always divides it).
-int kslice(long P) {
-  for (long k = P < 4096 ? P : 4096; k >= 8; k -= 8)
-    if (P % k == 0 && k % 8 == 0) return (int)k;
-  return 8;
-}
-
 cmg_status conv_forward(cmg_unet* u, int layer, const void* X, void* Y, int B) {
   const ConvSpec& c = kConvs[layer];
   const int H = u->S >> c.level;
-  const long P = pixels(u, B, c.level);
   const Param& p = u->prm[layer];
   const cudaError_t e = launch_conv3x3_patch(X, B, H, H, c.ci, p.w16, c.co, p.b, 1, 0, Y, u->status, u->stream, 1);
-  if (e != cudaErrorNotSupported) return e == cudaSuccess ? CMG_OK : cuda_fail(u, e, "convolution");
-  NN(cmg_nn_im2col(X, u->col, B, H, H, c.ci, 0, u->stream));
-  NN(cmg_nn_gemm_bf16(u->col, 9 * c.ci, p.w16, 9 * c.ci, (int)P, c.co, 9 * c.ci, p.b, 1, nullptr, Y, c.co, u->status,
-                      u->stream));
-  return CMG_OK;
+  return e == cudaSuccess ? CMG_OK : cuda_fail(u, e, "convolution");
 }
 
-// dY: gradient of the layer's output after its ReLU; fills gw, gb and, when
-// dX is given, the gradient of the input X.
-cmg_status conv_backward(cmg_unet* u, int layer, const void* X, const void* Y, const void* dY, void* dX, int B) {
+// dA (and dB, by mode: GradMode) lead to the gradient of the layer's output Y
+// after its ReLU; fills gw, gb and, when dX is given, the gradient of the
+// input X.  With the head's gradient, its own gw and gb too.
+cmg_status conv_backward(cmg_unet* u, int layer, const void* X, const void* Y, int mode, const void* dA, const void* dB,
+                         void* dX, int B) {
   const ConvSpec& c = kConvs[layer];
   const int H = u->S >> c.level;
-  const long P = pixels(u, B, c.level);
-  Param& p = u->prm[layer];
-  NN(cmg_nn_relu_bwd(Y, dY, u->dZ, P * c.co, u->stream));
-  NN(cmg_nn_colsum(u->dZ, P, c.co, p.gb, u->stream));
-  NN(cmg_nn_transpose(u->dZ, u->dZT, P, c.co, u->stream));
-  NN(cmg_nn_im2col(X, u->colT, B, H, H, c.ci, 1, u->stream));
-  const int ks = kslice(P);
-  const int nsl = (int)(P / ks);
-  NN(cmg_nn_gemm_bf16_splitk(u->dZT, P, u->colT, P, c.co, 9 * c.ci, ks, nsl, u->part, 9 * c.ci, u->status,
-                             u->stream));
-  NN(cmg_nn_sum_slices(u->part, nsl, p.gw, (long long)c.co * 9 * c.ci, u->stream));
-  if (!dX) return CMG_OK;
+  Param &p = u->prm[layer], &h = u->prm[HEAD];
+  const bool head = mode == kGradHead;
+  int nrows = 0, slices = 0;
+  cudaError_t e = launch_grad_act(mode, Y, dA, dB, h.w, u->dZ, B, H, H, c.co, u->rows, &nrows, u->stream);
+  if (e == cudaSuccess)
+    e = launch_conv3x3_wgrad(X, u->dZ, B, H, H, c.ci, c.co, u->part, &slices, u->status, u->stream);
+  if (e == cudaSuccess)
+    e = launch_finish_layer(u->part, slices, p.gw, c.co * 9 * c.ci, u->rows, nrows, head ? 2 * c.co + 1 : c.co, p.gb,
+                            c.co, head ? h.gw : nullptr, head ? h.gb : nullptr, u->stream);
   // dX as a 3x3 convolution of dZ with the turned weights
-  const cudaError_t e = launch_conv3x3_patch(u->dZ, B, H, H, c.co, p.w16, c.ci, nullptr, 0, 1, dX, u->status,
-                                             u->stream, 1);
-  if (e != cudaErrorNotSupported) return e == cudaSuccess ? CMG_OK : cuda_fail(u, e, "data-gradient convolution");
-  NN(cmg_nn_transpose(p.w16, u->WT, c.co, 9 * c.ci, u->stream));
-  NN(cmg_nn_gemm_bf16(u->dZ, c.co, u->WT, c.co, (int)P, 9 * c.ci, c.co, nullptr, 0, u->dcol, nullptr, 9 * c.ci,
-                      u->status, u->stream));
-  NN(cmg_nn_col2im(u->dcol, dX, B, H, H, c.ci, u->stream));
-  return CMG_OK;
+  if (e == cudaSuccess && dX)
+    e = launch_conv3x3_patch(u->dZ, B, H, H, c.co, p.w16, c.ci, nullptr, 0, 1, dX, u->status, u->stream, 1);
+  return e == cudaSuccess ? CMG_OK : cuda_fail(u, e, "gradient of a convolution");
 }
 
 cmg_status check_batch(cmg_unet* u, int B) {
@@ -269,42 +258,29 @@ cmg_status cmg_unet_create(int S, int max_batch, unsigned long long seed, void* 
     for (float* q : {p.gb, p.mb, p.vb})
       if (e == cudaSuccess) e = cudaMemset(q, 0, nb * sizeof(float));
   }
-  // activations, their gradients and the work buffers (largest layer)
-  size_t col = 0, dz = 0, colT = 0, part = 0, wt = 0, dcol = 0;
+  // activations, the gradients that a data-gradient convolution writes, and
+  // the work buffers (largest layer)
+  size_t dz = 0, part = 0;
   for (int l = 0; l < kConvCount; ++l) {
     const ConvSpec& c = kConvs[l];
-    const long P = pixels(u, B, c.level);
-    col = std::max(col, (size_t)P * 9 * c.ci * 2);
-    dz = std::max(dz, (size_t)P * c.co * 2);
-    colT = std::max(colT, (size_t)P * 9 * c.ci * 2);
-    part = std::max(part, (size_t)(P / kslice(P)) * c.co * 9 * c.ci * 4);
-    wt = std::max(wt, (size_t)9 * c.ci * c.co * 2);
-    dcol = std::max(dcol, (size_t)P * 9 * c.ci * 4);
+    const int H = S >> c.level;
+    dz = std::max(dz, (size_t)pixels(u, B, c.level) * c.co * 2);
+    part = std::max(part, (size_t)wgrad_max_slices(B, H, H) * c.co * 9 * c.ci * 4);
   }
   const long P0 = pixels(u, B, 0);
-  dz = std::max(dz, (size_t)P0 * kHeadC * 2);                         // head: e0 transposed
-  part = std::max(part, (size_t)(P0 / kslice(P0)) * kHeadC * 4);
-  size_t pool = 0;
-  for (int a = 0; a < kActs && e == cudaSuccess; ++a) {
-    const size_t bytes = (size_t)pixels(u, B, kActShape[a].level) * kActShape[a].ch * 2;
-    pool = std::max(pool, bytes);
-    e = ualloc(u, &u->act[a], bytes);
-    if (e == cudaSuccess) e = ualloc(u, &u->grad[a], bytes);
-  }
+  for (int a = 0; a < kActs && e == cudaSuccess; ++a)
+    e = ualloc(u, &u->act[a], (size_t)pixels(u, B, kActShape[a].level) * kActShape[a].ch * 2);
+  for (int a : {A0, P1, A1, P2, A2, P3, A3, T2, T1, T0})
+    if (e == cudaSuccess) e = ualloc(u, &u->grad[a], (size_t)pixels(u, B, kActShape[a].level) * kActShape[a].ch * 2);
   u->mse_cap = 152 * 32;
-  if (e == cudaSuccess) e = ualloc(u, &u->pool_tmp, pool);
   if (e == cudaSuccess) e = ualloc(u, &u->pred, (size_t)P0 * 4);
   if (e == cudaSuccess) e = ualloc(u, &u->dpred, (size_t)P0 * 2);
   if (e == cudaSuccess) e = ualloc(u, &u->mse_part, (size_t)u->mse_cap * 4);
   if (e == cudaSuccess) e = ualloc(u, &u->status, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(u->status, 0, sizeof(int));
-  if (e == cudaSuccess) e = ualloc(u, &u->col, col);
   if (e == cudaSuccess) e = ualloc(u, &u->dZ, dz);
-  if (e == cudaSuccess) e = ualloc(u, &u->dZT, dz);
-  if (e == cudaSuccess) e = ualloc(u, &u->colT, colT);
   if (e == cudaSuccess) e = ualloc(u, &u->part, part);
-  if (e == cudaSuccess) e = ualloc(u, &u->WT, wt);
-  if (e == cudaSuccess) e = ualloc(u, &u->dcol, dcol);
+  if (e == cudaSuccess) e = ualloc(u, &u->rows, (size_t)kGradRows * (2 * 64 + 1) * 4);
   if (e != cudaSuccess) {
     const cmg_status st = e == cudaErrorMemoryAllocation ? CMG_ERR_OOM : CMG_ERR_CUDA;
     (void)cudaGetLastError();
@@ -403,13 +379,8 @@ cmg_status cmg_unet_forward(cmg_unet* u, const void* X, int B, float* pred) {
   if ((st = conv_forward(u, D0, a[T0], a[E0], B)) != CMG_OK) return st;
   const Param& h = u->prm[HEAD];
   const long P0 = pixels(u, B, 0);
-  NN(cmg_nn_gemm_bf16(a[E0], kHeadC, h.w16, kHeadC, (int)P0, 1, kHeadC, h.b, 0, u->pred, nullptr, 1, u->status,
-                      u->stream));
-  if (pred && pred != u->pred) {
-    const cudaError_t e = cudaMemcpyAsync(pred, u->pred, (size_t)P0 * sizeof(float), cudaMemcpyDeviceToDevice,
-                                          u->stream);
-    if (e != cudaSuccess) return cuda_fail(u, e, "copy of the prediction");
-  }
+  const cudaError_t e = launch_head(a[E0], h.w16, h.b, P0, u->pred, pred != u->pred ? pred : nullptr, u->status, u->stream);
+  if (e != cudaSuccess) return cuda_fail(u, e, "head");
   return CMG_OK;
 }
 
@@ -419,7 +390,7 @@ cmg_status cmg_unet_loss(cmg_unet* u, const float* target, int m, double* loss) 
   if (m < 1 || m > u->S) return fail(u, CMG_ERR_INVALID_ARG, "m outside [1, S]");
   int used = 0;
   NN(cmg_nn_mse(u->pred, target, u->Bcur, u->S, m, u->dpred, u->mse_part, u->mse_cap, &used, u->stream));
-  loss_sum_kernel<<<1, 1, 0, u->stream>>>(u->mse_part, used, 1.0 / ((double)u->Bcur * m * m), loss);
+  loss_sum_kernel<<<1, 1024, 0, u->stream>>>(u->mse_part, used, 1.0 / ((double)u->Bcur * m * m), loss);
   count_launches(1);
   const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? CMG_OK : cuda_fail(u, e, "loss_sum_kernel");
@@ -428,42 +399,23 @@ cmg_status cmg_unet_loss(cmg_unet* u, const float* target, int m, double* loss) 
 cmg_status cmg_unet_backward(cmg_unet* u, const void* dpred) {
   if (!u) return CMG_ERR_INVALID_ARG;
   if (u->Bcur < 1 || !u->x0) return fail(u, CMG_ERR_INVALID_ARG, "no forward pass yet");
-  const int B = u->Bcur, S = u->S;
+  const int B = u->Bcur;
   void** a = u->act;
   void** g = u->grad;
   const void* dp = dpred ? dpred : u->dpred;
-  const long P0 = pixels(u, B, 0);
-  Param& h = u->prm[HEAD];
-  // head: e0 [P0][32] times w [1][32]^T + b
-  NN(cmg_nn_transpose(a[E0], u->dZT, P0, kHeadC, u->stream));
-  const int ks = kslice(P0);
-  const int nsl = (int)(P0 / ks);
-  NN(cmg_nn_gemm_bf16_splitk(dp, P0, u->dZT, P0, 1, kHeadC, ks, nsl, u->part, kHeadC, u->status, u->stream));
-  NN(cmg_nn_sum_slices(u->part, nsl, h.gw, kHeadC, u->stream));
-  NN(cmg_nn_colsum(dp, P0, 1, h.gb, u->stream));
-  NN(cmg_nn_outer(dp, h.w, g[E0], P0, kHeadC, u->stream));
   cmg_status st;
-  if ((st = conv_backward(u, D0, a[T0], a[E0], g[E0], g[T0], B)) != CMG_OK) return st;
-  NN(cmg_nn_upsample_bwd(g[T0], g[E1], B, S / 2, S / 2, 32, u->stream));
-  if ((st = conv_backward(u, D1, a[T1], a[E1], g[E1], g[T1], B)) != CMG_OK) return st;
-  NN(cmg_nn_upsample_bwd(g[T1], g[E2], B, S / 4, S / 4, 64, u->stream));
-  if ((st = conv_backward(u, D2, a[T2], a[E2], g[E2], g[T2], B)) != CMG_OK) return st;
-  NN(cmg_nn_upsample_bwd(g[T2], g[B3], B, S / 8, S / 8, 64, u->stream));
-  if ((st = conv_backward(u, C3B, a[A3], a[B3], g[B3], g[A3], B)) != CMG_OK) return st;
-  if ((st = conv_backward(u, C3A, a[P3], a[A3], g[A3], g[P3], B)) != CMG_OK) return st;
-  // s2 feeds the pooling and the skip into t2
-  NN(cmg_nn_avgpool(g[P3], u->pool_tmp, B, S / 4, S / 4, 64, 1, u->stream));
-  NN(cmg_nn_add(u->pool_tmp, g[T2], g[S2], pixels(u, B, 2) * 64, u->stream));
-  if ((st = conv_backward(u, C2B, a[A2], a[S2], g[S2], g[A2], B)) != CMG_OK) return st;
-  if ((st = conv_backward(u, C2A, a[P2], a[A2], g[A2], g[P2], B)) != CMG_OK) return st;
-  NN(cmg_nn_avgpool(g[P2], u->pool_tmp, B, S / 2, S / 2, 64, 1, u->stream));
-  NN(cmg_nn_add(u->pool_tmp, g[T1], g[S1], pixels(u, B, 1) * 64, u->stream));
-  if ((st = conv_backward(u, C1B, a[A1], a[S1], g[S1], g[A1], B)) != CMG_OK) return st;
-  if ((st = conv_backward(u, C1A, a[P1], a[A1], g[A1], g[P1], B)) != CMG_OK) return st;
-  NN(cmg_nn_avgpool(g[P1], u->pool_tmp, B, S, S, 32, 1, u->stream));
-  NN(cmg_nn_add(u->pool_tmp, g[T0], g[S0], pixels(u, B, 0) * 32, u->stream));
-  if ((st = conv_backward(u, C0B, a[A0], a[S0], g[S0], g[A0], B)) != CMG_OK) return st;
-  return conv_backward(u, C0A, u->x0, a[A0], g[A0], nullptr, B);
+  if ((st = conv_backward(u, D0, a[T0], a[E0], kGradHead, dp, nullptr, g[T0], B)) != CMG_OK) return st;
+  if ((st = conv_backward(u, D1, a[T1], a[E1], kGradUpsample, g[T0], nullptr, g[T1], B)) != CMG_OK) return st;
+  if ((st = conv_backward(u, D2, a[T2], a[E2], kGradUpsample, g[T1], nullptr, g[T2], B)) != CMG_OK) return st;
+  if ((st = conv_backward(u, C3B, a[A3], a[B3], kGradUpsample, g[T2], nullptr, g[A3], B)) != CMG_OK) return st;
+  if ((st = conv_backward(u, C3A, a[P3], a[A3], kGradDirect, g[A3], nullptr, g[P3], B)) != CMG_OK) return st;
+  // s2, s1, s0 each feed the pooling and a skip
+  if ((st = conv_backward(u, C2B, a[A2], a[S2], kGradPoolSkip, g[P3], g[T2], g[A2], B)) != CMG_OK) return st;
+  if ((st = conv_backward(u, C2A, a[P2], a[A2], kGradDirect, g[A2], nullptr, g[P2], B)) != CMG_OK) return st;
+  if ((st = conv_backward(u, C1B, a[A1], a[S1], kGradPoolSkip, g[P2], g[T1], g[A1], B)) != CMG_OK) return st;
+  if ((st = conv_backward(u, C1A, a[P1], a[A1], kGradDirect, g[A1], nullptr, g[P1], B)) != CMG_OK) return st;
+  if ((st = conv_backward(u, C0B, a[A0], a[S0], kGradPoolSkip, g[P1], g[T0], g[A0], B)) != CMG_OK) return st;
+  return conv_backward(u, C0A, u->x0, a[A0], kGradDirect, g[A0], nullptr, nullptr, B);
 }
 
 cmg_status cmg_unet_step(cmg_unet* u, float lr, float b1, float b2, float eps, float wd) {
