@@ -235,32 +235,56 @@ __global__ void __launch_bounds__(kCoarseThreads) coarse_solve_b(int m, int N, i
 // FP64.  The per-sample products run in the cycle's precision C: FP64 for
 // FP64 cycles, FP32 for FP32 cycles (GB300's FP64 pipe made them ~6 us of
 // the FP32 cycle's single-CTA critical path).
-constexpr int kCoarseCtaThreads = 512;
+//
+// One CTA's latency chain is what it costs (it runs once per cycle, 2^l times in
+// a W-cycle): the inverses are staged while the preceding kernel still runs
+// (they change only with the samples), the sums over the samples are a warp
+// per control row (a thread per row summed N values one after another in FP64:
+// half of the 20.6 us at N = 100), one thread per product up to 1024.
+constexpr int kCoarseCtaThreads = 1024;
 
 template <typename C>
 size_t coarse_cta_smem(int N, int m) {
-  return 2 * 64 * sizeof(double) + ((size_t)N * m * m + 4 * (size_t)N * m) * sizeof(C);
+  return (2 * 64 + (size_t)m * m) * sizeof(double) + 16 + ((size_t)N * m * m + 4 * (size_t)N * m) * sizeof(C);
 }
 
+// Shared memory of the single-CTA solve.
+template <typename C>
+struct CoarseSmem {
+  double *rhs, *us, *M;   // [m] control right side, [m] control, [m][m] its inverse
+  C *A, *by, *bp, *w, *z; // [N][m][m]; [N][m] f_y, later y; f_p, later w - c A^{-1} z; A^{-1} f_y; A^{-1} f_p
+  __device__ __forceinline__ CoarseSmem(double* sm, int m, int N) {
+    const int nm = N * m;
+    rhs = sm;
+    us = rhs + 64;
+    M = us + 64;
+    A = reinterpret_cast<C*>(M + ((m * m + 1) & ~1));   // 16-byte aligned
+    by = A + (size_t)nm * m;
+    bp = by + nm;
+    w = bp + nm;
+    z = w + nm;
+  }
+  // The inverses, 16 bytes per load (both start 16-byte aligned).
+  __device__ __forceinline__ void stage(int m, int N, const C* __restrict__ Ainv, const double* __restrict__ Minv) const {
+    const int cnt = N * m * m, nv = cnt / (16 / (int)sizeof(C));
+    for (int i = threadIdx.x; i < nv; i += blockDim.x)
+      reinterpret_cast<uint4*>(A)[i] = reinterpret_cast<const uint4*>(Ainv)[i];
+    for (int i = nv * (16 / (int)sizeof(C)) + threadIdx.x; i < cnt; i += blockDim.x) A[i] = Ainv[i];
+    for (int i = threadIdx.x; i < m * m; i += blockDim.x) M[i] = Minv[i];
+  }
+};
+
 // The coarsest solve by one CTA (the body shared by the single-instance
-// kernel and the batched one, which runs one CTA per instance).
+// kernel and the batched one, which runs one CTA per instance), after stage().
 template <typename T, typename C>
-__device__ __forceinline__ void coarse_cta_body(int m, int N, const C* __restrict__ Ainv,
-                                                const double* __restrict__ Minv, double c, double d, double e,
+__device__ __forceinline__ void coarse_cta_body(const CoarseSmem<C>& S, int m, int N, double c, double d, double e,
                                                 Vec3c<T> f, Vec3<T> x, int freeze_u, int nside, CtlBox ctl,
                                                 const float* __restrict__ dw) {
-  extern __shared__ __align__(16) double sm[];
   const int mm = m * m, nm = N * m;
-  double* rhs = sm;                  // [m] control right side
-  double* us = rhs + 64;             // [m] control
-  C* A = reinterpret_cast<C*>(us + 64);   // [N][m][m]
-  C* by = A + (size_t)N * mm;        // [N][m] f_y, later y
-  C* bp = by + nm;                   // [N][m] f_p, later w - c A^{-1} z
-  C* w = bp + nm;                    // [N][m] A^{-1} f_y
-  C* z = w + nm;                     // [N][m] A^{-1} f_p
+  const C *A = S.A;
+  C *by = S.by, *bp = S.bp, *w = S.w, *z = S.z;
   const C cc = (C)c, ec = (C)e;
-  const int tid = threadIdx.x, nt = blockDim.x;
-  for (int i = tid; i < N * mm; i += nt) A[i] = Ainv[i];
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warps = nt >> 5;
   for (int i = tid; i < nm; i += nt) {   // f.y, f.p are [node r][sample j]
     const int r = i / N, j = i - r * N;
     by[j * m + r] = (C)f.y[i];
@@ -287,26 +311,32 @@ __device__ __forceinline__ void coarse_cta_body(int m, int N, const C* __restric
     bp[i] = w[i] - cc * v;
   }
   __syncthreads();
-  for (int r = tid; r < m; r += nt) {
+  for (int r = tid >> 5; r < m; r += warps) {
     double q = 0.0;
-    for (int j = 0; j < N; ++j) q += (double)bp[j * m + r];
+    for (int j = lane; j < N; j += 32) q += (double)bp[j * m + r];
+    for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
     const double dr = dw ? d * (double)dw[r] : d;   // d_r (active-set factor)
-    rhs[r] = ctl.inside(r / nside, r % nside) ? (double)f.u[r] - dr * q : 0.0;   // control rows only at control nodes
+    if (lane == 0)
+      S.rhs[r] = ctl.inside(r / nside, r % nside) ? (double)f.u[r] - dr * q : 0.0;   // control rows only at control nodes
   }
   __syncthreads();
-  for (int r = tid; r < m; r += nt) {
+  for (int r = tid >> 5; r < m; r += warps) {
     double u = 0.0;
-    if (!freeze_u)   // frozen control: zero correction of u, state and adjoint solved for it
-      for (int k = 0; k < m; ++k) u += Minv[r * m + k] * rhs[k];
-    us[r] = u;
-    x.u[r] = (T)u;
+    if (!freeze_u) {   // frozen control: zero correction of u, state and adjoint solved for it
+      for (int k = lane; k < m; k += 32) u += S.M[r * m + k] * S.rhs[k];
+      for (int o = 16; o > 0; o >>= 1) u += __shfl_xor_sync(0xffffffffu, u, o);
+    }
+    if (lane == 0) {
+      S.us[r] = u;
+      x.u[r] = (T)u;
+    }
   }
   __syncthreads();
   for (int i = tid; i < nm; i += nt) {   // y = z - e A^{-1} u, into by
     const int j = i / m, r = i - j * m;
     const C* Ar = A + (size_t)j * mm + r * m;
     C t = 0;
-    for (int k = 0; k < m; ++k) t += Ar[k] * (C)us[k];
+    for (int k = 0; k < m; ++k) t += Ar[k] * (C)S.us[k];
     const C yv = z[i] - ec * t;
     by[i] = yv;
     x.y[(size_t)r * N + j] = (T)yv;
@@ -321,14 +351,19 @@ __device__ __forceinline__ void coarse_cta_body(int m, int N, const C* __restric
   }
 }
 
+// Every kernel that lets its successors start early (pdl_enter) leaves the
+// inverses alone, so they are read before the wait for the predecessor.
 template <typename T, typename C>
 __global__ void __launch_bounds__(kCoarseCtaThreads) coarse_solve_cta(int m, int N, const C* __restrict__ Ainv,
                                                                      const double* __restrict__ Minv, double c,
                                                                      double d, double e, Vec3c<T> f, Vec3<T> x,
                                                                      int freeze_u, int nside, CtlBox ctl,
                                                                      const float* __restrict__ dw) {
+  extern __shared__ __align__(16) double sm[];
+  const CoarseSmem<C> S(sm, m, N);
+  S.stage(m, N, Ainv, Minv);
   pdl_enter();
-  coarse_cta_body<T, C>(m, N, Ainv, Minv, c, d, e, f, x, freeze_u, nside, ctl, dw);
+  coarse_cta_body<T, C>(S, m, N, c, d, e, f, x, freeze_u, nside, ctl, dw);
 }
 
 // The coarsest solves of a batch of instances (FP32 cycles), CTA b for
@@ -339,7 +374,10 @@ __global__ void __launch_bounds__(kCoarseCtaThreads) batch_coarse_kernel(const B
                                                                         const int* __restrict__ err) {
   if (*err || !act[blockIdx.x]) return;
   const BatchCoarse& q = bc[blockIdx.x];
-  coarse_cta_body<float, float>(q.m, q.N, q.Ainv32, q.Minv, q.c, q.d, q.e, q.f, q.x, 0, q.nside, q.ctl, q.dw);
+  extern __shared__ __align__(16) double sm[];
+  const CoarseSmem<float> S(sm, q.m, q.N);
+  S.stage(q.m, q.N, q.Ainv32, q.Minv);
+  coarse_cta_body<float, float>(S, q.m, q.N, q.c, q.d, q.e, q.f, q.x, 0, q.nside, q.ctl, q.dw);
 }
 
 // FP32 copy of the A_j^{-1} for the FP32 coarse solve.
@@ -363,7 +401,7 @@ cudaError_t coarse_solve_mm(const CoarseData& C, double c, double d, double e, V
       if (ea != cudaSuccess) return ea;
       attr = true;
     }
-    const cudaError_t ek = launch_k(coarse_solve_cta<T, Cm>, dim3(1), dim3(kCoarseCtaThreads),
+    const cudaError_t ek = launch_k(coarse_solve_cta<T, Cm>, dim3(1), dim3(C.N * C.m > 512 ? 1024 : 512),
                                     coarse_cta_smem<Cm>(C.N, C.m), s, C.m, C.N, ainv, (const double*)C.Minv, c, d, e,
                                     f, x, freeze_u, C.n, C.ctl, C.dw);
     count_launches(1);
@@ -401,7 +439,7 @@ cudaError_t launch_batch_coarse(const BatchCoarse* bc, int count, int N_max, int
     if (ea != cudaSuccess) return ea;
     attr = true;
   }
-  batch_coarse_kernel<<<count, kCoarseCtaThreads, smem, s>>>(bc, act, err);
+  batch_coarse_kernel<<<count, N_max * m > 512 ? 1024 : 512, smem, s>>>(bc, act, err);
   count_launches(1);
   return cudaGetLastError();
 }
