@@ -77,12 +77,8 @@ __device__ __forceinline__ vec<T, V> inv_diag(const LevelView<T>& L, size_t off,
 
 // ---------------------------------------------------------------------------
 // r = f - S x (or r = S x when f.y == nullptr) at one node; y block times wy.
-// DIFF: (A v)_i formed as sum_f k_f (v_i - v_f) (v_f = 0 outside the grid)
-// instead of a_i v_i - sum_f k_f v_f: for a smooth v the differences are
-// small and nearly exact, so the rounding error scales with the differences
-// rather than with |v|.
 // ---------------------------------------------------------------------------
-template <typename T, int V, int SPL, bool CG, bool DIFF = false>
+template <typename T, int V, int SPL, bool CG>
 __device__ __forceinline__ void residual_item(const LevelView<T>& L, const Vec3c<T>& x, const Vec3c<T>& f,
                                               const Vec3<T>& r, long node, int lane, int lpn, T wy) {
   const int n = L.n, N = L.N;
@@ -116,33 +112,16 @@ __device__ __forceinline__ void residual_item(const LevelView<T>& L, const Vec3c
         const vec<T, V> pS = ldx_if<T, V, CG>(hS, x.p + o - (size_t)n * ld + j);
         const vec<T, V> pN = ldx_if<T, V, CG>(hN, x.p + o + (size_t)n * ld + j);
         vec<T, V> ry, rp;
-        if constexpr (DIFF) {
+        vec<T, V> offy = vzero<T, V>(), offp = vzero<T, V>();
+        fma_faces<T, V>(offy, kW, yW, kE, yE, kS, yS, kN, yN);
+        fma_faces<T, V>(offp, kW, pW, kE, pE, kS, pS, kN, pN);
 #pragma unroll
-          for (int k = 0; k < V; ++k) {
-            T ay = kW.v[k] * (y.v[k] - yW.v[k]);
-            ay = fma(kE.v[k], y.v[k] - yE.v[k], ay);
-            ay = fma(kS.v[k], y.v[k] - yS.v[k], ay);
-            ay = fma(kN.v[k], y.v[k] - yN.v[k], ay);
-            T ap = kW.v[k] * (p.v[k] - pW.v[k]);
-            ap = fma(kE.v[k], p.v[k] - pE.v[k], ap);
-            ap = fma(kS.v[k], p.v[k] - pS.v[k], ap);
-            ap = fma(kN.v[k], p.v[k] - pN.v[k], ap);
-            ry.v[k] = c * y.v[k] + ap;
-            rp.v[k] = ay + e * uu;
-            pacc += p.v[k];
-          }
-        } else {
-          vec<T, V> offy = vzero<T, V>(), offp = vzero<T, V>();
-          fma_faces<T, V>(offy, kW, yW, kE, yE, kS, yS, kN, yN);
-          fma_faces<T, V>(offp, kW, pW, kE, pE, kS, pS, kN, pN);
-#pragma unroll
-          for (int k = 0; k < V; ++k) {
-            const T a = (kW.v[k] + kE.v[k]) + (kS.v[k] + kN.v[k]);
-            // state rows: c y + A p ; adjoint rows: A y + e u
-            ry.v[k] = c * y.v[k] + (a * p.v[k] - offp.v[k]);
-            rp.v[k] = (a * y.v[k] - offy.v[k]) + e * uu;
-            pacc += p.v[k];
-          }
+        for (int k = 0; k < V; ++k) {
+          const T a = (kW.v[k] + kE.v[k]) + (kS.v[k] + kN.v[k]);
+          // state rows: c y + A p ; adjoint rows: A y + e u
+          ry.v[k] = c * y.v[k] + (a * p.v[k] - offp.v[k]);
+          rp.v[k] = (a * y.v[k] - offy.v[k]) + e * uu;
+          pacc += p.v[k];
         }
         if (!apply) {
           const vec<T, V> fy = ldx<T, V, CG>(f.y + o + j), fp = ldx<T, V, CG>(f.p + o + j);
@@ -172,31 +151,44 @@ __device__ __forceinline__ void residual_item(const LevelView<T>& L, const Vec3c
   }
 }
 
-// x + (P e) at fine node (fy, fx), samples j .. j+V-1: the value the
-// prolongation kernel would leave there (same operations in the same
-// order), formed where a half-sweep reads it as a neighbour.
+// The neighbours of colour-0 node (iy, ix) read as x + P e (coarse correction
+// e on the nc x nc grid), added to acc as sum_f k_f (x + P e)_f.  A colour-1
+// node has one odd and one even coordinate, so its (P e) is half the sum of
+// the two coarse nodes beside it along the even one; around an even-even
+// node these are the four coarse corners, around an odd-odd node the
+// coinciding coarse node and its four neighbours, each loaded once (a colour's
+// nodes of a grid row are all of one kind).  The same operations in the same
+// order as the prolongation kernel followed by the plain half-sweep.
 template <typename T, int V, bool CG>
-__device__ __forceinline__ vec<T, V> prolonged(const T* xv, const T* ev, int nf, int nc, size_t ld, int fy, int fx,
-                                               int j) {
-  vec<T, V> v = ldx<T, V, CG>(xv + ((size_t)fy * nf + fx) * ld + j);
-  int Jr[2] = {0, 0}, Ir[2] = {0, 0};
-  T wy[2] = {T(0), T(0)}, wx[2] = {T(0), T(0)};
-  int ny, nx;
-  if (fy & 1) { Jr[0] = (fy - 1) >> 1; wy[0] = T(1); ny = 1; }
-  else { Jr[0] = (fy >> 1) - 1; Jr[1] = fy >> 1; wy[0] = wy[1] = T(0.5); ny = 2; }
-  if (fx & 1) { Ir[0] = (fx - 1) >> 1; wx[0] = T(1); nx = 1; }
-  else { Ir[0] = (fx >> 1) - 1; Ir[1] = fx >> 1; wx[0] = wx[1] = T(0.5); nx = 2; }
-  for (int a = 0; a < ny; ++a) {
-    if (Jr[a] < 0 || Jr[a] >= nc) continue;
-    for (int b = 0; b < nx; ++b) {
-      if (Ir[b] < 0 || Ir[b] >= nc) continue;
-      const T wt = wy[a] * wx[b];
-      const vec<T, V> ec = ldx<T, V, CG>(ev + ((size_t)Jr[a] * nc + Ir[b]) * ld + j);
+__device__ __forceinline__ void fma_faces_prolonged(vec<T, V>& acc, const vec<T, V>& kW, const vec<T, V>& kE,
+                                                    const vec<T, V>& kS, const vec<T, V>& kN, const T* xv, const T* ev,
+                                                    int n, int nc, size_t ld, int iy, int ix, int j) {
+  const bool hW = ix > 0, hE = ix < n - 1, hS = iy > 0, hN = iy < n - 1;
+  const T* xo = xv + ((size_t)iy * n + ix) * ld + j;
+  vec<T, V> xW = ldx_if<T, V, CG>(hW, xo - ld), xE = ldx_if<T, V, CG>(hE, xo + ld);
+  vec<T, V> xS = ldx_if<T, V, CG>(hS, xo - (size_t)n * ld), xN = ldx_if<T, V, CG>(hN, xo + (size_t)n * ld);
+  const auto half = [](vec<T, V>& v, const vec<T, V>& a, const vec<T, V>& b) {
 #pragma unroll
-      for (int k = 0; k < V; ++k) v.v[k] = fma(wt, ec.v[k], v.v[k]);
-    }
+    for (int k = 0; k < V; ++k) v.v[k] = fma(T(0.5), b.v[k], fma(T(0.5), a.v[k], v.v[k]));
+  };
+  const int J = iy >> 1, I = ix >> 1;
+  const size_t row = (size_t)nc * ld;
+  const T* eo = ev + ((size_t)J * nc + I) * ld + j;   // coarse node (J, I)
+  if (iy & 1) {
+    const vec<T, V> c = ldx<T, V, CG>(eo);
+    half(xW, ldx_if<T, V, CG>(I > 0, eo - ld), c);
+    half(xE, c, ldx_if<T, V, CG>(I + 1 < nc, eo + ld));
+    half(xS, ldx_if<T, V, CG>(J > 0, eo - row), c);
+    half(xN, c, ldx_if<T, V, CG>(J + 1 < nc, eo + row));
+  } else {
+    const vec<T, V> sw = ldx_if<T, V, CG>(J > 0 && I > 0, eo - row - ld), se = ldx_if<T, V, CG>(J > 0 && I < nc, eo - row);
+    const vec<T, V> nw = ldx_if<T, V, CG>(J < nc && I > 0, eo - ld), ne = ldx_if<T, V, CG>(J < nc && I < nc, eo);
+    if (hW) half(xW, sw, nw);
+    if (hE) half(xE, se, ne);
+    if (hS) half(xS, sw, se);
+    if (hN) half(xN, nw, ne);
   }
-  return v;
+  fma_faces<T, V>(acc, kW, xW, kE, xE, kS, xS, kN, xN);
 }
 
 // ---------------------------------------------------------------------------
@@ -252,13 +244,8 @@ __device__ __forceinline__ void rbgs_node(const LevelView<T>& L, const Vec3c<T>&
         bp[s] = ldx<T, V, CG>(f.y + o + j);   // first block row: c y + A p = f_y
         by[s] = ldx<T, V, CG>(f.p + o + j);   // last block row:  A y + e u = f_p
         if constexpr (PRO) {
-          const auto nb = [&](bool h, const T* xv, const T* ev, int fy, int fx) {
-            return h ? prolonged<T, V, CG>(xv, ev, n, nc, ld, fy, fx, j) : vzero<T, V>();
-          };
-          fma_faces<T, V>(bp[s], kW, nb(hW, xs.p, e.p, iy, ix - 1), kE, nb(hE, xs.p, e.p, iy, ix + 1), kS,
-                          nb(hS, xs.p, e.p, iy - 1, ix), kN, nb(hN, xs.p, e.p, iy + 1, ix));
-          fma_faces<T, V>(by[s], kW, nb(hW, xs.y, e.y, iy, ix - 1), kE, nb(hE, xs.y, e.y, iy, ix + 1), kS,
-                          nb(hS, xs.y, e.y, iy - 1, ix), kN, nb(hN, xs.y, e.y, iy + 1, ix));
+          fma_faces_prolonged<T, V, CG>(bp[s], kW, kE, kS, kN, xs.p, e.p, n, nc, ld, iy, ix, j);
+          fma_faces_prolonged<T, V, CG>(by[s], kW, kE, kS, kN, xs.y, e.y, n, nc, ld, iy, ix, j);
         } else if constexpr (!ZG) {
           fma_faces<T, V>(bp[s], kW, ldx_if<T, V, CG>(hW, xs.p + o - ld + j), kE,
                           ldx_if<T, V, CG>(hE, xs.p + o + ld + j), kS,
@@ -617,42 +604,80 @@ __device__ __forceinline__ float residual_cast_item(const LevelView<double>& L, 
 
 // One node of the FP32 refinement between anchors (residual replacement):
 // the scaled residual r (the cycle's right side) is updated in place,
-// r <- r - S e (A e from neighbour differences, see residual_item), the
-// running correction d += e, and this lane's part of ||W r||^2 is returned
-// (squares in FP32; wy2 weights the state block).  Each lane reads its own r
-// entries before writing them, so the update in place is safe.
+// r <- r - S e, (A e)_i formed as sum_f k_f (e_i - e_f) (e_f = 0 outside the
+// grid) instead of a_i e_i - sum_f k_f e_f: for a smooth e the differences are
+// small and nearly exact, so the rounding error scales with them rather than
+// with |e|; the running correction d += e, and this lane's
+// part of ||W r||^2 is returned (squares in FP32; wy2 weights the state
+// block).  One pass: a lane loads its own r, d and e once and writes r and d
+// at the same place, so the update in place is safe.  (Running residual_item
+// and then re-reading r and e took 2.18 ms at n = 1023, N = 256.)
 template <int V, int SPL>
 __device__ __forceinline__ float recur_item(const LevelView<float>& L, const Vec3c<float>& e, const Vec3<float>& r,
                                             const Vec3<float>& d, long node, int lane, int lpn, float wy2) {
-  residual_item<float, V, SPL, false, true>(L, e, cview(r), r, node, lane, lpn, 1.0f);
-  const int N = L.N;
+  using T = float;
+  const int n = L.n, N = L.N;
   const size_t ld = (size_t)L.ld;
-  float sq = 0.f;
-  if (node < (long)L.n * L.n) {
+  const bool valid = node < (long)n * n;
+  const T c = (T)L.c, eb = (T)L.e;
+  T pacc = 0.f, sq = 0.f;
+  const int iy = valid ? (int)(node / n) : 0, ix = valid ? (int)(node - (long)iy * n) : 0;
+  const bool ctl = L.ctl.inside(iy, ix);   // local control: chi_i
+  T eu = 0.f;
+  if (valid) {
+    eu = e.u[node];
     const size_t o = (size_t)node * ld;
+    const T* kWp = L.kx + ((size_t)iy * (n + 1) + ix) * ld;
+    const T* kSp = L.ky + ((size_t)iy * n + ix) * ld;
+    const bool hW = ix > 0, hE = ix < n - 1, hS = iy > 0, hN = iy < n - 1;
+    const T uu = ctl ? eu : 0.f;
 #pragma unroll
     for (int s = 0; s < SPL; ++s) {
       const int j = (lane + s * lpn) * V;
       if (j < N) {
-        const vec<float, V> ry = ldv<float, V>(r.y + o + j), rp = ldv<float, V>(r.p + o + j);
-        const vec<float, V> ey = ldv<float, V>(e.y + o + j), ep = ldv<float, V>(e.p + o + j);
-        vec<float, V> dy = ldv<float, V>(d.y + o + j), dp = ldv<float, V>(d.p + o + j);
+        const vec<T, V> kW = ldv<T, V>(kWp + j), kE = ldv<T, V>(kWp + ld + j);
+        const vec<T, V> kS = ldv<T, V>(kSp + j), kN = ldv<T, V>(kSp + (size_t)n * ld + j);
+        const vec<T, V> y = ldv<T, V>(e.y + o + j), p = ldv<T, V>(e.p + o + j);
+        const vec<T, V> yW = ldv_if<T, V>(hW, e.y + o - ld + j), yE = ldv_if<T, V>(hE, e.y + o + ld + j);
+        const vec<T, V> yS = ldv_if<T, V>(hS, e.y + o - (size_t)n * ld + j);
+        const vec<T, V> yN = ldv_if<T, V>(hN, e.y + o + (size_t)n * ld + j);
+        const vec<T, V> pW = ldv_if<T, V>(hW, e.p + o - ld + j), pE = ldv_if<T, V>(hE, e.p + o + ld + j);
+        const vec<T, V> pS = ldv_if<T, V>(hS, e.p + o - (size_t)n * ld + j);
+        const vec<T, V> pN = ldv_if<T, V>(hN, e.p + o + (size_t)n * ld + j);
+        vec<T, V> ry = ldv<T, V>(r.y + o + j), rp = ldv<T, V>(r.p + o + j);
+        vec<T, V> dy = ldv<T, V>(d.y + o + j), dp = ldv<T, V>(d.p + o + j);
 #pragma unroll
         for (int k = 0; k < V; ++k) {
+          T ay = kW.v[k] * (y.v[k] - yW.v[k]);
+          ay = fma(kE.v[k], y.v[k] - yE.v[k], ay);
+          ay = fma(kS.v[k], y.v[k] - yS.v[k], ay);
+          ay = fma(kN.v[k], y.v[k] - yN.v[k], ay);
+          T ap = kW.v[k] * (p.v[k] - pW.v[k]);
+          ap = fma(kE.v[k], p.v[k] - pE.v[k], ap);
+          ap = fma(kS.v[k], p.v[k] - pS.v[k], ap);
+          ap = fma(kN.v[k], p.v[k] - pN.v[k], ap);
+          ry.v[k] = ry.v[k] - (c * y.v[k] + ap);
+          rp.v[k] = rp.v[k] - (ay + eb * uu);
+          pacc += p.v[k];
           sq = fmaf(wy2 * ry.v[k], ry.v[k], sq);
           sq = fmaf(rp.v[k], rp.v[k], sq);
-          dy.v[k] += ey.v[k];
-          dp.v[k] += ep.v[k];
+          dy.v[k] += y.v[k];
+          dp.v[k] += p.v[k];
         }
-        stv<float, V>(d.y + o + j, dy);
-        stv<float, V>(d.p + o + j, dp);
+        stv<T, V>(r.y + o + j, ry);
+        stv<T, V>(r.p + o + j, rp);
+        stv<T, V>(d.y + o + j, dy);
+        stv<T, V>(d.p + o + j, dp);
       }
     }
-    if (lane == 0) {
-      const float ru = r.u[node];
-      sq = fmaf(ru, ru, sq);
-      d.u[node] += e.u[node];
-    }
+  }
+  const T psum = group_sum(pacc, lpn);
+  if (valid && lane == 0) {
+    // control row: G u + d_i sum_j p_j
+    const T ru = ctl ? r.u[node] - ((T)L.G * eu + (T)d_of(L, node) * psum) : 0.f;
+    r.u[node] = ru;
+    sq = fmaf(ru, ru, sq);
+    d.u[node] += eu;
   }
   return sq;
 }
