@@ -83,13 +83,16 @@ struct SampleMap {
   int V;
   int spl;
 };
-// Lanes per node for a launch over `items` nodes.  A lane takes up to 4
+// Lanes per node for a launch over `items` nodes.  A lane takes several
 // chunks so that one warp covers several nodes and the per-node FP64 work
 // (control-row sum, u) is shared by one warp instruction, as long as the
-// launch keeps at least kMinLanes lanes (two 256-thread CTAs per SM);
-// small grids are latency-bound and use more lanes per node.  items = 0
-// asks for the most lanes (one chunk per lane where N allows).
-constexpr long kMinLanes = 2L * 152 * 256;
+// launch keeps enough lanes: kMinLanes2 at two chunks of 16 bytes, kMinLanes4
+// at four, kMinLanes1 at four single samples; small grids are latency-bound
+// and use more lanes per node.  items = 0 asks for the most lanes (one chunk
+// per lane where N allows).
+constexpr long kMinLanes2 = 20000;
+constexpr long kMinLanes4 = 400000;
+constexpr long kMinLanes1 = 40000;
 SampleMap choose_map(int N, int elem_bytes, long items, int spl_target = 0);
 
 // Coarsest-grid factors (FP64).

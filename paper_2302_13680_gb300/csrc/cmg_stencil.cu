@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(kBlock) residual_cast_kernel(LevelView<double>
 
 // FP32 refinement between FP64 anchors (residual replacement): the scaled
 // residual r (the cycle's right side) is updated in place, r <- r - S e (A e
-// from neighbour differences, see residual_item), the
+// from neighbour differences, see recur_item), the
 // running correction d += e, and per-CTA partial sums of ||W r||^2 are
 // written (squares in FP32, CTA sum in FP64).  Each lane reads its own f
 // entries before writing r at the same place, so the update in place is safe.
@@ -239,8 +239,20 @@ SampleMap choose_map(int N, int elem_bytes, long items, int spl_target) {
   const int vmax = 16 / elem_bytes;     // 2 for double, 4 for float
   m.V = (N % vmax == 0) ? vmax : 1;
   const int chunks = (N + m.V - 1) / m.V;
-  int target = 4;
-  while (target > 1 && items * chunks / target < kMinLanes) target >>= 1;
+  // Chunks per lane by what the launch has to offer (kMinLanes*): 16 samples
+  // per lane only where that still leaves a dozen waves of CTAs, 8 from a few CTAs per
+  // SM on; and at least two (four) lanes per node, else a warp's loads fall
+  // apart into single sectors.  FP64 takes two chunks at most: with four, the
+  // registers leave the FP64 pipe too few warps (n = 255, N = 64: 96 against 81
+  // us per half-sweep).  FP32 half-sweeps, 4 -> 2 chunks: n = 255, N = 64 20.8 -> 18.9 us,
+  // n = 511, N = 16 50.9 -> 25.9 us; 1 -> 2: n = 127, N = 64 7.2 -> 5.5 us.
+  int target = 1;
+  if (items > 0) {
+    const long lanes = items * chunks;
+    if (lanes >= 2 * kMinLanes2 && chunks >= 4) target = 2;
+    if (m.V == 1 ? lanes >= 4 * kMinLanes1 && chunks >= 16 : elem_bytes == 4 && lanes >= 4 * kMinLanes4 && chunks >= 16)
+      target = 4;
+  }
   if ((spl_target & 15) > 0) target = spl_target & 15;   // the staged and wide flags are not part of it
   const int want = (chunks + target - 1) / target;   // lanes needed at `target` chunks each
   int lpn = 1;
