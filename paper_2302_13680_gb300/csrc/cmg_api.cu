@@ -83,6 +83,7 @@ struct cmg_handle {
   bool g32_ready = false;      // Galerkin handles: the FP32 copies of the coarse planes are current
   CoarseData& c32() { return prob.coarse_coeff == CMG_COARSE_NODAL ? coarse : coarse32; }
   bool galerkin() const { return prob.coarse_coeff == CMG_COARSE_GALERKIN; }
+  int ld32 = 0;                // sample stride of the FP32 arrays (padded_samples; N unless averaged coarse grids)
   double* xi = nullptr;       // [N][K] device
   double* kap = nullptr;      // setup scratch
   double* red = nullptr;      // reduction partials
@@ -162,22 +163,26 @@ struct ProfScope {
 };
 
 // ctl32: the FP32 cycle's all-FP32 option (cmg_cycle.ctl32); FP64 views ignore it.
+// raw: for a caller's vectors, whose rows have N samples; else the view of the
+// handle's own, padded ones.
 template <typename T>
-LevelView<T> view(const cmg_handle* h, int l, int freeze_u = 0, int ctl32 = 0);
+LevelView<T> view(const cmg_handle* h, int l, int freeze_u = 0, int ctl32 = 0, bool raw = false);
 template <>
-LevelView<double> view<double>(const cmg_handle* h, int l, int freeze_u, int) {
+LevelView<double> view<double>(const cmg_handle* h, int l, int freeze_u, int, bool) {
   const Lev& v = h->lv[l];
   return {v.n, h->prob.N, h->prob.N, v.kx64, v.ky64, v.inva, v.isigma, v.c, v.G * h->gscale, v.d, v.e,
-          v.spl_target[0], freeze_u, nullptr, v.a64, v.ctl, h->dw_on ? v.dw : nullptr, 0};
+          v.spl_target[0], freeze_u, nullptr, v.a64, v.ctl, h->dw_on ? v.dw : nullptr, h->prob.N, h->prob.N, h->ld32, 0};
 }
 template <>
-LevelView<float> view<float>(const cmg_handle* h, int l, int freeze_u, int ctl32) {
+LevelView<float> view<float>(const cmg_handle* h, int l, int freeze_u, int ctl32, bool raw) {
   const Lev& v = h->lv[l];
+  const int N = raw ? h->prob.N : h->ld32;
   // nodal coarse grids round the FP64 operator's 1/sigma; averaged ones have
   // their own FP32 operator with its FP64 1/sigma
   const double* isd = h->prob.coarse_coeff == CMG_COARSE_NODAL ? v.isigma : v.isigd32;
-  return {v.n, h->prob.N, h->prob.N, v.kx32, v.ky32, v.inva, isd, v.c, v.G * h->gscale, v.d, v.e,
-          v.spl_target[1], freeze_u, v.isigma32, nullptr, v.ctl, h->dw_on ? v.dw : nullptr, ctl32 ? 1 : 0};
+  return {v.n, N, N, v.kx32, v.ky32, v.inva, isd, v.c, v.G * h->gscale, v.d, v.e,
+          v.spl_target[1], freeze_u, v.isigma32, nullptr, v.ctl, h->dw_on ? v.dw : nullptr, h->ld32, h->prob.N, h->ld32,
+          ctl32 ? 1 : 0};
 }
 
 // The coarsest-grid data for a cycle of precision T; its per-node factor on d
@@ -223,22 +228,24 @@ cudaError_t setup_coefficients(cmg_handle* h) {
   h->g32_ready = false;
   Lev& v0 = h->lv[0];
   cudaError_t e = launch_field_faces(v0.n, P.N, P.K, P.amp, h->xi, h->kap, v0.kx64, v0.ky64, v0.kx32, v0.ky32,
-                                     h->stream);
+                                     h->ld32, h->stream);
   if (e == cudaSuccess) e = launch_diag_sum(v0.n, P.N, v0.kx64, v0.ky64, v0.a64, h->stream);
   for (int l = 0; l < h->L && e == cudaSuccess; ++l) {
     Lev& v = h->lv[l];
     if (l > 0) {
       const Lev& f = h->lv[l - 1];
-      e = launch_coarse_faces32(f.n, P.N, f.kx32, f.ky32, v.kx32, v.ky32, h->stream);
+      e = launch_coarse_faces32(f.n, h->ld32, f.kx32, f.ky32, v.kx32, v.ky32, h->stream);   // the padding's faces too
     }
     if (e == cudaSuccess)
-      e = launch_diag32(v.n, P.N, v.kx32, v.ky32, v.isigma32, v.isigd32, v.d * v.c * v.e, v.G * h->gscale, h->stream, v.dw);
+      e = launch_diag32(v.n, P.N, v.kx32, v.ky32, h->ld32, v.isigma32, v.isigd32, v.d * v.c * v.e, v.G * h->gscale,
+                        h->stream, v.dw);
   }
   if (e != cudaSuccess) return e;
   const Lev& cl = h->lv[h->L - 1];
-  const size_t cf = (size_t)cl.n * (cl.n + 1) * P.N;
-  e = launch_scale_cast<float, double>(1.0, cl.kx32, h->cface64, cf, h->stream);
-  if (e == cudaSuccess) e = launch_scale_cast<float, double>(1.0, cl.ky32, h->cface64 + cf, cf, h->stream);
+  const size_t cfaces = (size_t)cl.n * (cl.n + 1), cf = cfaces * P.N;
+  e = launch_cast_rows<float, double>(1.0, cl.kx32, h->ld32, h->cface64, P.N, cfaces, P.N, h->stream);
+  if (e == cudaSuccess)
+    e = launch_cast_rows<float, double>(1.0, cl.ky32, h->ld32, h->cface64 + cf, P.N, cfaces, P.N, h->stream);
   if (e != cudaSuccess) return e;
   return launch_coarse_setup(h->coarse32, h->cface64, h->cface64 + cf, cl.c, cl.G * h->gscale, cl.d, cl.e,
                              h->stream);
@@ -325,7 +332,7 @@ cudaError_t refresh_dw(cmg_handle* h) {
       e = launch_diag64(v.n, P.N, v.kx64, v.ky64, v.inva, v.isigma, v.d * v.c * v.e, G, h->stream, v.dw);
     if (e != cudaSuccess) break;
     e = nodal ? launch_scale_cast<double, float>(1.0, v.isigma, v.isigma32, v.nodes, h->stream)
-              : launch_diag32(v.n, P.N, v.kx32, v.ky32, v.isigma32, v.isigd32, v.d * v.c * v.e, G, h->stream, v.dw);
+              : launch_diag32(v.n, P.N, v.kx32, v.ky32, h->ld32, v.isigma32, v.isigd32, v.d * v.c * v.e, G, h->stream, v.dw);
   }
   if (e != cudaSuccess) return e;
   const Lev& cl = h->lv[h->L - 1];
@@ -344,7 +351,7 @@ cudaError_t refresh_dw(cmg_handle* h) {
 // r = f - S_l x (r = S_l x when f.y == nullptr): the 9-point Galerkin
 // operator on the coarse grids of a Galerkin hierarchy, else the 5-point one.
 template <typename T>
-cudaError_t level_residual(cmg_handle* h, int l, Vec3c<T> x, Vec3c<T> f, Vec3<T> r) {
+cudaError_t level_residual(cmg_handle* h, int l, Vec3c<T> x, Vec3c<T> f, Vec3<T> r, bool raw = false) {
   if (h->galerkin() && l > 0) {
     const Lev& v = h->lv[l];
     const Lev& f0 = h->lv[0];
@@ -353,7 +360,7 @@ cudaError_t level_residual(cmg_handle* h, int l, Vec3c<T> x, Vec3c<T> f, Vec3<T>
     else a9 = v.a9f;
     return launch_residual9<T>(v.n, h->prob.N, a9, v.m9, f0.c, f0.G, f0.d, f0.e, x, f, r, v.psum, h->stream);
   }
-  return launch_residual<T>(view<T>(h, l), x, f, r, h->stream);
+  return launch_residual<T>(view<T>(h, l, 0, 0, raw), x, f, r, h->stream);
 }
 
 // The red-black sweeps on grid l run as one launch each (launch_rbgs_fused),
@@ -363,7 +370,7 @@ bool fused_on(cmg_handle* h, const cmg_cycle& o, int l) {
   const Lev& v = h->lv[l];
   if (o.smoother != CMG_SMOOTH_RBGS || o.freeze_u || !(v.spl_target[1] & kTuneFused) || !v.xs32[0]) return false;
   if (h->galerkin() && l > 0) return false;
-  return fused_plan(v.n, h->prob.N, v.spl_target[1]).ok;
+  return fused_plan(v.n, h->ld32, v.spl_target[1]).ok;
 }
 
 Vec3<float> second_iterate(Lev& v) { return {v.xs32[0], v.xs32[1], v.xs32[2]}; }
@@ -386,7 +393,7 @@ cudaError_t fused_pair(cmg_handle* h, const cmg_cycle& o, int l, Vec3<float> x, 
 }
 
 template <typename T>
-cudaError_t smooth(cmg_handle* h, const cmg_cycle& o, int l, int sweeps, Vec3<T> x, Vec3c<T> f) {
+cudaError_t smooth(cmg_handle* h, const cmg_cycle& o, int l, int sweeps, Vec3<T> x, Vec3c<T> f, bool raw = false) {
   if constexpr (sizeof(T) == 4) {
     if (sweeps >= 2 && fused_on(h, o, l)) {
       for (; sweeps >= 2; sweeps -= 2) {
@@ -435,7 +442,7 @@ cudaError_t smooth(cmg_handle* h, const cmg_cycle& o, int l, int sweeps, Vec3<T>
       return cudaSuccess;
     }
   }
-  const LevelView<T> L = view<T>(h, l, o.freeze_u, o.ctl32);
+  const LevelView<T> L = view<T>(h, l, o.freeze_u, o.ctl32, raw);
   for (int s = 0; s < sweeps; ++s) {
     if (o.smoother == CMG_SMOOTH_RBGS) {
       for (int colour = 0; colour < 2; ++colour) {
@@ -448,7 +455,7 @@ cudaError_t smooth(cmg_handle* h, const cmg_cycle& o, int l, int sweeps, Vec3<T>
       cudaError_t e;
       {
         ProfScope ps(h, CMG_KERNEL_RESIDUAL, l);
-        e = level_residual<T>(h, l, cview(x), f, r);
+        e = level_residual<T>(h, l, cview(x), f, r, raw);
       }
       if (e != cudaSuccess) return e;
       ProfScope ps(h, CMG_KERNEL_SMOOTH, l);
@@ -459,9 +466,14 @@ cudaError_t smooth(cmg_handle* h, const cmg_cycle& o, int l, int sweeps, Vec3<T>
   return cudaSuccess;
 }
 
+// Samples in a row of the handle's own vectors.
+template <typename T>
+int row(const cmg_handle* h) { return sizeof(T) == 4 ? h->ld32 : h->prob.N; }
+
+// x = 0 (FP32: one of the handle's own vectors).
 template <typename T>
 cudaError_t zero_vec(cmg_handle* h, int l, Vec3<T> x) {
-  const size_t nodes = h->lv[l].nodes, N = (size_t)h->prob.N;
+  const size_t nodes = h->lv[l].nodes, N = (size_t)row<T>(h);
   cudaError_t e = cudaMemsetAsync(x.y, 0, nodes * N * sizeof(T), h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(x.u, 0, nodes * sizeof(T), h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(x.p, 0, nodes * N * sizeof(T), h->stream);
@@ -476,7 +488,7 @@ cudaError_t zero_vec(cmg_handle* h, int l, Vec3<T> x) {
 template <typename T>
 cudaError_t tail_cycle(cmg_handle* h, const cmg_cycle& o, int l, Vec3<T> x, Vec3c<T> f) {
   const int nlev = h->L - l;
-  if (nlev > kTailMax || !tail_supported(h->prob.N, sizeof(T), h->coarse.m)) return cudaErrorNotSupported;
+  if (nlev > kTailMax || !tail_supported(row<T>(h), sizeof(T), h->coarse.m)) return cudaErrorNotSupported;
   TailParams<T> P{};
   P.nlev = nlev;
   for (int k = 0; k < nlev; ++k) {
@@ -497,7 +509,8 @@ cudaError_t tail_cycle(cmg_handle* h, const cmg_cycle& o, int l, Vec3<T> x, Vec3
   P.gamma = o.gamma;
   P.theta = o.theta;
   P.freeze_u = o.freeze_u;
-  P.lpn = choose_map(h->prob.N, sizeof(T), 0).lpn;
+  P.lpn = choose_map(row<T>(h), sizeof(T), 0).lpn;
+  P.cld = row<T>(h);
   const CoarseData& cd = sizeof(T) == 4 ? h->c32() : h->coarse;
   P.cm = cd.m;
   P.cN = cd.N;
@@ -530,7 +543,7 @@ bool zero_guess_ok(const cmg_handle* h, const cmg_cycle& o, int l) {
 template <typename T>
 cudaError_t cycle(cmg_handle* h, const cmg_cycle& o, int l, Vec3<T> x, Vec3c<T> f, bool zg = false) {
   Lev& v = h->lv[l];
-  const int N = h->prob.N;
+  const int N = row<T>(h);
   if (o.tail_n > 0 && v.n <= o.tail_n && !h->galerkin()) {
     const cudaError_t e = tail_cycle<T>(h, o, l, x, f);
     if (e != cudaErrorNotSupported) return e;
@@ -541,7 +554,7 @@ cudaError_t cycle(cmg_handle* h, const cmg_cycle& o, int l, Vec3<T> x, Vec3c<T> 
       const Lev& f0 = h->lv[0];
       return launch_galerkin_coarse_solve<T>(h->coarse, v.m9, f0.c, f0.d, f0.e, f, x, h->stream);
     }
-    return launch_coarse_solve<T>(coarse_for<T>(h), v.c, v.d, v.e, f, x, h->stream, o.freeze_u);
+    return launch_coarse_solve<T>(coarse_for<T>(h), v.c, v.d, v.e, f, x, h->stream, o.freeze_u, N);
   }
   cudaError_t e = cudaSuccess;
   bool fz = false;   // one-launch sweeps on this grid
@@ -618,6 +631,32 @@ cudaError_t cycle(cmg_handle* h, const cmg_cycle& o, int l, Vec3<T> x, Vec3c<T> 
   }
   if (e == cudaSuccess) e = smooth<T>(h, o, l, o.n2, x, f);
   return e;
+}
+
+// One cycle on a caller's vectors.  FP32 vectors whose rows are shorter than
+// the handle's padded ones go through the finest grid's own (two copies each
+// way, some 10 % of the cycle; scalar loads on the finest grid cost 40 %).
+template <typename T>
+cudaError_t cycle_on(cmg_handle* h, const cmg_cycle& o, Vec3<T> x, Vec3c<T> f) {
+  if constexpr (sizeof(T) == 4) {
+    const int N = h->prob.N, ld = h->ld32;
+    if (ld != N) {
+      Lev& v = h->lv[0];
+      const Vec3<float> xi = Work<float>::x(v), fi = Work<float>::f(v);
+      const float* src[4] = {f.y, f.p, x.y, x.p};
+      float* dst[4] = {fi.y, fi.p, xi.y, xi.p};
+      for (int k = 0; k < 4; ++k) {
+        const cudaError_t e = launch_cast_rows<float, float>(1.0, src[k], N, dst[k], ld, v.nodes, N, h->stream);
+        if (e != cudaSuccess) return e;
+      }
+      // the control block has no padding: the caller's is used in place
+      cudaError_t e = cycle<float>(h, o, 0, Vec3<float>{xi.y, x.u, xi.p}, Vec3c<float>{fi.y, f.u, fi.p});
+      if (e == cudaSuccess) e = launch_cast_rows<float, float>(1.0, xi.y, ld, x.y, N, v.nodes, N, h->stream);
+      if (e == cudaSuccess) e = launch_cast_rows<float, float>(1.0, xi.p, ld, x.p, N, v.nodes, N, h->stream);
+      return e;
+    }
+  }
+  return cycle<T>(h, o, 0, x, f);
 }
 
 cmg_status check_cycle(cmg_handle* h, const cmg_cycle* o) {
@@ -749,6 +788,9 @@ cmg_status cmg_create(const cmg_problem* prob, const double* xi_host, void* stre
     }
   }
   const size_t N = (size_t)P.N;
+  h->ld32 = P.coarse_coeff == CMG_COARSE_AVERAGED ? padded_samples(P.N) : P.N;
+  const size_t Np = (size_t)h->ld32;
+  const bool padded = h->ld32 != P.N;
   cudaError_t e = cudaSuccess;
 #define AL(ptr, cnt)                        \
   do {                                      \
@@ -757,12 +799,16 @@ cmg_status cmg_create(const cmg_problem* prob, const double* xi_host, void* stre
   for (int l = 0; l < L; ++l) {
     Lev& v = h->lv[l];
     const size_t faces = (size_t)v.n * (v.n + 1) * N;
-    AL(v.kx64, faces); AL(v.ky64, faces); AL(v.kx32, faces); AL(v.ky32, faces);
+    AL(v.kx64, faces); AL(v.ky64, faces); AL(v.kx32, faces / N * Np); AL(v.ky32, faces / N * Np);
     AL(v.inva, v.nodes * N); AL(v.isigma, v.nodes); AL(v.isigma32, v.nodes); AL(v.isigd32, v.nodes);
     for (int b = 0; b < 3; ++b) {
       const size_t cnt = (b == 1) ? v.nodes : v.nodes * N;
-      AL(v.r64[b], cnt); AL(v.x32[b], cnt); AL(v.f32[b], cnt); AL(v.r32[b], cnt); AL(v.f64[b], cnt);
+      const size_t cnt32 = (b == 1) ? v.nodes : v.nodes * Np;
+      AL(v.r64[b], cnt); AL(v.x32[b], cnt32); AL(v.f32[b], cnt32); AL(v.r32[b], cnt32); AL(v.f64[b], cnt);
       AL(v.x64[b], cnt);
+      // padding samples start at zero and have no other source of data
+      for (float* q : {v.x32[b], v.f32[b], v.r32[b]})
+        if (e == cudaSuccess && padded) e = cudaMemsetAsync(q, 0, cnt32 * sizeof(float), h->stream);
       if (P.N % 4 == 0 && l + 1 < L) AL(v.xs32[b], cnt);
     }
   }
@@ -784,7 +830,7 @@ cmg_status cmg_create(const cmg_problem* prob, const double* xi_host, void* stre
   AL(h->ir_state, 16);
   {
     Lev& l0 = h->lv[0];
-    AL(l0.d32[0], l0.nodes * N); AL(l0.d32[1], l0.nodes); AL(l0.d32[2], l0.nodes * N);
+    AL(l0.d32[0], l0.nodes * Np); AL(l0.d32[1], l0.nodes); AL(l0.d32[2], l0.nodes * Np);
   }
   const int cn = h->lv[L - 1].n;
   h->coarse.n = cn;
@@ -878,7 +924,7 @@ cmg_status cmg_rhs(cmg_handle* h, const double* yd, const double* fsrc, double* 
     if (!vec_ok(y, u, p) || !vec_ok(ry, ru, rp)) return fail(h, CMG_ERR_INVALID_ARG, "null pointer");          \
     if ((fy || fu || fp) && !vec_ok(fy, fu, fp)) return fail(h, CMG_ERR_INVALID_ARG, "partial rhs");           \
     CK(ensure_ops<T>(h));                                                                                       \
-    CK(level_residual<T>(h, level, Vec3c<T>{y, u, p}, Vec3c<T>{fy, fu, fp}, Vec3<T>{ry, ru, rp}));             \
+    CK(level_residual<T>(h, level, Vec3c<T>{y, u, p}, Vec3c<T>{fy, fu, fp}, Vec3<T>{ry, ru, rp}, true));       \
     return CMG_OK;                                                                                              \
   }                                                                                                             \
   cmg_status cmg_smooth##SUF(cmg_handle* h, int level, const cmg_cycle* opts, int sweeps, T* y, T* u, T* p,     \
@@ -892,7 +938,7 @@ cmg_status cmg_rhs(cmg_handle* h, const double* yd, const double* fsrc, double* 
     const cmg_status st = check_cycle(h, &o);                                                                   \
     if (st != CMG_OK) return st;                                                                                \
     CK(ensure_ops<T>(h));                                                                                       \
-    CK(smooth<T>(h, o, level, sweeps, Vec3<T>{y, u, p}, Vec3c<T>{fy, fu, fp}));                                \
+    CK(smooth<T>(h, o, level, sweeps, Vec3<T>{y, u, p}, Vec3c<T>{fy, fu, fp}, true));                          \
     return CMG_OK;                                                                                              \
   }                                                                                                             \
   cmg_status cmg_restrict##SUF(cmg_handle* h, int level, const T* ry, const T* ru, const T* rp, T* cy, T* cu,   \
@@ -937,7 +983,7 @@ cmg_status cmg_rhs(cmg_handle* h, const double* yd, const double* fsrc, double* 
       return fail(h, CMG_ERR_INVALID_ARG, "precision does not match the vector type");                         \
     if (!vec_ok(y, u, p) || !vec_ok(fy, fu, fp)) return fail(h, CMG_ERR_INVALID_ARG, "null pointer");          \
     CK(ensure_ops<T>(h));                                                                                       \
-    CK(cycle<T>(h, *opts, 0, Vec3<T>{y, u, p}, Vec3c<T>{fy, fu, fp}));                                          \
+    CK(cycle_on<T>(h, *opts, Vec3<T>{y, u, p}, Vec3c<T>{fy, fu, fp}));                                          \
     return CMG_OK;                                                                                              \
   }
 
@@ -1050,7 +1096,7 @@ cmg_status time_prolong(cmg_handle* h, int l, int t, int reps, bool unfused, flo
     if (r == 0) err = cudaEventRecord(e0, h->stream);
     if (err != cudaSuccess) break;
     if (unfused) {
-      err = launch_prolong_add<float>(v.n, h->prob.N, cview(e), x, h->stream, v.ctl);
+      err = launch_prolong_add<float>(v.n, h->ld32, cview(e), x, h->stream, v.ctl);
       if (err == cudaSuccess) err = launch_rbgs_half<float>(L, x, cview(f), 0, h->stream);
     } else {
       err = launch_rbgs_prolong<float>(L, x, cview(f), cview(e), c.n, h->stream);
@@ -1217,15 +1263,26 @@ cmg_status precondition(cmg_handle* h, const cmg_cycle& o, Vec3c<double> v, Vec3
   // is needed for the FP32 range), result converted into FP64.
   const double vscale = 1.0;
   Vec3<float> f32 = Work<float>::f(l0), x32 = Work<float>::x(l0);
-  CK((launch_scale_cast<double, float>(vscale / wy, v.y, f32.y, ny, h->stream)));
+  const int N = h->prob.N, ld = h->ld32;
   CK((launch_scale_cast<double, float>(vscale, v.u, f32.u, nu, h->stream)));
-  CK((launch_scale_cast<double, float>(vscale, v.p, f32.p, ny, h->stream)));
+  if (ld == N) {
+    CK((launch_scale_cast<double, float>(vscale / wy, v.y, f32.y, ny, h->stream)));
+    CK((launch_scale_cast<double, float>(vscale, v.p, f32.p, ny, h->stream)));
+  } else {
+    CK((launch_cast_rows<double, float>(vscale / wy, v.y, N, f32.y, ld, nu, N, h->stream)));
+    CK((launch_cast_rows<double, float>(vscale, v.p, N, f32.p, ld, nu, N, h->stream)));
+  }
   const bool zg = zero_guess_ok(h, o, 0);
   if (!zg) CK(zero_vec<float>(h, 0, x32));
   CK(cycle<float>(h, o, 0, x32, cview(f32), zg));
-  CK((launch_scale_cast<float, double>(1.0 / vscale, x32.y, z.y, ny, h->stream)));
   CK((launch_scale_cast<float, double>(1.0 / vscale, x32.u, z.u, nu, h->stream)));
-  CK((launch_scale_cast<float, double>(1.0 / vscale, x32.p, z.p, ny, h->stream)));
+  if (ld == N) {
+    CK((launch_scale_cast<float, double>(1.0 / vscale, x32.y, z.y, ny, h->stream)));
+    CK((launch_scale_cast<float, double>(1.0 / vscale, x32.p, z.p, ny, h->stream)));
+  } else {
+    CK((launch_cast_rows<float, double>(1.0 / vscale, x32.y, ld, z.y, N, nu, N, h->stream)));
+    CK((launch_cast_rows<float, double>(1.0 / vscale, x32.p, ld, z.p, N, nu, N, h->stream)));
+  }
   return CMG_OK;
 }
 
@@ -1319,11 +1376,10 @@ void ir_state_init(const cmg_handle* h, double* hs, double rho, double sc, int m
 cmg_status ir_iteration_anchor(cmg_handle* h, Vec3c<double> f, Vec3<double> x, cudaGraphConditionalHandle cond,
                                int graph) {
   Lev& l0 = h->lv[0];
-  const size_t ny = l0.nodes * h->prob.N, nu = l0.nodes;
   Vec3<float> f32 = Work<float>::f(l0);
   Vec3<float> d32{l0.d32[0], l0.d32[1], l0.d32[2]};
   double* st = h->ir_state;
-  CK(launch_fold(st + kInvSc, st + kAnchor, d32, x, ny, nu, h->stream));
+  CK(launch_fold(st + kInvSc, st + kAnchor, d32, x, l0.nodes, h->prob.N, h->ld32, h->stream));
   const int cnt = launch_residual_cast(view<double>(h, 0), cview(x), f, f32, 0.0, st + kSc, paper_wy(h), h->part,
                                        h->part_cap, h->stream, st + kAnchor);
   if (cnt < 0) return fail(h, CMG_ERR_CUDA, "refinement pass launch failed");
@@ -1343,7 +1399,7 @@ cmg_status ir_iteration(cmg_handle* h, const cmg_cycle& o, Vec3c<double> f, Vec3
   double* st = h->ir_state;
   // the correction equation starts from zero
   const bool zg = zero_guess_ok(h, o, 0);
-  if (!zg) CK(launch_zero3(x32, l0.nodes * h->prob.N, l0.nodes, h->stream));
+  if (!zg) CK(launch_zero3(x32, l0.nodes * h->ld32, l0.nodes, h->stream));
   CK(cycle<float>(h, o, 0, x32, cview(f32), zg));
   int cnt = launch_recur(view<float>(h, 0), cview(x32), f32, d32, paper_wy(h), h->part, h->part_cap, h->stream);
   if (cnt < 0) return fail(h, CMG_ERR_CUDA, "recursive residual launch failed");
@@ -2049,7 +2105,7 @@ cmg_status batch_build_tables(cmg_batch* b, const cmg_cycle& o, const double* co
     for (const cmg_handle* h : b->inst)
       if (d < h->L - 1) {
         int lpn, V, spl;
-        batch_map(h->prob.N, 1, kBatchMapCoop, lpn, V, spl);
+        batch_map(h->ld32, 1, kBatchMapCoop, lpn, V, spl);
         work += items((long)h->lv[d].n * h->lv[d].n, 32 / lpn);
       }
     b->leg_phases[d] = b->leg_force >= 0 ? b->leg_force : (work >= kBatchPhaseItems ? 1 : 0);
@@ -2069,7 +2125,7 @@ cmg_status batch_build_tables(cmg_batch* b, const cmg_cycle& o, const double* co
       B.x = Work<float>::x(h->lv[l]);
       B.f = Work<float>::f(h->lv[l]);
       B.r = Work<float>::r(h->lv[l]);
-      batch_map(N, 1, maps[l], B.lpn, B.V, B.spl);
+      batch_map(h->ld32, 1, maps[l], B.lpn, B.V, B.spl);
       V = B.V;
       B.nc = l + 1 < h->L ? h->lv[l + 1].n : 0;
     }
@@ -2088,7 +2144,7 @@ cmg_status batch_build_tables(cmg_batch* b, const cmg_cycle& o, const double* co
     const CoarseData cd = coarse_for<float>(h);
     const Lev& cl = h->lv[h->L - 1];
     co[i] = BatchCoarse{cd.m, N, cd.n, cd.ctl, cd.Ainv32, cd.Minv, cl.c, cl.d, cl.e, cd.dw,
-                        cview(Work<float>::f(h->lv[h->L - 1])), Work<float>::x(h->lv[h->L - 1])};
+                        cview(Work<float>::f(h->lv[h->L - 1])), Work<float>::x(h->lv[h->L - 1]), h->ld32};
     const int npw64 = 32 / lpn64;
     const int cls = V == 4 ? 1 : (V == 2 ? 2 : 3);
     for (int d = 0; d < D; ++d) {
@@ -2376,7 +2432,7 @@ extern "C" cmg_status cmg_batch_solve(cmg_batch* b, const cmg_cycle* opts, doubl
     ir_state_init(h, hs, rho, fnorm[i] > 0.0 ? 1.0 / fnorm[i] : 1.0, maxit, tol * fnorm[i]);
     BCK(cudaMemcpyAsync(h->ir_state, hs, kIrStateSize * sizeof(double), cudaMemcpyHostToDevice, b->stream));
     Lev& l0 = h->lv[0];
-    const size_t ny = l0.nodes * h->prob.N;
+    const size_t ny = l0.nodes * h->ld32;
     BCK(cudaMemsetAsync(l0.d32[0], 0, ny * sizeof(float), b->stream));
     BCK(cudaMemsetAsync(l0.d32[1], 0, l0.nodes * sizeof(float), b->stream));
     BCK(cudaMemsetAsync(l0.d32[2], 0, ny * sizeof(float), b->stream));

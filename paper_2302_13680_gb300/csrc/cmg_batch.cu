@@ -318,12 +318,12 @@ __global__ void __launch_bounds__(kBThreads) batch_fold_kernel(BatchTables T) {
     const long node = (long)w * (32 / I.lpn64) + lane / I.lpn64;
     if (node >= (long)n * n) return;
     const int ln = lane & (I.lpn64 - 1);
-    const size_t o = (size_t)node * N;
+    const size_t o = (size_t)node * N, q = (size_t)node * I.L64.ld32;
     for (int j = ln; j < N; j += I.lpn64) {
-      I.x64.y[o + j] = fma(a, (double)I.d32.y[o + j], I.x64.y[o + j]);
-      I.x64.p[o + j] = fma(a, (double)I.d32.p[o + j], I.x64.p[o + j]);
-      I.d32.y[o + j] = 0.f;
-      I.d32.p[o + j] = 0.f;
+      I.x64.y[o + j] = fma(a, (double)I.d32.y[q + j], I.x64.y[o + j]);
+      I.x64.p[o + j] = fma(a, (double)I.d32.p[q + j], I.x64.p[o + j]);
+      I.d32.y[q + j] = 0.f;
+      I.d32.p[q + j] = 0.f;
     }
     if (ln == 0) {
       I.x64.u[node] = fma(a, (double)I.d32.u[node], I.x64.u[node]);

@@ -168,6 +168,31 @@ cudaError_t launch_axpy(double a, const Tx* x, Ty* y, size_t n, cudaStream_t s) 
   return cudaGetLastError();
 }
 
+namespace {
+template <typename Tx, typename Ty>
+__global__ void cast_rows_kernel(double a, const Tx* __restrict__ src, int lds, Ty* __restrict__ dst, int ldd,
+                                 size_t rows, int N) {
+  const size_t total = rows * (size_t)ldd, stride = (size_t)gridDim.x * blockDim.x;
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
+    const size_t r = i / ldd;
+    const int j = (int)(i - r * ldd);
+    dst[i] = j < N ? (Ty)((decltype(Tx() + Ty()))a * src[r * lds + j]) : Ty(0);
+  }
+}
+}  // namespace
+
+template <typename Tx, typename Ty>
+cudaError_t launch_cast_rows(double a, const Tx* src, int lds, Ty* dst, int ldd, size_t rows, int N, cudaStream_t s) {
+  size_t blocks = (rows * (size_t)ldd + 255) / 256;
+  if (blocks > 152 * 32) blocks = 152 * 32;
+  cast_rows_kernel<<<(unsigned)blocks, 256, 0, s>>>(a, src, lds, dst, ldd, rows, N);
+  count_launches(1);
+  return cudaGetLastError();
+}
+template cudaError_t launch_cast_rows<double, float>(double, const double*, int, float*, int, size_t, int, cudaStream_t);
+template cudaError_t launch_cast_rows<float, double>(double, const float*, int, double*, int, size_t, int, cudaStream_t);
+template cudaError_t launch_cast_rows<float, float>(double, const float*, int, float*, int, size_t, int, cudaStream_t);
+
 template <typename Tx, typename Ty>
 cudaError_t launch_scale_cast(double a, const Tx* x, Ty* y, size_t n, cudaStream_t s) {
   scale_cast_kernel<Tx, Ty><<<stream_blocks(n), kRedThreads, 0, s>>>(a, x, y, n);

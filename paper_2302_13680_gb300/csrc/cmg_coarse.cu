@@ -121,7 +121,7 @@ constexpr int kCoarseThreads = 32;   // one warp per CTA: samples spread over SM
 template <typename T, int MM>
 __global__ void __launch_bounds__(kCoarseThreads) coarse_solve_a(int m, int N, const double* __restrict__ Ainv,
                                                                 double c, const T* __restrict__ fy,
-                                                                const T* __restrict__ fp, double* __restrict__ wz,
+                                                                const T* __restrict__ fp, int ld, double* __restrict__ wz,
                                                                 double* __restrict__ partial) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   const bool valid = j < N;
@@ -133,8 +133,8 @@ __global__ void __launch_bounds__(kCoarseThreads) coarse_solve_a(int m, int N, c
     double by[MM], bp[MM], z[MM];
 #pragma unroll
     for (int r = 0; r < MM; ++r) {
-      by[r] = r < m ? (double)fy[(size_t)r * N + j] : 0.0;
-      bp[r] = r < m ? (double)fp[(size_t)r * N + j] : 0.0;
+      by[r] = r < m ? (double)fy[(size_t)r * ld + j] : 0.0;
+      bp[r] = r < m ? (double)fp[(size_t)r * ld + j] : 0.0;
     }
 #pragma unroll
     for (int r = 0; r < MM; ++r) {
@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(kCoarseThreads) coarse_solve_b(int m, int N, i
                                                                 double e, const T* __restrict__ fu,
                                                                 const double* __restrict__ wz,
                                                                 const double* __restrict__ partial, T* __restrict__ y,
-                                                                T* __restrict__ u, T* __restrict__ p, int freeze_u,
+                                                                T* __restrict__ u, T* __restrict__ p, int ld, int freeze_u,
                                                                 int n, CtlBox ctl, const float* __restrict__ dw) {
   __shared__ double rhs[MM], us[MM];
   for (int r = threadIdx.x; r < m; r += blockDim.x) {
@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(kCoarseThreads) coarse_solve_b(int m, int N, i
       for (int k = 0; k < MM; ++k)
         if (k < m) t += A[r * m + k] * us[k];
       yv[r] = wz[(size_t)N * m + (size_t)j * m + r] - e * t;
-      y[(size_t)r * N + j] = (T)yv[r];
+      y[(size_t)r * ld + j] = (T)yv[r];
     } else {
       yv[r] = 0.0;
     }
@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(kCoarseThreads) coarse_solve_b(int m, int N, i
 #pragma unroll
       for (int k = 0; k < MM; ++k)
         if (k < m) t += A[r * m + k] * yv[k];
-      p[(size_t)r * N + j] = (T)(wz[(size_t)j * m + r] - c * t);
+      p[(size_t)r * ld + j] = (T)(wz[(size_t)j * m + r] - c * t);
     }
   }
 }
@@ -278,7 +278,7 @@ struct CoarseSmem {
 // kernel and the batched one, which runs one CTA per instance), after stage().
 template <typename T, typename C>
 __device__ __forceinline__ void coarse_cta_body(const CoarseSmem<C>& S, int m, int N, double c, double d, double e,
-                                                Vec3c<T> f, Vec3<T> x, int freeze_u, int nside, CtlBox ctl,
+                                                Vec3c<T> f, Vec3<T> x, int ld, int freeze_u, int nside, CtlBox ctl,
                                                 const float* __restrict__ dw) {
   const int mm = m * m, nm = N * m;
   const C *A = S.A;
@@ -287,8 +287,8 @@ __device__ __forceinline__ void coarse_cta_body(const CoarseSmem<C>& S, int m, i
   const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warps = nt >> 5;
   for (int i = tid; i < nm; i += nt) {   // f.y, f.p are [node r][sample j]
     const int r = i / N, j = i - r * N;
-    by[j * m + r] = (C)f.y[i];
-    bp[j * m + r] = (C)f.p[i];
+    by[j * m + r] = (C)f.y[(size_t)r * ld + j];
+    bp[j * m + r] = (C)f.p[(size_t)r * ld + j];
   }
   __syncthreads();
   for (int i = tid; i < nm; i += nt) {
@@ -339,7 +339,7 @@ __device__ __forceinline__ void coarse_cta_body(const CoarseSmem<C>& S, int m, i
     for (int k = 0; k < m; ++k) t += Ar[k] * (C)S.us[k];
     const C yv = z[i] - ec * t;
     by[i] = yv;
-    x.y[(size_t)r * N + j] = (T)yv;
+    x.y[(size_t)r * ld + j] = (T)yv;
   }
   __syncthreads();
   for (int i = tid; i < nm; i += nt) {   // p = w - c A^{-1} y
@@ -347,7 +347,7 @@ __device__ __forceinline__ void coarse_cta_body(const CoarseSmem<C>& S, int m, i
     const C* Ar = A + (size_t)j * mm + r * m;
     C t = 0;
     for (int k = 0; k < m; ++k) t += Ar[k] * by[j * m + k];
-    x.p[(size_t)r * N + j] = (T)(w[i] - cc * t);
+    x.p[(size_t)r * ld + j] = (T)(w[i] - cc * t);
   }
 }
 
@@ -356,14 +356,14 @@ __device__ __forceinline__ void coarse_cta_body(const CoarseSmem<C>& S, int m, i
 template <typename T, typename C>
 __global__ void __launch_bounds__(kCoarseCtaThreads) coarse_solve_cta(int m, int N, const C* __restrict__ Ainv,
                                                                      const double* __restrict__ Minv, double c,
-                                                                     double d, double e, Vec3c<T> f, Vec3<T> x,
+                                                                     double d, double e, Vec3c<T> f, Vec3<T> x, int ld,
                                                                      int freeze_u, int nside, CtlBox ctl,
                                                                      const float* __restrict__ dw) {
   extern __shared__ __align__(16) double sm[];
   const CoarseSmem<C> S(sm, m, N);
   S.stage(m, N, Ainv, Minv);
   pdl_enter();
-  coarse_cta_body<T, C>(S, m, N, c, d, e, f, x, freeze_u, nside, ctl, dw);
+  coarse_cta_body<T, C>(S, m, N, c, d, e, f, x, ld, freeze_u, nside, ctl, dw);
 }
 
 // The coarsest solves of a batch of instances (FP32 cycles), CTA b for
@@ -377,7 +377,7 @@ __global__ void __launch_bounds__(kCoarseCtaThreads) batch_coarse_kernel(const B
   extern __shared__ __align__(16) double sm[];
   const CoarseSmem<float> S(sm, q.m, q.N);
   S.stage(q.m, q.N, q.Ainv32, q.Minv);
-  coarse_cta_body<float, float>(S, q.m, q.N, q.c, q.d, q.e, q.f, q.x, 0, q.nside, q.ctl, q.dw);
+  coarse_cta_body<float, float>(S, q.m, q.N, q.c, q.d, q.e, q.f, q.x, q.ld, 0, q.nside, q.ctl, q.dw);
 }
 
 // FP32 copy of the A_j^{-1} for the FP32 coarse solve.
@@ -388,7 +388,7 @@ __global__ void cast_ainv_kernel(const double* __restrict__ a, float* __restrict
 
 template <typename T, int MM>
 cudaError_t coarse_solve_mm(const CoarseData& C, double c, double d, double e, Vec3c<T> f, Vec3<T> x,
-                            cudaStream_t s, int freeze_u) {
+                            cudaStream_t s, int freeze_u, int ld) {
   using Cm = std::conditional_t<sizeof(T) == 4, float, double>;   // precision of the per-sample products
   const Cm* ainv = nullptr;
   if constexpr (sizeof(T) == 4) ainv = C.Ainv32;
@@ -403,14 +403,14 @@ cudaError_t coarse_solve_mm(const CoarseData& C, double c, double d, double e, V
     }
     const cudaError_t ek = launch_k(coarse_solve_cta<T, Cm>, dim3(1), dim3(C.N * C.m > 512 ? 1024 : 512),
                                     coarse_cta_smem<Cm>(C.N, C.m), s, C.m, C.N, ainv, (const double*)C.Minv, c, d, e,
-                                    f, x, freeze_u, C.n, C.ctl, C.dw);
+                                    f, x, ld, freeze_u, C.n, C.ctl, C.dw);
     count_launches(1);
     return ek != cudaSuccess ? ek : cudaGetLastError();
   }
   const int nblk = (C.N + kCoarseThreads - 1) / kCoarseThreads;
-  coarse_solve_a<T, MM><<<nblk, kCoarseThreads, 0, s>>>(C.m, C.N, C.Ainv, c, f.y, f.p, C.wz, C.partial);
+  coarse_solve_a<T, MM><<<nblk, kCoarseThreads, 0, s>>>(C.m, C.N, C.Ainv, c, f.y, f.p, ld, C.wz, C.partial);
   coarse_solve_b<T, MM><<<nblk, kCoarseThreads, 0, s>>>(C.m, C.N, nblk, C.Ainv, C.Minv, c, d, e, f.u, C.wz,
-                                                         C.partial, x.y, x.u, x.p, freeze_u, C.n, C.ctl, C.dw);
+                                                         C.partial, x.y, x.u, x.p, ld, freeze_u, C.n, C.ctl, C.dw);
   count_launches(2);
   return cudaGetLastError();
 }
@@ -419,10 +419,11 @@ cudaError_t coarse_solve_mm(const CoarseData& C, double c, double d, double e, V
 
 template <typename T>
 cudaError_t launch_coarse_solve(const CoarseData& C, double c, double d, double e, Vec3c<T> f, Vec3<T> x,
-                                cudaStream_t s, int freeze_u) {
-  if (C.m == 1) return coarse_solve_mm<T, 1>(C, c, d, e, f, x, s, freeze_u);
-  if (C.m == 9) return coarse_solve_mm<T, 9>(C, c, d, e, f, x, s, freeze_u);
-  if (C.m == 49) return coarse_solve_mm<T, 49>(C, c, d, e, f, x, s, freeze_u);
+                                cudaStream_t s, int freeze_u, int ld) {
+  if (ld == 0) ld = C.N;
+  if (C.m == 1) return coarse_solve_mm<T, 1>(C, c, d, e, f, x, s, freeze_u, ld);
+  if (C.m == 9) return coarse_solve_mm<T, 9>(C, c, d, e, f, x, s, freeze_u, ld);
+  if (C.m == 49) return coarse_solve_mm<T, 49>(C, c, d, e, f, x, s, freeze_u, ld);
   return cudaErrorInvalidValue;
 }
 
@@ -669,8 +670,8 @@ template cudaError_t launch_galerkin_coarse_solve<float>(const CoarseData&, cons
                                                          Vec3c<float>, Vec3<float>, cudaStream_t);
 
 template cudaError_t launch_coarse_solve<double>(const CoarseData&, double, double, double, Vec3c<double>,
-                                                 Vec3<double>, cudaStream_t, int);
+                                                 Vec3<double>, cudaStream_t, int, int);
 template cudaError_t launch_coarse_solve<float>(const CoarseData&, double, double, double, Vec3c<float>,
-                                                Vec3<float>, cudaStream_t, int);
+                                                Vec3<float>, cudaStream_t, int, int);
 
 }  // namespace cmg

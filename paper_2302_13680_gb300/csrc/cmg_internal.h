@@ -64,11 +64,28 @@ struct LevelView {
   const double* a64;      // diag(A_j) = sum of the four faces per node-sample (FP64, finest grid only, else null)
   CtlBox ctl{};           // nodes with a control basis function (elsewhere u_i = 0, no control row)
   const float* dw = nullptr;   // per-node factor on d (semismooth Newton active sets); null = 1
+  int ldk = 0;            // sample stride of the face arrays
+  int nr = 0;             // samples of the problem: N, less the padding of a padded FP32 view (kPadFace)
+  int ld32 = 0;           // sample stride of the handle's FP32 work vectors
   // FP32 views: 0 (default) = the per-node Schur scalar of Eq. (13) (the sum
   // over samples for u_i, 1/sigma_i and u_i) in FP64 from the lanes' FP32
   // partial sums; 1 = that work in FP32 as well (all-FP32 option)
   int ctl32 = 0;
 };
+
+// Padding of the FP32 cycle's samples.  The node kernels move four FP32 samples
+// per load where a node's row is a multiple of four; for other sample counts
+// (N >= kPadFrom, averaged coarse grids) the handle's own FP32 arrays have
+// rows of padded_samples(N), and the FP32 cycle runs on that many.  The extra
+// samples have faces kPadFace and zero data: their equations are decoupled
+// from the rest by 1/kPadFace (y, p of about h^2 u / kPadFace, some 1e-15 of a
+// real sample's, below half an FP32 unit of every sum over samples), and the
+// refinement keeps their residual at zero and out of its norm (recur_item).
+// N = 125 against 128 samples, scalar loads: half-sweep at n = 255 55 against
+// 41 us, V(2,2) cycle at n = 127 363 against 254 us.
+constexpr float kPadFace = 1e15f;
+constexpr int kPadFrom = 8;
+inline int padded_samples(int N) { return N >= kPadFrom ? (N + 3) & ~3 : N; }
 
 // d_i = d * dw[node] (the control row's coupling to the adjoint at node i).
 template <typename T>
@@ -243,7 +260,7 @@ struct TailParams {
   int freeze_u;                    // coarsest solve with a zero control correction
   int lpn;                         // lanes per node (SampleMap of N)
   // coarsest grid (CoarseData) and its blocks c, d, e
-  int cm, cN;
+  int cm, cN, cld;                 // nodes, samples, sample stride of the coarsest vectors
   const double* Ainv;
   const double* Minv;
   double* wz;
@@ -271,8 +288,9 @@ int launch_residual_cast(const LevelView<double>& L, Vec3c<double> x, Vec3c<doub
 // gated anchor fold x += (*adev) d, d = 0 (nothing when *gate == 0).
 int launch_recur(const LevelView<float>& L, Vec3c<float> e, Vec3<float> r, Vec3<float> d, double wy, double* partial,
                  int max_partials, cudaStream_t s);
-cudaError_t launch_fold(const double* adev, const double* gate, Vec3<float> d, Vec3<double> x, size_t ny, size_t nu,
-                        cudaStream_t s);
+// d has rows of ld samples, x of N.
+cudaError_t launch_fold(const double* adev, const double* gate, Vec3<float> d, Vec3<double> x, size_t nodes, int N,
+                        int ld, cudaStream_t s);
 cudaError_t launch_zero3(Vec3<float> v, size_t ny, size_t nu, cudaStream_t s);
 cudaError_t launch_axpy3(double a, const double* adev, Vec3c<float> e, Vec3<double> x, size_t ny, size_t nu,
                          cudaStream_t st);
@@ -345,6 +363,7 @@ struct BatchCoarse {
   const float* dw;
   Vec3c<float> f;
   Vec3<float> x;
+  int ld;            // sample stride of f and x
 };
 
 size_t batch_coarse_smem(int N_max, int m);
@@ -402,7 +421,7 @@ cudaError_t launch_batch_anchor_control(const BatchTables& T, cudaStream_t s);
 // ---- coarsest grid (cmg_coarse.cu) ----
 template <typename T>
 cudaError_t launch_coarse_solve(const CoarseData& C, double c, double d, double e,
-                                Vec3c<T> f, Vec3<T> x, cudaStream_t s, int freeze_u = 0);
+                                Vec3c<T> f, Vec3<T> x, cudaStream_t s, int freeze_u = 0, int ld = 0);   // rows of ld (0: N)
 cudaError_t launch_coarse_setup(const CoarseData& C, const double* kx, const double* ky,
                                 double c, double G, double d, double e, cudaStream_t s);
 
@@ -427,7 +446,7 @@ cudaError_t launch_coarse_level_setup(int nf, int N, const double* kxf, const do
 // in FP32, 1/sigma from those) are built with every new sample set; the FP64
 // coarse operators only when an FP64 cycle needs them.
 cudaError_t launch_field_faces(int n, int N, int K, double amp, const double* xi, double* kap, double* kx64,
-                               double* ky64, float* kx32, float* ky32, cudaStream_t s);
+                               double* ky64, float* kx32, float* ky32, int ld32, cudaStream_t s);
 cudaError_t launch_diag64(int n, int N, const double* kx64, const double* ky64, double* inva, double* isigma,
                           double dce, double G, cudaStream_t s, const float* dw = nullptr);
 cudaError_t launch_coarse_faces64(int nf, int N, const double* kxf, const double* kyf, double* kx64, double* ky64,
@@ -436,8 +455,8 @@ cudaError_t launch_coarse_faces32(int nf, int N, const float* kxf, const float* 
                                   cudaStream_t s);
 // 1/sigma of the FP32 operator (sum over samples in FP64): FP64 isigma_d and
 // its FP32 rounding isigma32.
-cudaError_t launch_diag32(int n, int N, const float* kx32, const float* ky32, float* isigma32, double* isigma_d,
-                          double dce, double G, cudaStream_t s, const float* dw = nullptr);
+cudaError_t launch_diag32(int n, int N, const float* kx32, const float* ky32, int ld, float* isigma32,
+                          double* isigma_d, double dce, double G, cudaStream_t s, const float* dw = nullptr);
 
 // ---- vector kernels (cmg_blas.cu) ----
 constexpr int kRedBlocks = 304;    // fixed partial count: deterministic reductions
@@ -458,6 +477,9 @@ cudaError_t launch_axpy(double a, const Tx* x, Ty* y, size_t n, cudaStream_t s);
 // y = (Ty)(a * x)
 template <typename Tx, typename Ty>
 cudaError_t launch_scale_cast(double a, const Tx* x, Ty* y, size_t n, cudaStream_t s);
+// dst[r][j] = (Ty)(a * src[r][j]) for j < N, zero for N <= j < ldd; rows of lds and ldd.
+template <typename Tx, typename Ty>
+cudaError_t launch_cast_rows(double a, const Tx* src, int lds, Ty* dst, int ldd, size_t rows, int N, cudaStream_t s);
 // y = (h^2/N) yd broadcast over samples, u = 0, p = h^2 f broadcast
 cudaError_t launch_rhs(int n, int N, double h, const double* yd, const double* fsrc, double* fy,
                        double* fu, double* fp, cudaStream_t s);

@@ -94,16 +94,17 @@ __device__ __forceinline__ void residual_item(const LevelView<T>& L, const Vec3c
   const bool ctl = L.ctl.inside(iy, ix);
   if (valid) {
     const size_t o = (size_t)node * ld;
-    const T* kWp = L.kx + ((size_t)iy * (n + 1) + ix) * ld;
-    const T* kSp = L.ky + ((size_t)iy * n + ix) * ld;
+    const size_t lk = (size_t)L.ldk;
+    const T* kWp = L.kx + ((size_t)iy * (n + 1) + ix) * lk;
+    const T* kSp = L.ky + ((size_t)iy * n + ix) * lk;
     const bool hW = ix > 0, hE = ix < n - 1, hS = iy > 0, hN = iy < n - 1;
     const T uu = ctl ? ld1<T, CG>(x.u + node) : T(0);
 #pragma unroll
     for (int s = 0; s < SPL; ++s) {
       const int j = (lane + s * lpn) * V;
       if (j < N) {
-        const vec<T, V> kW = ldx<T, V, CG>(kWp + j), kE = ldx<T, V, CG>(kWp + ld + j);
-        const vec<T, V> kS = ldx<T, V, CG>(kSp + j), kN = ldx<T, V, CG>(kSp + (size_t)n * ld + j);
+        const vec<T, V> kW = ldx<T, V, CG>(kWp + j), kE = ldx<T, V, CG>(kWp + lk + j);
+        const vec<T, V> kS = ldx<T, V, CG>(kSp + j), kN = ldx<T, V, CG>(kSp + (size_t)n * lk + j);
         const vec<T, V> y = ldx<T, V, CG>(x.y + o + j), p = ldx<T, V, CG>(x.p + o + j);
         const vec<T, V> yW = ldx_if<T, V, CG>(hW, x.y + o - ld + j), yE = ldx_if<T, V, CG>(hE, x.y + o + ld + j);
         const vec<T, V> yS = ldx_if<T, V, CG>(hS, x.y + o - (size_t)n * ld + j);
@@ -232,15 +233,16 @@ __device__ __forceinline__ void rbgs_node(const LevelView<T>& L, const Vec3c<T>&
     bu = L.freeze_u ? (double)ld1<T, CG>(xs.u + node) : (double)ld1<T, CG>(f.u + node);
     isg = isigma_of<T>(L, node);
     if (L.dw) dwv = (double)L.dw[node];
-    const T* kWp = L.kx + ((size_t)iy * (n + 1) + ix) * ld;
-    const T* kSp = L.ky + ((size_t)iy * n + ix) * ld;
+    const size_t lk = (size_t)L.ldk;
+    const T* kWp = L.kx + ((size_t)iy * (n + 1) + ix) * lk;
+    const T* kSp = L.ky + ((size_t)iy * n + ix) * lk;
     const bool hW = ix > 0, hE = ix < n - 1, hS = iy > 0, hN = iy < n - 1;
 #pragma unroll
     for (int s = 0; s < SPL; ++s) {
       const int j = (lane + s * lpn) * V;
       if (j < N) {
-        const vec<T, V> kW = ldx<T, V, CG>(kWp + j), kE = ldx<T, V, CG>(kWp + ld + j);
-        const vec<T, V> kS = ldx<T, V, CG>(kSp + j), kN = ldx<T, V, CG>(kSp + (size_t)n * ld + j);
+        const vec<T, V> kW = ldx<T, V, CG>(kWp + j), kE = ldx<T, V, CG>(kWp + lk + j);
+        const vec<T, V> kS = ldx<T, V, CG>(kSp + j), kN = ldx<T, V, CG>(kSp + (size_t)n * lk + j);
         bp[s] = ldx<T, V, CG>(f.y + o + j);   // first block row: c y + A p = f_y
         by[s] = ldx<T, V, CG>(f.p + o + j);   // last block row:  A y + e u = f_p
         if constexpr (PRO) {
@@ -322,16 +324,17 @@ __device__ __forceinline__ void jacobi_item(const LevelView<T>& L, const Vec3<T>
     xu = ld1<T, CG>(x.u + node);
     isg = isigma_of<T>(L, node);
     if (L.dw) dwv = (double)L.dw[node];
-    const T* kWp = L.kx + ((size_t)iy * (n + 1) + ix) * ld;
-    const T* kSp = L.ky + ((size_t)iy * n + ix) * ld;
+    const size_t lk = (size_t)L.ldk;
+    const T* kWp = L.kx + ((size_t)iy * (n + 1) + ix) * lk;
+    const T* kSp = L.ky + ((size_t)iy * n + ix) * lk;
 #pragma unroll
     for (int s = 0; s < SPL; ++s) {
       const int j = (lane + s * lpn) * V;
       if (j < N) {
         bp[s] = ldx<T, V, CG>(r.y + o + j);
         by[s] = ldx<T, V, CG>(r.p + o + j);
-        ia[s] = inv_diag<T, V, CG>(L, o + j, ldx<T, V, CG>(kWp + j), ldx<T, V, CG>(kWp + ld + j),
-                                   ldx<T, V, CG>(kSp + j), ldx<T, V, CG>(kSp + (size_t)n * ld + j));
+        ia[s] = inv_diag<T, V, CG>(L, o + j, ldx<T, V, CG>(kWp + j), ldx<T, V, CG>(kWp + lk + j),
+                                   ldx<T, V, CG>(kSp + j), ldx<T, V, CG>(kSp + (size_t)n * lk + j));
 #pragma unroll
         for (int k = 0; k < V; ++k) {
           const T iak = ia[s].v[k];
@@ -524,9 +527,10 @@ __device__ __forceinline__ float residual_cast_item(const LevelView<double>& L, 
   const int iy = valid ? (int)(node / n) : 0, ix = valid ? (int)(node - (long)iy * n) : 0;
   const bool ctl = L.ctl.inside(iy, ix);   // local control: chi_i
   if (valid) {
-    const size_t o = (size_t)node * ld;
-    const T* kWp = L.kx + ((size_t)iy * (n + 1) + ix) * ld;
-    const T* kSp = L.ky + ((size_t)iy * n + ix) * ld;
+    const size_t o = (size_t)node * ld, o32 = (size_t)node * (size_t)L.ld32;
+    const size_t lk = (size_t)L.ldk;
+    const T* kWp = L.kx + ((size_t)iy * (n + 1) + ix) * lk;
+    const T* kSp = L.ky + ((size_t)iy * n + ix) * lk;
     const bool hW = ix > 0, hE = ix < n - 1, hS = iy > 0, hN = iy < n - 1;
     const T xu = ctl ? x.u[node] : 0.0;
     const unsigned long long xu_bits = dbits(xu);
@@ -535,8 +539,8 @@ __device__ __forceinline__ float residual_cast_item(const LevelView<double>& L, 
     for (int q = 0; q < SPL; ++q) {
       const int j = (lane + q * lpn) * V;
       if (j < N) {
-        const vec<T, V> kW = ldv<T, V>(kWp + j), kE = ldv<T, V>(kWp + ld + j);
-        const vec<T, V> kS = ldv<T, V>(kSp + j), kN = ldv<T, V>(kSp + (size_t)n * ld + j);
+        const vec<T, V> kW = ldv<T, V>(kWp + j), kE = ldv<T, V>(kWp + lk + j);
+        const vec<T, V> kS = ldv<T, V>(kSp + j), kN = ldv<T, V>(kSp + (size_t)n * lk + j);
         const vec<T, V> y = ldv<T, V>(x.y + o + j), p = ldv<T, V>(x.p + o + j);
         const vec<T, V> fy = ldv<T, V>(f.y + o + j), fp = ldv<T, V>(f.p + o + j);
         // diag(A_j) read (finest grid) instead of three FP64 adds: this pass is
@@ -588,10 +592,13 @@ __device__ __forceinline__ float residual_cast_item(const LevelView<double>& L, 
             pacc += p.v[k];
           }
         }
-        stv<float, V>(r.y + o + j, ry);
-        stv<float, V>(r.p + o + j, rp);
+        stv<float, V>(r.y + o32 + j, ry);
+        stv<float, V>(r.p + o32 + j, rp);
       }
     }
+    // padding samples have a zero right side (at most three per node)
+    if (lane == 0)
+      for (int j = N; j < L.ld32; ++j) r.y[o32 + j] = r.p[o32 + j] = 0.f;
   }
   const double psum = group_sum(pacc, lpn);
   if (valid && lane == 0) {
@@ -627,16 +634,17 @@ __device__ __forceinline__ float recur_item(const LevelView<float>& L, const Vec
   if (valid) {
     eu = e.u[node];
     const size_t o = (size_t)node * ld;
-    const T* kWp = L.kx + ((size_t)iy * (n + 1) + ix) * ld;
-    const T* kSp = L.ky + ((size_t)iy * n + ix) * ld;
+    const size_t lk = (size_t)L.ldk;
+    const T* kWp = L.kx + ((size_t)iy * (n + 1) + ix) * lk;
+    const T* kSp = L.ky + ((size_t)iy * n + ix) * lk;
     const bool hW = ix > 0, hE = ix < n - 1, hS = iy > 0, hN = iy < n - 1;
     const T uu = ctl ? eu : 0.f;
 #pragma unroll
     for (int s = 0; s < SPL; ++s) {
       const int j = (lane + s * lpn) * V;
       if (j < N) {
-        const vec<T, V> kW = ldv<T, V>(kWp + j), kE = ldv<T, V>(kWp + ld + j);
-        const vec<T, V> kS = ldv<T, V>(kSp + j), kN = ldv<T, V>(kSp + (size_t)n * ld + j);
+        const vec<T, V> kW = ldv<T, V>(kWp + j), kE = ldv<T, V>(kWp + lk + j);
+        const vec<T, V> kS = ldv<T, V>(kSp + j), kN = ldv<T, V>(kSp + (size_t)n * lk + j);
         const vec<T, V> y = ldv<T, V>(e.y + o + j), p = ldv<T, V>(e.p + o + j);
         const vec<T, V> yW = ldv_if<T, V>(hW, e.y + o - ld + j), yE = ldv_if<T, V>(hE, e.y + o + ld + j);
         const vec<T, V> yS = ldv_if<T, V>(hS, e.y + o - (size_t)n * ld + j);
@@ -659,6 +667,7 @@ __device__ __forceinline__ float recur_item(const LevelView<float>& L, const Vec
           ry.v[k] = ry.v[k] - (c * y.v[k] + ap);
           rp.v[k] = rp.v[k] - (ay + eb * uu);
           pacc += p.v[k];
+          if (V == 4 && j + k >= L.nr) ry.v[k] = rp.v[k] = 0.f;   // a padding sample: no residual (kPadFace)
           sq = fmaf(wy2 * ry.v[k], ry.v[k], sq);
           sq = fmaf(rp.v[k], rp.v[k], sq);
           dy.v[k] += y.v[k];

@@ -47,8 +47,9 @@ __device__ __forceinline__ double harmonic(double a, double b) { return 2.0 * a 
 
 // kx[iy][f][j] between grid columns f and f+1 of interior row iy (grid row iy+1);
 // ky[f][ix][j] between grid rows f and f+1 of interior column ix.
+// The FP32 copies have rows of ld32 samples, those past N the padding's kPadFace.
 __global__ void faces_kernel(int n, int N, const double* __restrict__ kap, double* __restrict__ kx64,
-                             double* __restrict__ ky64, float* __restrict__ kx32, float* __restrict__ ky32) {
+                             double* __restrict__ ky64, float* __restrict__ kx32, float* __restrict__ ky32, int ld32) {
   const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
   const long per = (long)n * (n + 1) * N;
   if (t >= 2 * per) return;
@@ -59,7 +60,9 @@ __global__ void faces_kernel(int n, int N, const double* __restrict__ kap, doubl
     const int iy = (int)(face / (n + 1)), f = (int)(face - (long)iy * (n + 1));
     const double v = harmonic(kap[((iy + 1) * g + f) * N + j], kap[((iy + 1) * g + f + 1) * N + j]);
     kx64[t] = v;
-    kx32[t] = (float)v;
+    kx32[(size_t)face * ld32 + j] = (float)v;
+    if (j == N - 1)
+      for (int q = N; q < ld32; ++q) kx32[(size_t)face * ld32 + q] = kPadFace;
   } else {
     const long tt = t - per;
     const long face = tt / N;
@@ -67,7 +70,9 @@ __global__ void faces_kernel(int n, int N, const double* __restrict__ kap, doubl
     const int f = (int)(face / n), ix = (int)(face - (long)f * n);
     const double v = harmonic(kap[((size_t)f * g + ix + 1) * N + j], kap[((size_t)(f + 1) * g + ix + 1) * N + j]);
     ky64[tt] = v;
-    ky32[tt] = (float)v;
+    ky32[(size_t)face * ld32 + j] = (float)v;
+    if (j == N - 1)
+      for (int q = N; q < ld32; ++q) ky32[(size_t)face * ld32 + q] = kPadFace;
   }
 }
 
@@ -167,18 +172,18 @@ __global__ void coarse_faces32_kernel(int nf, int N, const float* __restrict__ k
 // FP32 faces and 1/a_j in FP32 as the FP32 sweeps form them, the sum over
 // samples and the quotient in FP64; written in FP64 (isigma_d, read by the
 // FP32 cycle's Schur scalar) and rounded to FP32 (isigma32, all-FP32 option).
-__global__ void diag32_kernel(int n, int N, const float* __restrict__ kx, const float* __restrict__ ky,
+__global__ void diag32_kernel(int n, int N, const float* __restrict__ kx, const float* __restrict__ ky, int ld,
                               float* __restrict__ isigma32, double* __restrict__ isigma_d, double dce, double G,
                               const float* __restrict__ dw) {
   const long warp = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (warp >= (long)n * n) return;
   const int iy = (int)(warp / n), ix = (int)(warp - (long)iy * n);
-  const float* kW = kx + ((size_t)iy * (n + 1) + ix) * N;
-  const float* kS = ky + ((size_t)iy * n + ix) * N;
+  const float* kW = kx + ((size_t)iy * (n + 1) + ix) * ld;
+  const float* kS = ky + ((size_t)iy * n + ix) * ld;
   double s = 0.0;
   for (int j = lane; j < N; j += 32) {
-    const float ia = __frcp_rn((kW[j] + kW[N + j]) + (kS[j] + kS[(size_t)n * N + j]));
+    const float ia = __frcp_rn((kW[j] + kW[ld + j]) + (kS[j] + kS[(size_t)n * ld + j]));
     s = fma((double)ia, (double)ia, s);
   }
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
@@ -248,7 +253,7 @@ cudaError_t launch_level_setup(int n, int N, int K, double amp, const double* xi
   double* gx = kap + (size_t)(n + 2) * (n + 2) * N;
   field_x_kernel<<<blocks_for((long)(n + 2) * N, 256), 256, 0, s>>>(n, N, K, xi, gx);
   field_kernel<<<blocks_for((long)((n + 1) / 2 + 1) * (n + 2) * N, 256), 256, 0, s>>>(n, N, amp, gx, kap);
-  faces_kernel<<<blocks_for(2L * n * (n + 1) * N, 256), 256, 0, s>>>(n, N, kap, kx64, ky64, kx32, ky32);
+  faces_kernel<<<blocks_for(2L * n * (n + 1) * N, 256), 256, 0, s>>>(n, N, kap, kx64, ky64, kx32, ky32, N);
   diag_kernel<<<blocks_for((long)n * n * 32, 256), 256, 0, s>>>(n, N, kx64, ky64, inva, isigma, d * c * e, G);
   count_launches(4);
   return cudaGetLastError();
@@ -262,11 +267,11 @@ cudaError_t launch_diag_sum(int n, int N, const double* kx, const double* ky, do
 
 // Finest grid (or a nodal grid): field and FP64 + FP32 faces only.
 cudaError_t launch_field_faces(int n, int N, int K, double amp, const double* xi, double* kap, double* kx64,
-                               double* ky64, float* kx32, float* ky32, cudaStream_t s) {
+                               double* ky64, float* kx32, float* ky32, int ld32, cudaStream_t s) {
   double* gx = kap + (size_t)(n + 2) * (n + 2) * N;
   field_x_kernel<<<blocks_for((long)(n + 2) * N, 256), 256, 0, s>>>(n, N, K, xi, gx);
   field_kernel<<<blocks_for((long)((n + 1) / 2 + 1) * (n + 2) * N, 256), 256, 0, s>>>(n, N, amp, gx, kap);
-  faces_kernel<<<blocks_for(2L * n * (n + 1) * N, 256), 256, 0, s>>>(n, N, kap, kx64, ky64, kx32, ky32);
+  faces_kernel<<<blocks_for(2L * n * (n + 1) * N, 256), 256, 0, s>>>(n, N, kap, kx64, ky64, kx32, ky32, ld32);
   count_launches(3);
   return cudaGetLastError();
 }
@@ -295,9 +300,9 @@ cudaError_t launch_coarse_faces32(int nf, int N, const float* kxf, const float* 
   return cudaGetLastError();
 }
 
-cudaError_t launch_diag32(int n, int N, const float* kx32, const float* ky32, float* isigma32, double* isigma_d,
-                          double dce, double G, cudaStream_t s, const float* dw) {
-  diag32_kernel<<<blocks_for((long)n * n * 32, 256), 256, 0, s>>>(n, N, kx32, ky32, isigma32, isigma_d, dce, G, dw);
+cudaError_t launch_diag32(int n, int N, const float* kx32, const float* ky32, int ld, float* isigma32,
+                          double* isigma_d, double dce, double G, cudaStream_t s, const float* dw) {
+  diag32_kernel<<<blocks_for((long)n * n * 32, 256), 256, 0, s>>>(n, N, kx32, ky32, ld, isigma32, isigma_d, dce, G, dw);
   count_launches(1);
   return cudaGetLastError();
 }

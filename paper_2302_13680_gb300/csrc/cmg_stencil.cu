@@ -186,6 +186,35 @@ __global__ void fold_kernel(const double* __restrict__ adev, const double* __res
   }
 }
 
+// The same where d's rows are padded (ld > N, a multiple of 4): a thread takes
+// four samples of d at a time.
+__global__ void fold_rows_kernel(const double* __restrict__ adev, const double* __restrict__ gate, Vec3<float> d,
+                                 Vec3<double> x, size_t nodes, int N, int ld) {
+  pdl_enter();
+  if (*gate == 0.0) return;
+  const double a = *adev;
+  const size_t per = (size_t)ld / 4, total = nodes * per;
+  const size_t stride = (size_t)gridDim.x * blockDim.x;
+  const size_t t0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  for (size_t i = t0; i < 2 * total; i += stride) {
+    const bool isp = i >= total;
+    const size_t c = isp ? i - total : i, node = c / per;
+    const int j = (int)(c - node * per) * 4;
+    float4* dv = reinterpret_cast<float4*>((isp ? d.p : d.y) + node * ld + j);
+    const float4 dd = *dv;
+    const float e[4] = {dd.x, dd.y, dd.z, dd.w};
+    double* xv = (isp ? x.p : x.y) + node * N + j;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (j + k < N) xv[k] = fma(a, (double)e[k], xv[k]);
+    *dv = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  for (size_t i = t0; i < nodes; i += stride) {
+    x.u[i] = fma(a, (double)d.u[i], x.u[i]);
+    d.u[i] = 0.f;
+  }
+}
+
 // (y, u, p) = 0 for an FP32 level vector (a kernel, so that it can be a
 // programmatic dependent of the kernels around it).
 __global__ void zero3_kernel(Vec3<float> v, size_t ny, size_t nu) {
@@ -322,7 +351,9 @@ cudaError_t launch_rbgs_zero(const LevelView<T>& L, Vec3<T> x, Vec3c<T> f, cudaS
 template <typename T>
 cudaError_t launch_rbgs_prolong(const LevelView<T>& L, Vec3<T> x, Vec3c<T> f, Vec3c<T> e, int nc, cudaStream_t st) {
   const long groups = colour_count(L.n, 0);
-  const SampleMap m = choose_map(L.N, sizeof(T), groups, L.spl_target);
+  SampleMap m = choose_map(L.N, sizeof(T), groups, L.spl_target);
+  // 16 samples per lane take 128 registers here (the coarse loads): eight then
+  if (m.V * m.spl > 8 && (L.spl_target & 15) == 0) m = choose_map(L.N, sizeof(T), groups, L.spl_target | 2);
   const unsigned grid = grid_for(groups, m.lpn);
   cudaError_t e_ = cudaSuccess;
   CMG_DISPATCH(T, m, (e_ = launch_k(rbgs_prolong_kernel<T, V, SPL>, grid, kBlock, 0, st, L, x, f, e, nc, m.lpn)));
@@ -397,12 +428,14 @@ int launch_recur(const LevelView<float>& L, Vec3c<float> e, Vec3<float> r, Vec3<
   return (int)grid;
 }
 
-cudaError_t launch_fold(const double* adev, const double* gate, Vec3<float> d, Vec3<double> x, size_t ny, size_t nu,
-                        cudaStream_t st) {
-  const size_t total = ny + nu;
+cudaError_t launch_fold(const double* adev, const double* gate, Vec3<float> d, Vec3<double> x, size_t nodes, int N,
+                        int ld, cudaStream_t st) {
+  const size_t ny = nodes * N, total = ny + nodes;
   size_t blocks = (total + kBlock - 1) / kBlock;
   if (blocks > 152 * 16) blocks = 152 * 16;
-  const cudaError_t e_ = launch_k(fold_kernel, dim3((unsigned)blocks), dim3(kBlock), 0, st, adev, gate, d, x, ny, nu);
+  const cudaError_t e_ =
+      ld == N ? launch_k(fold_kernel, dim3((unsigned)blocks), dim3(kBlock), 0, st, adev, gate, d, x, ny, nodes)
+              : launch_k(fold_rows_kernel, dim3((unsigned)blocks), dim3(kBlock), 0, st, adev, gate, d, x, nodes, N, ld);
   if (e_ != cudaSuccess) return e_;
   count_launches(1);
   return e_ != cudaSuccess ? e_ : cudaGetLastError();

@@ -47,8 +47,8 @@ __device__ void coarse_cta(const TailParams<T>& P, const Vec3<T>& x, const Vec3<
     double by[MM], bp[MM], z[MM];
 #pragma unroll
     for (int r = 0; r < MM; ++r) {
-      by[r] = r < m ? (double)ld1<T, true>(f.y + (size_t)r * N + j) : 0.0;
-      bp[r] = r < m ? (double)ld1<T, true>(f.p + (size_t)r * N + j) : 0.0;
+      by[r] = r < m ? (double)ld1<T, true>(f.y + (size_t)r * P.cld + j) : 0.0;
+      bp[r] = r < m ? (double)ld1<T, true>(f.p + (size_t)r * P.cld + j) : 0.0;
     }
 #pragma unroll
     for (int r = 0; r < MM; ++r) {
@@ -113,7 +113,7 @@ __device__ void coarse_cta(const TailParams<T>& P, const Vec3<T>& x, const Vec3<
         for (int k = 0; k < MM; ++k)
           if (k < m) t += A[r * m + k] * us[k];
         yv[r] = P.wz[(size_t)N * m + (size_t)j * m + r] - e * t;
-        x.y[(size_t)r * N + j] = (T)yv[r];
+        x.y[(size_t)r * P.cld + j] = (T)yv[r];
       }
     }
 #pragma unroll
@@ -123,7 +123,7 @@ __device__ void coarse_cta(const TailParams<T>& P, const Vec3<T>& x, const Vec3<
 #pragma unroll
         for (int k = 0; k < MM; ++k)
           if (k < m) t += A[r * m + k] * yv[k];
-        x.p[(size_t)r * N + j] = (T)(P.wz[(size_t)j * m + r] - c * t);
+        x.p[(size_t)r * P.cld + j] = (T)(P.wz[(size_t)j * m + r] - c * t);
       }
     }
   }

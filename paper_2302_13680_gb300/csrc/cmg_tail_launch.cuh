@@ -69,7 +69,7 @@ cudaError_t launch_mm(const TailParams<T>& P, cudaStream_t s) {
 
 template <typename T>
 cudaError_t launch(const TailParams<T>& P, cudaStream_t s) {
-  const SampleMap m = choose_map(P.cN, sizeof(T), 0);
+  const SampleMap m = choose_map(P.lev[0].L.N, sizeof(T), 0);
   if (m.spl > 4 || P.nlev > kTailMax || P.cN > kTailThreads * 8) return cudaErrorNotSupported;
   const int vmax = 16 / (int)sizeof(T);
   if (m.V == 1) {
