@@ -12,6 +12,8 @@
 #include <algorithm>
 #include <type_traits>
 
+#include <cooperative_groups.h>
+
 #include "cmg_common.cuh"
 
 namespace cmg {
@@ -641,6 +643,89 @@ __global__ void galerkin_coarse_solve_kernel(int n, int N, const double* __restr
   }
 }
 
+// The same elimination for m <= 9 by a cluster of eight CTAs, each with an eighth of the
+// samples (its inverses and vectors in shared memory, a thread per (sample,
+// row)); the partial control sums are added over the cluster in rank order
+// and every CTA then solves the control system.  The single-CTA form above
+// gives a thread a whole sample, reads the inverses from memory and has one
+// SM's FP64 pipe: 47 us at N = 64, once per cycle.
+constexpr int kGalClusterThreads = 256;
+template <typename T>
+__global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(kGalClusterThreads)
+    galerkin_coarse_cluster_kernel(int n, int N, const double* __restrict__ Ainv, const double* __restrict__ Minv,
+                                   const __grid_constant__ Stencil9 M, double c, double d, double e, Vec3c<T> f,
+                                   Vec3<T> x) {
+  namespace cg = cooperative_groups;
+  const cg::cluster_group cl = cg::this_cluster();
+  extern __shared__ __align__(16) double gsm[];
+  __shared__ double part[16], sum[16], rhs[16], us[16], mu[16];
+  const int m = n * n, mm = m * m, per = (N + 7) / 8, tid = threadIdx.x, lane = tid & 31;
+  const int j0 = min(N, (int)cl.block_rank() * per), cnt = min(N, j0 + per) - j0, nm = cnt * m;
+  double *A = gsm, *fy = A + (size_t)per * mm, *w = fy + per * m, *t = w + per * m, *z = t + per * m;
+  for (int i = tid; i < cnt * mm; i += kGalClusterThreads) A[i] = Ainv[(size_t)j0 * mm + i];
+  pdl_enter();   // the inverses are written by set-up kernels only
+  for (int i = tid; i < nm; i += kGalClusterThreads) {   // f.y, f.p are [node r][sample j]
+    const int r = i / cnt, q = i - r * cnt;
+    fy[q * m + r] = (double)f.y[(size_t)r * N + j0 + q];
+    t[q * m + r] = (double)f.p[(size_t)r * N + j0 + q];
+  }
+  // out = A_j in, one thread per (sample, row)
+  const auto product = [&](int i, const double* in) {
+    const int q = i / m, r = i - q * m;
+    const double* Ar = A + (size_t)q * mm + r * m;
+    double s = 0.0;
+    for (int k = 0; k < m; ++k) s = fma(Ar[k], in[q * m + k], s);
+    return s;
+  };
+  const auto masses = [&](int i, const double* v) { return mass_apply(M, v + (i / m) * m, n, i % m); };
+  __syncthreads();
+  for (int i = tid; i < nm; i += kGalClusterThreads) w[i] = product(i, t);             // A^{-1} f_p
+  __syncthreads();
+  for (int i = tid; i < nm; i += kGalClusterThreads) t[i] = fy[i] - c * masses(i, w);
+  __syncthreads();
+  for (int i = tid; i < nm; i += kGalClusterThreads) z[i] = product(i, t);
+  __syncthreads();
+  for (int r = tid >> 5; r < m; r += kGalClusterThreads / 32) {
+    double s = 0.0;
+    for (int q = lane; q < cnt; q += 32) s += z[q * m + r];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) part[r] = s;
+  }
+  cl.sync();
+  if (tid < m) {
+    double s = 0.0;
+    for (int b = 0; b < 8; ++b) s += cl.map_shared_rank(part, b)[tid];
+    sum[tid] = s;
+  }
+  cl.sync();   // nobody leaves while its sums are read
+  if (tid < m) rhs[tid] = (double)f.u[tid] - d * mass_apply(M, sum, n, tid);
+  __syncthreads();
+  if (tid < m) {
+    double s = 0.0;
+    for (int k = 0; k < m; ++k) s = fma(Minv[tid * m + k], rhs[k], s);
+    us[tid] = s;
+    if (cl.block_rank() == 0) x.u[tid] = (T)s;
+  }
+  __syncthreads();
+  if (tid < m) mu[tid] = mass_apply(M, us, n, tid);   // M u
+  __syncthreads();
+  for (int i = tid; i < nm; i += kGalClusterThreads) {
+    const int q = i / m, r = i - q * m;
+    const double* Ar = A + (size_t)q * mm + r * m;
+    double s = 0.0;
+    for (int k = 0; k < m; ++k) s = fma(Ar[k], mu[k], s);
+    w[i] -= e * s;   // y_j
+    x.y[(size_t)r * N + j0 + q] = (T)w[i];
+  }
+  __syncthreads();
+  for (int i = tid; i < nm; i += kGalClusterThreads) t[i] = fy[i] - c * masses(i, w);
+  __syncthreads();
+  for (int i = tid; i < nm; i += kGalClusterThreads) {
+    const int q = i / m, r = i - q * m;
+    x.p[(size_t)r * N + j0 + q] = (T)product(i, t);
+  }
+}
+
 }  // namespace
 
 cudaError_t launch_galerkin_coarse_setup(const CoarseData& C, const double* a9, const Stencil9& M, double c,
@@ -658,6 +743,20 @@ template <typename T>
 cudaError_t launch_galerkin_coarse_solve(const CoarseData& C, const Stencil9& M, double c, double d, double e,
                                          Vec3c<T> f, Vec3<T> x, cudaStream_t s) {
   if (C.m > kMaxCoarseM || C.N > 1024) return cudaErrorInvalidValue;
+  if (C.m <= 9) {
+    const size_t per = (size_t)(C.N + 7) / 8, smem = per * (C.m * C.m + 4 * C.m) * sizeof(double);   // <= 120 KB
+    static bool attr = false;
+    if (!attr) {
+      const cudaError_t ea = cudaFuncSetAttribute(galerkin_coarse_cluster_kernel<T>,
+                                                  cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024);
+      if (ea != cudaSuccess) return ea;
+      attr = true;
+    }
+    const cudaError_t e_ = launch_k(galerkin_coarse_cluster_kernel<T>, dim3(8), dim3(kGalClusterThreads), smem, s, C.n,
+                                    C.N, (const double*)C.Ainv, (const double*)C.Minv, M, c, d, e, f, x);
+    count_launches(1);
+    return e_;
+  }
   const int threads = std::max(32, std::min(1024, (std::max(C.N, C.m) + 31) / 32 * 32));
   galerkin_coarse_solve_kernel<T><<<1, threads, 0, s>>>(C.n, C.N, C.Ainv, C.Minv, M, c, d, e, f, x, C.wz);
   count_launches(1);

@@ -128,6 +128,40 @@ __device__ __forceinline__ void nine_neighbours(int n, int iy, int ix, bool* ok,
   }
 }
 
+// The mass stencil and the constants of the per-sample work in T, rounded on the
+// host: in the kernels the conversions from FP64 went through the FP64 pipe
+// (two lanes per clock and SM), a dozen per node-sample in the FP32 residual.
+template <typename T>
+struct MassT {
+  T w[9];         // M_l
+  T c, e;         // the finest grid's c, e
+  T cd, ed;       // diagonal entries c M_ii, e M_ii
+};
+template <typename T>
+MassT<T> mass_t(const Stencil9& M, double c, double e) {
+  MassT<T> m;
+  for (int k = 0; k < 9; ++k) m.w[k] = (T)M.w[k];
+  m.c = (T)c;
+  m.e = (T)e;
+  m.cd = (T)(c * M.w[4]);
+  m.ed = (T)(e * M.w[4]);
+  return m;
+}
+
+// (M u)_i of the node of an LPN-lane group (LPN = 16 or 32), with or without
+// the centre: lane k < 9 takes neighbour k, then a group sum, instead of
+// every lane adding nine terms one after another in FP64.
+template <typename T, int LPN>
+__device__ __forceinline__ double group_mass_u(const Stencil9& M, const T* __restrict__ u, int n, int iy, int ix, int l,
+                                               bool valid, bool centre) {
+  const int ny = iy + l / 3 - 1, nx = ix + l % 3 - 1;
+  double v = 0.0;
+  if (valid && l < 9 && (centre || l != 4) && ny >= 0 && ny < n && nx >= 0 && nx < n)
+    v = M.w[l] * (double)u[ny * n + nx];
+  for (int o = LPN / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
 // psum[i] = sum_j p[i][j]: the lanes' parts in T, then a fixed-order FP64
 // shuffle reduction; one warp per node (the three-launch residual and the
 // four-colour sweep above 32 kGsMaxR samples).
@@ -152,15 +186,14 @@ __global__ void galerkin_psum_kernel(long nodes, int N, const T* __restrict__ p,
 //   r_y = f_y - (c (M y_j)_i + (A_j p_j)_i),  r_p = f_p - ((A_j y_j)_i + e (M u)_i),
 // with (M u)_i from the control-row kernel (mu).
 template <typename T>
-__global__ void residual9_yp_kernel(int n, int N, const T* __restrict__ a9, Stencil9 M, double c, double e,
+__global__ void residual9_yp_kernel(int n, int N, const T* __restrict__ a9, const __grid_constant__ MassT<T> M,
                                     const double* __restrict__ mu, Vec3c<T> x, Vec3c<T> f, Vec3<T> r) {
   pdl_enter();
   const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
   const size_t nodes = (size_t)n * n;
   if (t >= (long)nodes * N) return;
-  const int j = (int)(t % N);
-  const long i = t / N;
-  const int iy = (int)(i / n), ix = (int)(i - (long)iy * n);
+  const int i = (int)(t / N), j = (int)(t - (long)i * N);
+  const int iy = i / n, ix = i - iy * n;
   T Ap = 0, Ay = 0, My = 0;
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
@@ -171,9 +204,9 @@ __global__ void residual9_yp_kernel(int n, int N, const T* __restrict__ a9, Sten
     const T yv = x.y[nb * N + j], pv = x.p[nb * N + j];
     Ap = fma(a, pv, Ap);
     Ay = fma(a, yv, Ay);
-    My = fma((T)M.w[k], yv, My);
+    My = fma(M.w[k], yv, My);
   }
-  const T sy = (T)c * My + Ap, sp = Ay + (T)e * (T)mu[i];
+  const T sy = M.c * My + Ap, sp = Ay + M.e * (T)mu[i];
   const size_t o = (size_t)i * N + j;
   r.y[o] = f.y ? f.y[o] - sy : sy;
   r.p[o] = f.y ? f.p[o] - sp : sp;
@@ -208,26 +241,24 @@ __global__ void residual9_u_kernel(int n, const double* __restrict__ psum, Stenc
 //   r_y = f_y - (c (M y_j)_i + (A_j p_j)_i),
 //   r_p = f_p - ((A_j y_j)_i + e (M u)_i),
 //   r_u = f_u - (G (M u)_i + d sum_j (M p_j)_i).
-// (M u)_i in FP64 by every lane (the same nine loads); the control row's
+// (M u)_i in FP64 by the group; the control row's
 // sum over samples is formed from the p values the state rows load.
 // r = S x when f.y == nullptr.
 template <typename T>
-__global__ void residual9_kernel(int n, int N, const T* __restrict__ a9, Stencil9 M, double c, double G, double d,
-                                 double e, Vec3c<T> x, Vec3c<T> f, Vec3<T> r) {
+__global__ void residual9_kernel(int n, int N, const T* __restrict__ a9, const __grid_constant__ Stencil9 M,
+                                 const __grid_constant__ MassT<T> mt, double G, double d, double e, Vec3c<T> x,
+                                 Vec3c<T> f, Vec3<T> r) {
   pdl_enter();
   const long i = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   const size_t nodes = (size_t)n * n;
   if (i >= (long)nodes) return;   // whole warp
-  const int iy = (int)(i / n), ix = (int)(i - (long)iy * n);
+  const int iy = (int)i / n, ix = (int)i - iy * n;
   bool ok[9];
   int nb[9];
   nine_neighbours(n, iy, ix, ok, nb);
-  double Mu = 0.0;
-#pragma unroll
-  for (int k = 0; k < 9; ++k)
-    if (ok[k]) Mu = fma(M.w[k], (double)x.u[nb[k]], Mu);
-  const T eMu = (T)(e * Mu), cT = (T)c;
+  const double Mu = group_mass_u<T, 32>(M, x.u, n, iy, ix, lane, true, true);
+  const T eMu = (T)(e * Mu), cT = mt.c;
   T pm = 0;   // this lane's share of sum_j (M p_j)_i
 #pragma unroll 1
   for (int j = lane; j < N; j += 32) {
@@ -237,7 +268,7 @@ __global__ void residual9_kernel(int n, int N, const T* __restrict__ a9, Stencil
       if (!ok[k]) continue;
       const T a = a9[((size_t)k * nodes + i) * N + j];
       const T yv = x.y[(size_t)nb[k] * N + j], pv = x.p[(size_t)nb[k] * N + j];
-      const T m = (T)M.w[k];
+      const T m = mt.w[k];
       Ap = fma(a, pv, Ap);
       Ay = fma(a, yv, Ay);
       My = fma(m, yv, My);
@@ -354,13 +385,17 @@ __global__ void gs4_colour_kernel(int n, int N, int cy, int cx, const T* __restr
 // between launches):
 //   B_u = f_u - G (M u)_i - d sum_j (M p_j)_i   (off-centre entries, FP64).
 // A warp takes 32 / LPN nodes, so each warp instruction of the node's FP64
-// work (the off-centre (M u)_i, the two group sums, u_i) serves as many
-// nodes: on this GPU the FP64 pipe, not memory, bounds a warp per node.
+// work (the off-centre (M u)_i, the group sum, u_i) serves as many nodes: on
+// this GPU the FP64 pipe, not memory, bounds a warp per node.  About twenty
+// FP64 instructions per warp; with the stencil converted in the kernel, (M u)_i
+// added by every lane and two group sums they were 55, and a launch took 15.5
+// us whatever the grid (n = 7, N = 64).
 template <typename T, int R, int LPN>
 __global__ void __launch_bounds__(kGBlock) gs4_colour_reg_kernel(int n, int N, int cy, int cx,
-                                                                 const T* __restrict__ a9, Stencil9 M, double c,
-                                                                 double G, double d, double e,
-                                                                 const T* __restrict__ inva,
+                                                                 const T* __restrict__ a9,
+                                                                 const __grid_constant__ Stencil9 M,
+                                                                 const __grid_constant__ MassT<T> mt, double G,
+                                                                 double d, double e, const T* __restrict__ inva,
                                                                  const double* __restrict__ isigma, Vec3<T> x,
                                                                  Vec3c<T> f) {
   pdl_enter();
@@ -371,22 +406,19 @@ __global__ void __launch_bounds__(kGBlock) gs4_colour_reg_kernel(int n, int N, i
   const long g = t / LPN;
   const int l = (int)(threadIdx.x & (LPN - 1));
   const bool valid = g < count;
-  const int iy = valid ? cy + 2 * (int)(g / nbx) : 0, ix = valid ? cx + 2 * (int)(g % nbx) : 0;
+  const int gy = (int)g / nbx, gx = (int)g - gy * nbx;
+  const int iy = valid ? cy + 2 * gy : 0, ix = valid ? cx + 2 * gx : 0;
   const size_t nodes = (size_t)n * n;
   const size_t i = (size_t)iy * n + ix;
   const double mc = M.w[4];
-  const T cd = (T)(c * mc), ed = (T)(e * mc);   // diagonal entries of the mass blocks
+  const T cd = mt.cd, ed = mt.ed;   // diagonal entries of the mass blocks
+  const double fu = valid ? (double)f.u[i] : 0.0, isg = valid ? isigma[i] : 0.0;
   bool ok[9];
   int nb[9];
   nine_neighbours(n, iy, ix, ok, nb);
   ok[4] = false;
-  double Mu = 0.0;   // off-centre (M u)_i
-  if (valid) {
-#pragma unroll
-    for (int k = 0; k < 9; ++k)
-      if (ok[k]) Mu = fma(M.w[k], (double)x.u[nb[k]], Mu);
-  }
-  const T eMu = (T)(e * Mu), cT = (T)c;
+  const double Mu = group_mass_u<T, LPN>(M, x.u, n, iy, ix, l, valid, false);   // off-centre (M u)_i
+  const T eMu = (T)(e * Mu), cT = mt.c;
   T By[R], Bp[R], ia[R];
   T tacc = 0, pm = 0;
 #pragma unroll
@@ -400,7 +432,7 @@ __global__ void __launch_bounds__(kGBlock) gs4_colour_reg_kernel(int n, int N, i
         if (!ok[k]) continue;
         const T a = a9[((size_t)k * nodes + i) * N + j];
         const T yv = x.y[(size_t)nb[k] * N + j], pv = x.p[(size_t)nb[k] * N + j];
-        const T m = (T)M.w[k];
+        const T m = mt.w[k];
         by -= cT * m * yv + a * pv;
         bp -= a * yv;
         mp = fma(m, pv, mp);
@@ -413,14 +445,11 @@ __global__ void __launch_bounds__(kGBlock) gs4_colour_reg_kernel(int n, int N, i
       ia[q] = iq;
     }
   }
-  double ts = (double)tacc, ps = (double)pm;
-  for (int o = LPN / 2; o > 0; o >>= 1) {
-    ts += __shfl_xor_sync(0xffffffffu, ts, o);
-    ps += __shfl_xor_sync(0xffffffffu, ps, o);
-  }
+  // B_u + d m_ii sum_j t_j = f_u - G (M u)_i + d sum_j (m_ii t_j - (M p_j)_i): one FP64 group sum
+  double ts = fma(mc, (double)tacc, -(double)pm);
+  for (int o = LPN / 2; o > 0; o >>= 1) ts += __shfl_xor_sync(0xffffffffu, ts, o);
   if (!valid) return;
-  const double Bu = (double)f.u[i] - G * Mu - d * ps;
-  const double u = (Bu + d * mc * ts) * isigma[i];
+  const double u = fma(d, ts, fma(-G, Mu, fu)) * isg;
   const T uT = (T)u;
 #pragma unroll
   for (int q = 0; q < R; ++q) {
@@ -523,7 +552,8 @@ cudaError_t launch_residual9(int n, int N, const T* a9, const Stencil9& M, doubl
   const long nodes = (long)n * n;
   if (n <= (sizeof(T) == 4 ? kResidual9OnePass32 : kResidual9OnePass64)) {
     const cudaError_t err =
-        launch_k(residual9_kernel<T>, blocks_for(nodes * 32), kGBlock, 0, s, n, N, a9, M, c, G, d, e, x, f, r);
+        launch_k(residual9_kernel<T>, ctas_for(nodes * 32), block_for(nodes * 32), 0, s, n, N, a9, M, mass_t<T>(M, c, e),
+                 G, d, e, x, f, r);
     count_launches(1);
     return err != cudaSuccess ? err : cudaGetLastError();
   }
@@ -533,7 +563,7 @@ cudaError_t launch_residual9(int n, int N, const T* a9, const Stencil9& M, doubl
     err = launch_k(residual9_u_kernel<T>, blocks_for(nodes), kGBlock, 0, s, n, (const double*)psum, M, G, d, x, f, r,
                    mu);
   if (err == cudaSuccess)
-    err = launch_k(residual9_yp_kernel<T>, blocks_for(nodes * N), kGBlock, 0, s, n, N, a9, M, c, e,
+    err = launch_k(residual9_yp_kernel<T>, blocks_for(nodes * N), kGBlock, 0, s, n, N, a9, mass_t<T>(M, c, e),
                    (const double*)mu, x, f, r);
   count_launches(3);
   return err != cudaSuccess ? err : cudaGetLastError();
@@ -555,14 +585,14 @@ cudaError_t launch_gs4_sweep(int n, int N, const T* a9, const Stencil9& M, doubl
     const int need = (N + lpn - 1) / lpn;
     const int R = need <= 1 ? 1 : need <= 2 ? 2 : need <= 4 ? 4 : 8;
     cudaError_t err = cudaSuccess;
+    const MassT<T> mt = mass_t<T>(M, c, e);
     for (int col = 0; col < 4 && err == cudaSuccess; ++col) {
       const int cy = col >> 1, cx = col & 1;
       const long groups = (long)((n - cx + 1) / 2) * ((n - cy + 1) / 2);
       if (groups == 0) continue;
-      const unsigned grid = blocks_for(groups * lpn);
 #define CMG_GS4(RR, LL)                                                                                         \
-  err = launch_k(gs4_colour_reg_kernel<T, RR, LL>, grid, kGBlock, 0, s, n, N, cy, cx, a9, M, c, G, d, e, inva, \
-                 isigma, x, f)
+  err = launch_k(gs4_colour_reg_kernel<T, RR, LL>, ctas_for(groups * LL), block_for(groups * LL), 0, s, n, N, cy, cx, a9, \
+                 M, mt, G, d, e, inva, isigma, x, f)
       if (lpn == 16) {
         if (R == 1) CMG_GS4(1, 16);
         else if (R == 2) CMG_GS4(2, 16);

@@ -126,6 +126,12 @@ struct CoarseData {
 };
 
 // ---- launches ----
+// CTA size of a node kernel's launch over `threads` threads: launches of one or
+// two 256-thread CTAs per SM and fewer are latency-bound, and small CTAs spread
+// their warps over more SMs, whose FP64 pipes (two lanes per clock each) then
+// share the nodes' control-row work.
+inline unsigned block_for(long threads) { return threads <= 152L * 128 ? 64u : threads <= 152L * 512 ? 128u : 256u; }
+inline unsigned ctas_for(long threads) { return (unsigned)((threads + block_for(threads) - 1) / block_for(threads)); }
 // Programmatic dependent launch for the kernels of the cycle and the
 // refinement loop (every kernel launched this way starts with pdl_enter);
 // CMG_PDL=0 in the environment turns the attribute off.

@@ -241,6 +241,7 @@ __global__ void axpy3_kernel(double a0, const double* __restrict__ adev, Vec3c<f
   }
 }
 
+// Whole CTAs of kBlock threads (the kernels that sum over their CTA).
 inline unsigned grid_for(long groups, int lpn) {
   const long threads = groups * lpn;
   return (unsigned)((threads + kBlock - 1) / kBlock);
@@ -299,9 +300,9 @@ SampleMap choose_map(int N, int elem_bytes, long items, int spl_target) {
 template <typename T>
 cudaError_t launch_residual(const LevelView<T>& L, Vec3c<T> x, Vec3c<T> f, Vec3<T> r, cudaStream_t st, double wy) {
   const SampleMap m = choose_map(L.N, sizeof(T), (long)L.n * L.n, L.spl_target);
-  const unsigned grid = grid_for((long)L.n * L.n, m.lpn);
+  const long threads = ((long)L.n * L.n) * m.lpn;
   cudaError_t e_ = cudaSuccess;
-  CMG_DISPATCH(T, m, (e_ = launch_k(residual_kernel<T, V, SPL>, grid, kBlock, 0, st, L, x, f, r, m.lpn, (T)wy)));
+  CMG_DISPATCH(T, m, (e_ = launch_k(residual_kernel<T, V, SPL>, ctas_for(threads), block_for(threads), 0, st, L, x, f, r, m.lpn, (T)wy)));
   count_launches(1);
   return e_ != cudaSuccess ? e_ : cudaGetLastError();
 }
@@ -310,9 +311,9 @@ template <typename T>
 cudaError_t launch_residual_c0(const LevelView<T>& L, Vec3c<T> x, Vec3c<T> f, Vec3<T> r, cudaStream_t st) {
   const long groups = colour_count(L.n, 0);
   const SampleMap m = choose_map(L.N, sizeof(T), groups, L.spl_target);
-  const unsigned grid = grid_for(groups, m.lpn);
+  const long threads = (groups) * m.lpn;
   cudaError_t e_ = cudaSuccess;
-  CMG_DISPATCH(T, m, (e_ = launch_k(residual_c0_kernel<T, V, SPL>, grid, kBlock, 0, st, L, x, f, r, m.lpn)));
+  CMG_DISPATCH(T, m, (e_ = launch_k(residual_c0_kernel<T, V, SPL>, ctas_for(threads), block_for(threads), 0, st, L, x, f, r, m.lpn)));
   count_launches(1);
   return e_ != cudaSuccess ? e_ : cudaGetLastError();
 }
@@ -330,9 +331,9 @@ cudaError_t launch_rbgs_half(const LevelView<T>& L, Vec3<T> x, Vec3c<T> f, int c
       if (e != cudaErrorNotSupported) return e;
     }
   }
-  const unsigned grid = grid_for(colour_count(L.n, colour), m.lpn);
+  const long threads = (colour_count(L.n, colour)) * m.lpn;
   cudaError_t e_ = cudaSuccess;
-  CMG_DISPATCH(T, m, (e_ = launch_k(rbgs_half_kernel<T, V, SPL>, grid, kBlock, 0, st, L, x, f, colour, m.lpn)));
+  CMG_DISPATCH(T, m, (e_ = launch_k(rbgs_half_kernel<T, V, SPL>, ctas_for(threads), block_for(threads), 0, st, L, x, f, colour, m.lpn)));
   count_launches(1);
   return e_ != cudaSuccess ? e_ : cudaGetLastError();
 }
@@ -341,9 +342,9 @@ template <typename T>
 cudaError_t launch_rbgs_zero(const LevelView<T>& L, Vec3<T> x, Vec3c<T> f, cudaStream_t st) {
   const long groups = colour_count(L.n, 0);
   const SampleMap m = choose_map(L.N, sizeof(T), groups, L.spl_target);
-  const unsigned grid = grid_for(groups, m.lpn);
+  const long threads = (groups) * m.lpn;
   cudaError_t e_ = cudaSuccess;
-  CMG_DISPATCH(T, m, (e_ = launch_k(rbgs_zero_kernel<T, V, SPL>, grid, kBlock, 0, st, L, x, f, m.lpn)));
+  CMG_DISPATCH(T, m, (e_ = launch_k(rbgs_zero_kernel<T, V, SPL>, ctas_for(threads), block_for(threads), 0, st, L, x, f, m.lpn)));
   count_launches(1);
   return e_ != cudaSuccess ? e_ : cudaGetLastError();
 }
@@ -354,9 +355,9 @@ cudaError_t launch_rbgs_prolong(const LevelView<T>& L, Vec3<T> x, Vec3c<T> f, Ve
   SampleMap m = choose_map(L.N, sizeof(T), groups, L.spl_target);
   // 16 samples per lane take 128 registers here (the coarse loads): eight then
   if (m.V * m.spl > 8 && (L.spl_target & 15) == 0) m = choose_map(L.N, sizeof(T), groups, L.spl_target | 2);
-  const unsigned grid = grid_for(groups, m.lpn);
+  const long threads = (groups) * m.lpn;
   cudaError_t e_ = cudaSuccess;
-  CMG_DISPATCH(T, m, (e_ = launch_k(rbgs_prolong_kernel<T, V, SPL>, grid, kBlock, 0, st, L, x, f, e, nc, m.lpn)));
+  CMG_DISPATCH(T, m, (e_ = launch_k(rbgs_prolong_kernel<T, V, SPL>, ctas_for(threads), block_for(threads), 0, st, L, x, f, e, nc, m.lpn)));
   count_launches(1);
   return e_ != cudaSuccess ? e_ : cudaGetLastError();
 }
@@ -364,9 +365,9 @@ cudaError_t launch_rbgs_prolong(const LevelView<T>& L, Vec3<T> x, Vec3c<T> f, Ve
 template <typename T>
 cudaError_t launch_jacobi_update(const LevelView<T>& L, Vec3<T> x, Vec3c<T> r, double theta, cudaStream_t st) {
   const SampleMap m = choose_map(L.N, sizeof(T), (long)L.n * L.n, L.spl_target);
-  const unsigned grid = grid_for((long)L.n * L.n, m.lpn);
+  const long threads = ((long)L.n * L.n) * m.lpn;
   cudaError_t e_ = cudaSuccess;
-  CMG_DISPATCH(T, m, (e_ = launch_k(jacobi_update_kernel<T, V, SPL>, grid, kBlock, 0, st, L, x, r, theta, m.lpn)));
+  CMG_DISPATCH(T, m, (e_ = launch_k(jacobi_update_kernel<T, V, SPL>, ctas_for(threads), block_for(threads), 0, st, L, x, r, theta, m.lpn)));
   count_launches(1);
   return e_ != cudaSuccess ? e_ : cudaGetLastError();
 }
@@ -375,9 +376,9 @@ template <typename T>
 cudaError_t launch_restrict(int nf, int N, Vec3c<T> r, Vec3<T> c, cudaStream_t st, Vec3<T> zx, int colour0) {
   const int nc = (nf - 1) / 2;
   const SampleMap m = choose_map(N, sizeof(T), (long)nc * nc);
-  const unsigned grid = grid_for((long)nc * nc, m.lpn);
+  const long threads = ((long)nc * nc) * m.lpn;
   cudaError_t e_ = cudaSuccess;
-  CMG_DISPATCH(T, m, (e_ = launch_k(restrict_kernel<T, V, SPL>, grid, kBlock, 0, st, nf, N, r, c, zx, m.lpn, colour0)));
+  CMG_DISPATCH(T, m, (e_ = launch_k(restrict_kernel<T, V, SPL>, ctas_for(threads), block_for(threads), 0, st, nf, N, r, c, zx, m.lpn, colour0)));
   count_launches(1);
   return e_ != cudaSuccess ? e_ : cudaGetLastError();
 }
@@ -385,9 +386,9 @@ cudaError_t launch_restrict(int nf, int N, Vec3c<T> r, Vec3<T> c, cudaStream_t s
 template <typename T>
 cudaError_t launch_prolong_add(int nf, int N, Vec3c<T> e, Vec3<T> x, cudaStream_t st, CtlBox ctl) {
   const SampleMap m = choose_map(N, sizeof(T), (long)nf * nf);
-  const unsigned grid = grid_for((long)nf * nf, m.lpn);
+  const long threads = ((long)nf * nf) * m.lpn;
   cudaError_t e_ = cudaSuccess;
-  CMG_DISPATCH(T, m, (e_ = launch_k(prolong_add_kernel<T, V, SPL>, grid, kBlock, 0, st, nf, N, e, x, m.lpn, ctl)));
+  CMG_DISPATCH(T, m, (e_ = launch_k(prolong_add_kernel<T, V, SPL>, ctas_for(threads), block_for(threads), 0, st, nf, N, e, x, m.lpn, ctl)));
   count_launches(1);
   return e_ != cudaSuccess ? e_ : cudaGetLastError();
 }
