@@ -1306,6 +1306,7 @@ cmg_status precondition(cmg_handle* h, const cmg_cycle& o, Vec3c<double> v, Vec3
 __device__ double block_total(const double* __restrict__ partial, int count) {
   __shared__ double sh[32];
   double v = 0.0;
+#pragma unroll 8
   for (int i = threadIdx.x; i < count; i += blockDim.x) v += partial[i];
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
@@ -1383,7 +1384,7 @@ cmg_status ir_iteration_anchor(cmg_handle* h, Vec3c<double> f, Vec3<double> x, c
   const int cnt = launch_residual_cast(view<double>(h, 0), cview(x), f, f32, 0.0, st + kSc, paper_wy(h), h->part,
                                        h->part_cap, h->stream, st + kAnchor);
   if (cnt < 0) return fail(h, CMG_ERR_CUDA, "refinement pass launch failed");
-  CK(launch_k(ir_anchor_control_kernel, dim3(1), dim3(256), 0, h->stream, (const double*)h->part, cnt, st, cond,
+  CK(launch_k(ir_anchor_control_kernel, dim3(1), dim3(1024), 0, h->stream, (const double*)h->part, cnt, st, cond,
               graph));
   count_launches(1);
   return CMG_OK;
@@ -1403,7 +1404,7 @@ cmg_status ir_iteration(cmg_handle* h, const cmg_cycle& o, Vec3c<double> f, Vec3
   CK(cycle<float>(h, o, 0, x32, cview(f32), zg));
   int cnt = launch_recur(view<float>(h, 0), cview(x32), f32, d32, paper_wy(h), h->part, h->part_cap, h->stream);
   if (cnt < 0) return fail(h, CMG_ERR_CUDA, "recursive residual launch failed");
-  CK(launch_k(ir_recur_control_kernel, dim3(1), dim3(256), 0, h->stream, (const double*)h->part, cnt, st, cond,
+  CK(launch_k(ir_recur_control_kernel, dim3(1), dim3(1024), 0, h->stream, (const double*)h->part, cnt, st, cond,
               graph));
   count_launches(1);
   if (!anchor_kernels) return CMG_OK;

@@ -27,6 +27,8 @@
 #include <string>
 #include <vector>
 
+#include <cooperative_groups.h>
+
 #include "cmg_common.cuh"
 
 using namespace cmg;
@@ -247,8 +249,125 @@ __global__ void bnd_residual_u_kernel(int n, St3 g3, St3 b3, const double* __res
   r.u[k] = f.y ? f.u[k] - su : su;
 }
 
+// One warp per node, lanes over samples (j = lane + 32 q, q < R, N <= 32 R):
+// JAC = false: the residual rows above (o = f - S x, or S x when f is null);
+// JAC = true: a whole damped collective Jacobi sweep, Eq. (11), from x into o,
+// o_i = x_i + theta S~_i^{-1} (f - S x)_i, with no residual written and read
+// back.  On Gamma the control row's sum over samples of B^T p comes from the
+// p values the state rows load, in one warp sum with Eq. (13)'s.  FIVE (the
+// finest grid): A_j has five entries and the mass is lumped, so the four
+// corner planes and eight of the mass's are zero and not touched.
+//
+// Why: bound by the FP64 pipe (two lanes per clock and SM).  A sweep was four
+// launches (sums of p, rows, control row, update), nine-point everywhere, with an
+// FP64 division by N per node-sample: 69 us on the finest grid at n = 63, N =
+// 125 and 31 us on the grids of a few hundred nodes, where it was the launches' and the
+// dependent loads' latency (the nine neighbours were loaded one branch at a time;
+// here all of a chunk's loads are in flight together, masked afterwards).
+template <int R, bool FIVE, bool JAC>
+__global__ void __launch_bounds__(kBT)
+    bnd_node_kernel(int n, int N, double rN, const double* __restrict__ a9, const double* __restrict__ m9, St3 g3, St3 b3,
+                    const double* __restrict__ inva, const double* __restrict__ isigma, double theta, Vec3c<double> x,
+                    Vec3c<double> f, Vec3<double> o) {
+  pdl_enter();
+  const size_t nodes = (size_t)(n + 1) * n;
+  const long i = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (i >= (long)nodes) return;   // whole warp
+  const int ry = (int)i / n, rx = (int)i - ry * n;
+  const bool gam = ry == 0, apply = f.y == nullptr;
+  bool ok[9];
+  size_t g[9];
+  double mk[9];
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    const int gy = ry + k / 3 - 1, gx = rx + k % 3 - 1;
+    ok[k] = gy >= 0 && gy <= n && gx >= 0 && gx < n && (!FIVE || (k & 1) || k == 4);
+    g[k] = ok[k] ? (size_t)gy * n + gx : (size_t)i;
+    mk[k] = ok[k] && (!FIVE || k == 4) ? m9[(size_t)k * nodes + i] : 0.0;
+  }
+  double Bu = 0.0, Gu = 0.0, fu = 0.0, xu = 0.0, isg = 0.0;
+  if (gam) {
+#pragma unroll
+    for (int d = -1; d <= 1; ++d)
+      if (rx + d >= 0 && rx + d < n) {
+        const double v = x.u[rx + d];
+        Bu = fma(b3.w[d + 1], v, Bu);
+        Gu = fma(g3.w[d + 1], v, Gu);
+        if (d == 0) xu = v;
+      }
+    if (!apply) fu = f.u[rx];
+    if (JAC) isg = isigma[rx];
+  }
+  const double c = mk[4] * rN, db = -b3.w[1];   // Eq. (12) at the node: c_j = M_ii / N, d = e = -B_ii
+  double sy[R], sp[R], ia[R], yc[R], pc[R], s = 0.0;
+#pragma unroll
+  for (int q = 0; q < R; ++q) {
+    const int j = lane + 32 * q;
+    const bool in = j < N;
+    const int jj = in ? j : 0;
+    double av[9], yv[9], pv[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      if (FIVE && !(k & 1) && k != 4) continue;
+      av[k] = a9[((size_t)k * nodes + i) * N + jj];
+      yv[k] = x.y[g[k] * N + jj];
+      pv[k] = x.p[g[k] * N + jj];
+    }
+    const size_t e = (size_t)i * N + jj;
+    const double fy = apply ? 0.0 : f.y[e], fp = apply ? 0.0 : f.p[e];
+    ia[q] = JAC ? inva[e] : 0.0;
+    double Ap = 0.0, Ay = 0.0, My = 0.0;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      if (FIVE && !(k & 1) && k != 4) continue;
+      const double a = ok[k] ? av[k] : 0.0, yk = ok[k] ? yv[k] : 0.0, pk = ok[k] ? pv[k] : 0.0;
+      Ap = fma(a, pk, Ap);
+      Ay = fma(a, yk, Ay);
+      if (!FIVE || k == 4) My = fma(mk[k], yk, My);
+    }
+    const double ty = fma(My, rN, Ap), tp = Ay - Bu;
+    sy[q] = apply ? ty : fy - ty;
+    sp[q] = apply ? tp : fp - tp;
+    yc[q] = yv[4];
+    pc[q] = pv[4];
+    if (gam && in) {
+      // (B^T)_{k, k+d} = B_{k+d, k} on the row's nodes (planes 3, 4, 5)
+      double Bp = b3.w[1] * pv[4];
+      if (ok[3]) Bp = fma(b3.w[2], pv[3], Bp);
+      if (ok[5]) Bp = fma(b3.w[0], pv[5], Bp);
+      s += JAC ? Bp + db * ((c * ia[q]) * (ia[q] * sp[q]) - ia[q] * sy[q]) : Bp;
+    }
+  }
+  double du = 0.0;
+  if (gam) {   // uniform over the warp
+    for (int w = 16; w > 0; w >>= 1) s += __shfl_xor_sync(0xffffffffu, s, w);
+    if (JAC) {
+      du = ((fu - Gu) + s) * isg;
+      if (lane == 0) o.u[rx] = xu + theta * du;
+    } else if (lane == 0) {
+      o.u[rx] = apply ? Gu - s : fu - (Gu - s);
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < R; ++q) {
+    const int j = lane + 32 * q;
+    if (j >= N) continue;
+    const size_t e = (size_t)i * N + j;
+    if (JAC) {
+      const double dy = ia[q] * (sp[q] - db * du);
+      const double dp = ia[q] * (sy[q] - c * dy);
+      o.y[e] = yc[q] + theta * dy;
+      o.p[e] = pc[q] + theta * dp;
+    } else {
+      o.y[e] = sy[q];
+      o.p[e] = sp[q];
+    }
+  }
+}
+
 // Damped collective Jacobi, Eq. (11): x_i += theta S~_i^{-1} r_i, one warp
-// per node.  On Gamma the node block is Eq. (12)'s arrow system with
+// per node (sample counts above the kernel's above).  On Gamma the node block is Eq. (12)'s arrow system with
 // c = M_ii / N, a_j = (A_j)_ii, d = e = -B_ii, G = G_ii, solved by Eq. (13);
 // elsewhere u_i is absent (Eq. (14)).
 __global__ void bnd_jacobi_kernel(int n, int N, const double* __restrict__ m9, const double* __restrict__ inva,
@@ -282,16 +401,25 @@ __global__ void bnd_jacobi_kernel(int n, int N, const double* __restrict__ m9, c
   if (gam && lane == 0) x.u[i] += theta * du;
 }
 
+// t = i N + j (32-bit division where it fits).
+__device__ __forceinline__ void split(long t, int N, long& i, int& j) {
+  i = t < 0x7fffffffL ? (long)((int)t / N) : t / N;
+  j = (int)(t - i * N);
+}
+
 // c = P^T r from the nf grid to the (nf-1)/2 grid, one thread per (coarse
 // node, sample); the control block (sample slot 0 of row-0 nodes) by P_x^T.
-__global__ void bnd_restrict_kernel(int nf, int N, Vec3c<double> rf, Vec3<double> cc) {
+// Given zx, the coarse iterate is cleared as well.
+__global__ void bnd_restrict_kernel(int nf, int N, Vec3c<double> rf, Vec3<double> cc, Vec3<double> zx) {
+  pdl_enter();
   const int nc = (nf - 1) / 2;
   const size_t cnodes = (size_t)(nc + 1) * nc;
   const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (long)cnodes * N) return;
-  const int j = (int)(t % N);
-  const long C = t / N;
-  const int R = (int)(C / nc), I = (int)(C % nc);
+  long C;
+  int j;
+  split(t, N, C, j);
+  const int R = (int)C / nc, I = (int)C - R * nc;
   double ay = 0.0, ap = 0.0;
   for (int fy = 2 * R - 1; fy <= 2 * R + 1; ++fy) {
     if (fy < 0 || fy > nf) continue;
@@ -304,6 +432,11 @@ __global__ void bnd_restrict_kernel(int nf, int N, Vec3c<double> rf, Vec3<double
   }
   cc.y[(size_t)C * N + j] = ay;
   cc.p[(size_t)C * N + j] = ap;
+  if (zx.y) {
+    zx.y[(size_t)C * N + j] = 0.0;
+    zx.p[(size_t)C * N + j] = 0.0;
+    if (j == 0 && R == 0) zx.u[I] = 0.0;
+  }
   if (j == 0 && R == 0) {
     double au = 0.0;
     for (int fx = 2 * I; fx <= 2 * I + 2; ++fx) au = fma(px(fx, I), rf.u[fx], au);
@@ -313,13 +446,15 @@ __global__ void bnd_restrict_kernel(int nf, int N, Vec3c<double> rf, Vec3<double
 
 // x_f += P e_c, one thread per (fine node, sample); u by P_x.
 __global__ void bnd_prolong_kernel(int nf, int N, Vec3c<double> ec, Vec3<double> xf) {
+  pdl_enter();
   const int nc = (nf - 1) / 2;
   const size_t fnodes = (size_t)(nf + 1) * nf;
   const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (long)fnodes * N) return;
-  const int j = (int)(t % N);
-  const long F = t / N;
-  const int fy = (int)(F / nf), fx = (int)(F % nf);
+  long F;
+  int j;
+  split(t, N, F, j);
+  const int fy = (int)F / nf, fx = (int)F - fy * nf;
   const int R0 = fy / 2, R1 = (fy + 1) / 2;   // the coarse rows (equal when fy is even)
   const int I0 = (fx - 1) / 2, I1 = fx / 2;    // the coarse columns (equal when fx is odd)
   double vy = 0.0, vp = 0.0;
@@ -594,19 +729,121 @@ __global__ void bnd_coarse_solve_kernel(int n, int N, const double* __restrict__
   }
 }
 
-// Sum of squares with the state block weighted by wy^2, fixed-order per block.
-__global__ void bnd_sumsq_kernel(const double* __restrict__ a, size_t n, double w2, double* __restrict__ partial) {
+// The same elimination for m <= 12 by a cluster of eight CTAs, each with an eighth
+// of the samples, its inverses and vectors in shared memory; the partial
+// control sums are added over the cluster in rank order.  One CTA on vectors
+// in memory took 70 us at N = 125.
+constexpr int kBndClusterM = 12;
+__global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(kBT)
+    bnd_coarse_cluster_kernel(int n, int N, const double* __restrict__ Ainv, const double* __restrict__ m9,
+                              const double* __restrict__ Zinv, St3 b3, Vec3c<double> f, Vec3<double> x) {
+  namespace cg = cooperative_groups;
+  const cg::cluster_group cl = cg::this_cluster();
+  extern __shared__ __align__(16) double sm[];
+  __shared__ double Mm[kBndClusterM * kBndClusterM], part[4], rhs[4], us[4], bu[4];
+  const int m = (n + 1) * n, mm = m * m, per = (N + 7) / 8, tid = threadIdx.x, lane = tid & 31;
+  const int j0 = min(N, (int)cl.block_rank() * per), cnt = min(N, j0 + per) - j0, nm = cnt * m;
+  double *A = sm, *w = A + (size_t)per * mm, *z = w + per * m, *t = z + per * m, *q = t + per * m;
+  for (int i = tid; i < cnt * mm; i += kBT) A[i] = Ainv[(size_t)j0 * mm + i];
+  for (int i = tid; i < mm; i += kBT) {   // dense M / N
+    const int r = i / m, c = i - r * m, dy = c / n - r / n, dx = c % n - r % n;
+    Mm[i] = dy >= -1 && dy <= 1 && dx >= -1 && dx <= 1 ? m9[(size_t)((dy + 1) * 3 + dx + 1) * m + r] / N : 0.0;
+  }
+  pdl_enter();   // the factors are written at creation only
+  for (int i = tid; i < nm; i += kBT) {   // f.y, f.p are [node r][sample j]
+    const int r = i / cnt, k = i - r * cnt;
+    t[k * m + r] = f.y[(size_t)r * N + j0 + k];
+    q[k * m + r] = f.p[(size_t)r * N + j0 + k];
+  }
+  const auto product = [&](const double* mat, const double* v) {
+    double s = 0.0;
+    for (int k = 0; k < m; ++k) s = fma(mat[k], v[k], s);
+    return s;
+  };
+  __syncthreads();
+  for (int i = tid; i < nm; i += kBT) {
+    const int k = i / m, r = i - k * m;
+    w[i] = product(A + (size_t)k * mm + r * m, t + k * m);   // A^{-1} f_y
+    z[i] = product(A + (size_t)k * mm + r * m, q + k * m);   // A^{-1} f_p
+  }
+  __syncthreads();
+  for (int i = tid; i < nm; i += kBT) t[i] = product(Mm + (i % m) * m, z + (i / m) * m);
+  __syncthreads();
+  for (int i = tid; i < nm; i += kBT) {   // w - A^{-1} (M/N) z
+    const int k = i / m, r = i - k * m;
+    q[i] = w[i] - product(A + (size_t)k * mm + r * m, t + k * m);
+  }
+  __syncthreads();
+  for (int r = tid >> 5; r < n; r += kBT / 32) {   // sums over this CTA's samples at the row-0 nodes
+    double s = 0.0;
+    for (int k = lane; k < cnt; k += 32) s += q[k * m + r];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) part[r] = s;
+  }
+  cl.sync();
+  if (tid < n) {
+    double s = 0.0;
+    for (int b = 0; b < 8; ++b) s += cl.map_shared_rank(part, b)[tid];
+    us[tid] = s;
+  }
+  cl.sync();   // nobody leaves while its sums are read
+  if (tid < n) {   // rhs = f_u + B^T sum_j q_j
+    double s = f.u[tid];
+    for (int d = -1; d <= 1; ++d)
+      if (tid + d >= 0 && tid + d < n) s += b3.w[1 - d] * us[tid + d];   // (B^T)_{k, ix} = B_{ix, k}
+    rhs[tid] = s;
+  }
+  __syncthreads();
+  if (tid < n) {
+    double s = 0.0;
+    for (int c = 0; c < n; ++c) s += Zinv[tid * n + c] * rhs[c];
+    us[tid] = s;
+    if (cl.block_rank() == 0) x.u[tid] = s;
+  }
+  __syncthreads();
+  if (tid < n) {   // B u, on row 0
+    double s = 0.0;
+    for (int d = -1; d <= 1; ++d)
+      if (tid + d >= 0 && tid + d < n) s += b3.w[d + 1] * us[tid + d];
+    bu[tid] = s;
+  }
+  __syncthreads();
+  for (int i = tid; i < nm; i += kBT) {   // y = z + A^{-1} B u
+    const int k = i / m, r = i - k * m;
+    double s = 0.0;
+    for (int ix = 0; ix < n; ++ix) s += A[(size_t)k * mm + r * m + ix] * bu[ix];
+    t[i] = z[i] + s;
+    x.y[(size_t)r * N + j0 + k] = t[i];
+  }
+  __syncthreads();
+  for (int i = tid; i < nm; i += kBT) q[i] = product(Mm + (i % m) * m, t + (i / m) * m);
+  __syncthreads();
+  for (int i = tid; i < nm; i += kBT) {   // p = w - A^{-1} (M/N) y
+    const int k = i / m, r = i - k * m;
+    x.p[(size_t)r * N + j0 + k] = w[i] - product(A + (size_t)k * mm + r * m, q + k * m);
+  }
+}
+
+// Per-CTA parts of wy2 ||y||^2 + ||u||^2 + ||p||^2, fixed order.
+__global__ void __launch_bounds__(kBT) bnd_sumsq_kernel(Vec3c<double> v, size_t ny, size_t nu, double wy2,
+                                                        double* __restrict__ partial) {
+  pdl_enter();
   __shared__ double sh[kBT / 32];
-  double s = 0.0;
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-    s = fma(a[i], a[i], s);
+  double s = 0.0, sp = 0.0;
+  const size_t stride = (size_t)gridDim.x * blockDim.x, t0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  for (size_t i = t0; i < ny; i += stride) {
+    s = fma(v.y[i], v.y[i], s);
+    sp = fma(v.p[i], v.p[i], sp);
+  }
+  for (size_t i = t0; i < nu; i += stride) sp = fma(v.u[i], v.u[i], sp);
+  s = fma(s, wy2, sp);
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
   __syncthreads();
   if (threadIdx.x == 0) {
     double t = 0.0;
     for (int k = 0; k < kBT / 32; ++k) t += sh[k];
-    partial[blockIdx.x] = t * w2;
+    partial[blockIdx.x] = t;
   }
 }
 
@@ -685,7 +922,38 @@ cmg_status vec_ok3(const double* y, const double* u, const double* p) {
   return (a16(y) && a16(u) && a16(p)) ? CMG_OK : CMG_ERR_INVALID_ARG;
 }
 
+// The one-kernel residual (JAC = false) or Jacobi sweep from x into o (true);
+// cudaErrorNotSupported above 256 samples.
+template <bool JAC>
+cudaError_t node_pass(cmg_bnd* h, int l, double theta, Vec3c<double> x, Vec3c<double> f, Vec3<double> o) {
+  const BLev& v = h->lv[l];
+  const St3 g3{{v.g3[0], v.g3[1], v.g3[2]}}, b3{{v.b3[0], v.b3[1], v.b3[2]}};
+  const int need = (h->N + 31) / 32;
+  if (need > 8) return cudaErrorNotSupported;
+  const long threads = (long)v.nodes * 32;
+  const auto go = [&](auto* k) {
+    return launch_k(k, dim3(ctas_for(threads)), dim3(block_for(threads)), 0, h->stream, v.n, h->N, 1.0 / h->N,
+                    (const double*)v.a9, (const double*)v.m9, g3, b3, (const double*)v.inva, (const double*)v.isigma,
+                    theta, x, f, o);
+  };
+  cudaError_t e;
+  if (l == 0)
+    e = need <= 1   ? go(bnd_node_kernel<1, true, JAC>)
+        : need <= 2 ? go(bnd_node_kernel<2, true, JAC>)
+        : need <= 4 ? go(bnd_node_kernel<4, true, JAC>)
+                    : go(bnd_node_kernel<8, true, JAC>);
+  else
+    e = need <= 1   ? go(bnd_node_kernel<1, false, JAC>)
+        : need <= 2 ? go(bnd_node_kernel<2, false, JAC>)
+        : need <= 4 ? go(bnd_node_kernel<4, false, JAC>)
+                    : go(bnd_node_kernel<8, false, JAC>);
+  count_launches(1);
+  return e;
+}
+
 cudaError_t residual(cmg_bnd* h, int l, Vec3c<double> x, Vec3c<double> f, Vec3<double> r) {
+  const cudaError_t e = node_pass<false>(h, l, 0.0, x, f, r);
+  if (e != cudaErrorNotSupported) return e;
   const BLev& v = h->lv[l];
   const int N = h->N;
   St3 g3{{v.g3[0], v.g3[1], v.g3[2]}}, b3{{v.b3[0], v.b3[1], v.b3[2]}};
@@ -699,6 +967,12 @@ cudaError_t residual(cmg_bnd* h, int l, Vec3c<double> x, Vec3c<double> f, Vec3<d
 cudaError_t smooth(cmg_bnd* h, int l, double theta, int sweeps, Vec3<double> x, Vec3c<double> f) {
   BLev& v = h->lv[l];
   const Vec3<double> r = vx(v, v.r);
+  // pairs of sweeps through the residual vector; an odd one in place
+  for (; sweeps >= 2 && h->N <= 256; sweeps -= 2) {
+    cudaError_t e = node_pass<true>(h, l, theta, cview(x), f, r);
+    if (e == cudaSuccess) e = node_pass<true>(h, l, theta, cview(r), f, x);
+    if (e != cudaSuccess) return e;
+  }
   for (int s = 0; s < sweeps; ++s) {
     cudaError_t e = residual(h, l, cview(x), f, r);
     if (e != cudaSuccess) return e;
@@ -710,34 +984,33 @@ cudaError_t smooth(cmg_bnd* h, int l, double theta, int sweeps, Vec3<double> x, 
   return cudaSuccess;
 }
 
-cudaError_t restrict_to(cmg_bnd* h, int l, Vec3c<double> r, Vec3<double> c) {
-  const BLev& v = h->lv[l + 1];
-  bnd_restrict_kernel<<<bblocks((long)v.nodes * h->N), kBT, 0, h->stream>>>(h->lv[l].n, h->N, r, c);
+cudaError_t restrict_to(cmg_bnd* h, int l, Vec3c<double> r, Vec3<double> c,
+                        Vec3<double> zx = Vec3<double>{nullptr, nullptr, nullptr}) {
+  const long threads = (long)h->lv[l + 1].nodes * h->N;
   count_launches(1);
-  return cudaGetLastError();
+  return launch_k(bnd_restrict_kernel, dim3(ctas_for(threads)), dim3(block_for(threads)), 0, h->stream, h->lv[l].n, h->N,
+                  r, c, zx);
 }
 
 cudaError_t prolong_add(cmg_bnd* h, int l, Vec3c<double> e, Vec3<double> x) {
   const BLev& v = h->lv[l];
-  bnd_prolong_kernel<<<bblocks((long)v.nodes * h->N), kBT, 0, h->stream>>>(v.n, h->N, e, x);
+  const long threads = (long)v.nodes * h->N;
   count_launches(1);
-  return cudaGetLastError();
+  return launch_k(bnd_prolong_kernel, dim3(ctas_for(threads)), dim3(block_for(threads)), 0, h->stream, v.n, h->N, e, x);
 }
 
 cudaError_t coarse_solve(cmg_bnd* h, Vec3c<double> f, Vec3<double> x) {
   const BLev& v = h->lv[h->L - 1];
   St3 b3{{v.b3[0], v.b3[1], v.b3[2]}};
+  if (v.nodes <= kBndClusterM) {
+    const size_t per = (size_t)(h->N + 7) / 8, smem = per * (v.nodes * v.nodes + 4 * v.nodes) * sizeof(double);
+    count_launches(1);
+    return launch_k(bnd_coarse_cluster_kernel, dim3(8), dim3(kBT), smem, h->stream, v.n, h->N, (const double*)h->Ainv,
+                    (const double*)v.m9, (const double*)h->Zinv, b3, f, x);
+  }
   bnd_coarse_solve_kernel<<<1, kBT, 0, h->stream>>>(v.n, h->N, h->Ainv, v.m9, h->Zinv, b3, f, x, h->work);
   count_launches(1);
   return cudaGetLastError();
-}
-
-cudaError_t zero3(cmg_bnd* h, int l, Vec3<double> x) {
-  const BLev& v = h->lv[l];
-  cudaError_t e = cudaMemsetAsync(x.y, 0, v.nodes * h->N * sizeof(double), h->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(x.u, 0, v.n * sizeof(double), h->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(x.p, 0, v.nodes * h->N * sizeof(double), h->stream);
-  return e;
 }
 
 // Algorithm 1 on grid l (gamma = 1: V-cycle, 2: W-cycle) with damped
@@ -749,8 +1022,9 @@ cudaError_t cycle(cmg_bnd* h, int l, double theta, int n1, int n2, int gamma, Ve
   cudaError_t e = smooth(h, l, theta, n1, x, f);
   const Vec3<double> r = vx(v, v.r), fc = vx(c, c.f), xc = vx(c, c.x);
   if (e == cudaSuccess) e = residual(h, l, cview(x), f, r);
-  if (e == cudaSuccess) e = restrict_to(h, l, cview(r), fc);
-  if (e == cudaSuccess) e = zero3(h, l + 1, xc);
+  // the coarse iterate starts from zero (the direct solve does not read it)
+  if (e == cudaSuccess)
+    e = restrict_to(h, l, cview(r), fc, l + 2 < h->L ? xc : Vec3<double>{nullptr, nullptr, nullptr});
   for (int g = 0; g < gamma && e == cudaSuccess; ++g) e = cycle(h, l + 1, theta, n1, n2, gamma, xc, cview(fc));
   if (e == cudaSuccess) e = prolong_add(h, l, cview(xc), x);
   if (e == cudaSuccess) e = smooth(h, l, theta, n2, x, f);
@@ -763,15 +1037,12 @@ cmg_status paper_norm(cmg_bnd* h, Vec3c<double> v, double* out) {
   const BLev& l0 = h->lv[0];
   const size_t ny = l0.nodes * h->N;
   const double wy2 = (double)h->N * h->N;
-  bnd_sumsq_kernel<<<kNormBlocks, kBT, 0, h->stream>>>(v.y, ny, wy2, h->part);
-  bnd_sumsq_kernel<<<kNormBlocks, kBT, 0, h->stream>>>(v.u, (size_t)l0.n, 1.0, h->part + kNormBlocks);
-  bnd_sumsq_kernel<<<kNormBlocks, kBT, 0, h->stream>>>(v.p, ny, 1.0, h->part + 2 * kNormBlocks);
-  count_launches(3);
-  BK(cudaGetLastError());
-  BK(cudaMemcpyAsync(h->hpart, h->part, 3 * kNormBlocks * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+  BK(launch_k(bnd_sumsq_kernel, dim3(kNormBlocks), dim3(kBT), 0, h->stream, v, ny, (size_t)l0.n, wy2, h->part));
+  count_launches(1);
+  BK(cudaMemcpyAsync(h->hpart, h->part, kNormBlocks * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   BK(cudaStreamSynchronize(h->stream));
   double s = 0.0;
-  for (int k = 0; k < 3 * kNormBlocks; ++k) s += h->hpart[k];
+  for (int k = 0; k < kNormBlocks; ++k) s += h->hpart[k];
   *out = std::sqrt(s);
   return CMG_OK;
 }
@@ -840,8 +1111,8 @@ cmg_status cmg_bnd_create(int n, int N, int K, double nu, double amp, int coarse
   if (e == cudaSuccess) e = balloc(h, &h->Ainv, (size_t)N * m * m);
   if (e == cudaSuccess) e = balloc(h, &h->Zinv, (size_t)cl.n * cl.n);
   if (e == cudaSuccess) e = balloc(h, &h->work, (size_t)4 * N * m);
-  if (e == cudaSuccess) e = balloc(h, &h->part, 3 * kNormBlocks);
-  if (e == cudaSuccess) e = cudaMallocHost(&h->hpart, 3 * kNormBlocks * sizeof(double));
+  if (e == cudaSuccess) e = balloc(h, &h->part, kNormBlocks);
+  if (e == cudaSuccess) e = cudaMallocHost(&h->hpart, kNormBlocks * sizeof(double));
   if (e != cudaSuccess) return fin(e);
   if (K > 0) e = cudaMemcpy(h->xi, xi_host, (size_t)N * K * sizeof(double), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) return fin(e);
@@ -879,6 +1150,8 @@ cmg_status cmg_bnd_create(int n, int N, int K, double nu, double amp, int coarse
   e = cudaFuncSetAttribute(bnd_coarse_inv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(bnd_coarse_schur_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(bnd_coarse_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
   if (e != cudaSuccess) return fin(e);
   bnd_coarse_inv_kernel<<<N, kBT, inv_smem, h->stream>>>(cl.n, N, cl.a9, h->Ainv);
   St3 g3{{cl.g3[0], cl.g3[1], cl.g3[2]}}, b3{{cl.b3[0], cl.b3[1], cl.b3[2]}};

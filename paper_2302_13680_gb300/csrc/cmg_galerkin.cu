@@ -194,17 +194,22 @@ __global__ void residual9_yp_kernel(int n, int N, const T* __restrict__ a9, cons
   if (t >= (long)nodes * N) return;
   const int i = (int)(t / N), j = (int)(t - (long)i * N);
   const int iy = i / n, ix = i - iy * n;
-  T Ap = 0, Ay = 0, My = 0;
+  T Ap = 0, Ay = 0, My = 0, av[9], yv[9], pv[9];
+  bool ok[9];
+  int nb[9];
+  nine_neighbours(n, iy, ix, ok, nb);
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
-    const int ny = iy + k / 3 - 1, nx = ix + k % 3 - 1;
-    if (ny < 0 || ny >= n || nx < 0 || nx >= n) continue;
-    const size_t nb = (size_t)ny * n + nx;
-    const T a = a9[((size_t)k * nodes + i) * N + j];
-    const T yv = x.y[nb * N + j], pv = x.p[nb * N + j];
-    Ap = fma(a, pv, Ap);
-    Ay = fma(a, yv, Ay);
-    My = fma(M.w[k], yv, My);
+    av[k] = a9[((size_t)k * nodes + i) * N + j];
+    yv[k] = x.y[(size_t)nb[k] * N + j];
+    pv[k] = x.p[(size_t)nb[k] * N + j];
+  }
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    const T a = ok[k] ? av[k] : T(0), yk = ok[k] ? yv[k] : T(0), pk = ok[k] ? pv[k] : T(0);
+    Ap = fma(a, pk, Ap);
+    Ay = fma(a, yk, Ay);
+    My = fma(M.w[k], yk, My);
   }
   const T sy = M.c * My + Ap, sp = Ay + M.e * (T)mu[i];
   const size_t o = (size_t)i * N + j;
@@ -262,17 +267,20 @@ __global__ void residual9_kernel(int n, int N, const T* __restrict__ a9, const _
   T pm = 0;   // this lane's share of sum_j (M p_j)_i
 #pragma unroll 1
   for (int j = lane; j < N; j += 32) {
-    T Ap = 0, Ay = 0, My = 0, Mp = 0;
+    T Ap = 0, Ay = 0, My = 0, Mp = 0, av[9], yv[9], pv[9];   // loads in flight together, as in the colour kernel
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
-      if (!ok[k]) continue;
-      const T a = a9[((size_t)k * nodes + i) * N + j];
-      const T yv = x.y[(size_t)nb[k] * N + j], pv = x.p[(size_t)nb[k] * N + j];
-      const T m = mt.w[k];
-      Ap = fma(a, pv, Ap);
-      Ay = fma(a, yv, Ay);
-      My = fma(m, yv, My);
-      Mp = fma(m, pv, Mp);
+      av[k] = a9[((size_t)k * nodes + i) * N + j];
+      yv[k] = x.y[(size_t)nb[k] * N + j];
+      pv[k] = x.p[(size_t)nb[k] * N + j];
+    }
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      const T m = mt.w[k], a = ok[k] ? av[k] : T(0), yk = ok[k] ? yv[k] : T(0), pk = ok[k] ? pv[k] : T(0);
+      Ap = fma(a, pk, Ap);
+      Ay = fma(a, yk, Ay);
+      My = fma(m, yk, My);
+      Mp = fma(m, pk, Mp);
     }
     const T sy = cT * My + Ap, sp = Ay + eMu;
     const size_t o = (size_t)i * N + j;
@@ -427,15 +435,23 @@ __global__ void __launch_bounds__(kGBlock) gs4_colour_reg_kernel(int n, int N, i
     By[q] = Bp[q] = ia[q] = 0;
     if (valid && j < N) {
       T by = f.y[i * N + j], bp = f.p[i * N + j] - eMu, mp = 0;
+      // all loads of a sample in flight together, masked afterwards (nb falls back to the node itself); a
+      // branch per neighbour made them a chain of nine
+      T av[9], yv[9], pv[9];
 #pragma unroll
       for (int k = 0; k < 9; ++k) {
-        if (!ok[k]) continue;
-        const T a = a9[((size_t)k * nodes + i) * N + j];
-        const T yv = x.y[(size_t)nb[k] * N + j], pv = x.p[(size_t)nb[k] * N + j];
-        const T m = mt.w[k];
-        by -= cT * m * yv + a * pv;
-        bp -= a * yv;
-        mp = fma(m, pv, mp);
+        if (k == 4) continue;
+        av[k] = a9[((size_t)k * nodes + i) * N + j];
+        yv[k] = x.y[(size_t)nb[k] * N + j];
+        pv[k] = x.p[(size_t)nb[k] * N + j];
+      }
+#pragma unroll
+      for (int k = 0; k < 9; ++k) {
+        if (k == 4) continue;
+        const T m = mt.w[k], a = ok[k] ? av[k] : T(0), yk = ok[k] ? yv[k] : T(0), pk = ok[k] ? pv[k] : T(0);
+        by -= cT * m * yk + a * pk;
+        bp -= a * yk;
+        mp = fma(m, pk, mp);
       }
       const T iq = inva[i * N + j];
       tacc += (cd * iq) * (iq * bp) - iq * by;

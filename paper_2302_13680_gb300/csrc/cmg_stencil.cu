@@ -396,7 +396,10 @@ cudaError_t launch_prolong_add(int nf, int N, Vec3c<T> e, Vec3<T> x, cudaStream_
 int launch_residual_cast(const LevelView<double>& L, Vec3c<double> x, Vec3c<double> f, Vec3<float> r, double s,
                          const double* sdev, double wy, double* partial, int max_partials, cudaStream_t st,
                          const double* gate) {
-  const SampleMap m = choose_map(L.N, 8, (long)L.n * L.n);
+  // four chunks per lane where two 256-thread CTAs per SM remain: here they hide
+  // the loads better than twice the warps (n = 255, N = 64: 166 against 186 us)
+  const long nodes = (long)L.n * L.n, chunks = L.N % 2 == 0 ? L.N / 2 : L.N;
+  const SampleMap m = choose_map(L.N, 8, nodes, chunks >= 4 && nodes * chunks >= 4 * 2L * 152 * 256 ? 4 : 0);
   const unsigned grid = grid_for((long)L.n * L.n, m.lpn);
   if ((int)grid > max_partials) return -1;
   const float wy2 = (float)(wy * wy);
