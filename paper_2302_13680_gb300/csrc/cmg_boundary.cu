@@ -249,12 +249,13 @@ __global__ void bnd_residual_u_kernel(int n, St3 g3, St3 b3, const double* __res
   r.u[k] = f.y ? f.u[k] - su : su;
 }
 
-// One warp per node, lanes over samples (j = lane + 32 q, q < R, N <= 32 R):
+// One thread per (node, sample), N <= 256: a node's W = ceil(N / 32) warps are a CTA (four nodes to a CTA
+// for W = 1).
 // JAC = false: the residual rows above (o = f - S x, or S x when f is null);
 // JAC = true: a whole damped collective Jacobi sweep, Eq. (11), from x into o,
 // o_i = x_i + theta S~_i^{-1} (f - S x)_i, with no residual written and read
 // back.  On Gamma the control row's sum over samples of B^T p comes from the
-// p values the state rows load, in one warp sum with Eq. (13)'s.  FIVE (the
+// p values the state rows load, in one sum with Eq. (13)'s.  FIVE (the
 // finest grid): A_j has five entries and the mass is lumped, so the four
 // corner planes and eight of the mass's are zero and not touched.
 //
@@ -263,17 +264,21 @@ __global__ void bnd_residual_u_kernel(int n, St3 g3, St3 b3, const double* __res
 // FP64 division by N per node-sample: 69 us on the finest grid at n = 63, N =
 // 125 and 31 us on the grids of a few hundred nodes, where it was the launches' and the
 // dependent loads' latency (the nine neighbours were loaded one branch at a time;
-// here all of a chunk's loads are in flight together, masked afterwards).
-template <int R, bool FIVE, bool JAC>
+// here all loads are in flight together, masked afterwards, and a node's samples go over several warps: a
+// warp per node took 39 us on that finest grid and 21 us on the small ones).
+template <bool FIVE, bool JAC>
 __global__ void __launch_bounds__(kBT)
     bnd_node_kernel(int n, int N, double rN, const double* __restrict__ a9, const double* __restrict__ m9, St3 g3, St3 b3,
                     const double* __restrict__ inva, const double* __restrict__ isigma, double theta, Vec3c<double> x,
                     Vec3c<double> f, Vec3<double> o) {
   pdl_enter();
+  __shared__ double part[kBT / 32];
   const size_t nodes = (size_t)(n + 1) * n;
-  const long i = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (i >= (long)nodes) return;   // whole warp
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool one = N <= 32;   // a warp per node
+  const long i = one ? (long)blockIdx.x * (blockDim.x >> 5) + warp : (long)blockIdx.x;
+  if (i >= (long)nodes) return;   // whole warp (one) or none
+  const int j = one ? lane : (int)threadIdx.x, jj = j < N ? j : 0;
   const int ry = (int)i / n, rx = (int)i - ry * n;
   const bool gam = ry == 0, apply = f.y == nullptr;
   bool ok[9];
@@ -300,69 +305,61 @@ __global__ void __launch_bounds__(kBT)
     if (JAC) isg = isigma[rx];
   }
   const double c = mk[4] * rN, db = -b3.w[1];   // Eq. (12) at the node: c_j = M_ii / N, d = e = -B_ii
-  double sy[R], sp[R], ia[R], yc[R], pc[R], s = 0.0;
+  double av[9], yv[9], pv[9];
 #pragma unroll
-  for (int q = 0; q < R; ++q) {
-    const int j = lane + 32 * q;
-    const bool in = j < N;
-    const int jj = in ? j : 0;
-    double av[9], yv[9], pv[9];
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-      if (FIVE && !(k & 1) && k != 4) continue;
-      av[k] = a9[((size_t)k * nodes + i) * N + jj];
-      yv[k] = x.y[g[k] * N + jj];
-      pv[k] = x.p[g[k] * N + jj];
-    }
-    const size_t e = (size_t)i * N + jj;
-    const double fy = apply ? 0.0 : f.y[e], fp = apply ? 0.0 : f.p[e];
-    ia[q] = JAC ? inva[e] : 0.0;
-    double Ap = 0.0, Ay = 0.0, My = 0.0;
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-      if (FIVE && !(k & 1) && k != 4) continue;
-      const double a = ok[k] ? av[k] : 0.0, yk = ok[k] ? yv[k] : 0.0, pk = ok[k] ? pv[k] : 0.0;
-      Ap = fma(a, pk, Ap);
-      Ay = fma(a, yk, Ay);
-      if (!FIVE || k == 4) My = fma(mk[k], yk, My);
-    }
-    const double ty = fma(My, rN, Ap), tp = Ay - Bu;
-    sy[q] = apply ? ty : fy - ty;
-    sp[q] = apply ? tp : fp - tp;
-    yc[q] = yv[4];
-    pc[q] = pv[4];
-    if (gam && in) {
-      // (B^T)_{k, k+d} = B_{k+d, k} on the row's nodes (planes 3, 4, 5)
-      double Bp = b3.w[1] * pv[4];
-      if (ok[3]) Bp = fma(b3.w[2], pv[3], Bp);
-      if (ok[5]) Bp = fma(b3.w[0], pv[5], Bp);
-      s += JAC ? Bp + db * ((c * ia[q]) * (ia[q] * sp[q]) - ia[q] * sy[q]) : Bp;
-    }
+  for (int k = 0; k < 9; ++k) {
+    if (FIVE && !(k & 1) && k != 4) continue;
+    av[k] = a9[((size_t)k * nodes + i) * N + jj];
+    yv[k] = x.y[g[k] * N + jj];
+    pv[k] = x.p[g[k] * N + jj];
   }
+  const size_t e = (size_t)i * N + jj;
+  const double fy = apply ? 0.0 : f.y[e], fp = apply ? 0.0 : f.p[e], ia = JAC ? inva[e] : 0.0;
+  double Ap = 0.0, Ay = 0.0, My = 0.0;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    if (FIVE && !(k & 1) && k != 4) continue;
+    const double a = ok[k] ? av[k] : 0.0, yk = ok[k] ? yv[k] : 0.0, pk = ok[k] ? pv[k] : 0.0;
+    Ap = fma(a, pk, Ap);
+    Ay = fma(a, yk, Ay);
+    if (!FIVE || k == 4) My = fma(mk[k], yk, My);
+  }
+  const double ty = fma(My, rN, Ap), tp = Ay - Bu;
+  const double sy = apply ? ty : fy - ty, sp = apply ? tp : fp - tp;
   double du = 0.0;
-  if (gam) {   // uniform over the warp
+  if (gam) {   // uniform over the node's threads
+    // (B^T)_{k, k+d} = B_{k+d, k} on the row's nodes (planes 3, 4, 5)
+    double s = 0.0;
+    if (j < N) {
+      s = b3.w[1] * pv[4];
+      if (ok[3]) s = fma(b3.w[2], pv[3], s);
+      if (ok[5]) s = fma(b3.w[0], pv[5], s);
+      if (JAC) s += db * ((c * ia) * (ia * sp) - ia * sy);
+    }
     for (int w = 16; w > 0; w >>= 1) s += __shfl_xor_sync(0xffffffffu, s, w);
+    if (!one) {
+      if (lane == 0) part[warp] = s;
+      __syncthreads();
+      s = 0.0;
+      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += part[w];
+    }
+    const bool first = one ? lane == 0 : threadIdx.x == 0;
     if (JAC) {
       du = ((fu - Gu) + s) * isg;
-      if (lane == 0) o.u[rx] = xu + theta * du;
-    } else if (lane == 0) {
+      if (first) o.u[rx] = xu + theta * du;
+    } else if (first) {
       o.u[rx] = apply ? Gu - s : fu - (Gu - s);
     }
   }
-#pragma unroll
-  for (int q = 0; q < R; ++q) {
-    const int j = lane + 32 * q;
-    if (j >= N) continue;
-    const size_t e = (size_t)i * N + j;
-    if (JAC) {
-      const double dy = ia[q] * (sp[q] - db * du);
-      const double dp = ia[q] * (sy[q] - c * dy);
-      o.y[e] = yc[q] + theta * dy;
-      o.p[e] = pc[q] + theta * dp;
-    } else {
-      o.y[e] = sy[q];
-      o.p[e] = sp[q];
-    }
+  if (j >= N) return;
+  if (JAC) {
+    const double dy = ia * (sp - db * du);
+    const double dp = ia * (sy - c * dy);
+    o.y[e] = yv[4] + theta * dy;
+    o.p[e] = pv[4] + theta * dp;
+  } else {
+    o.y[e] = sy;
+    o.p[e] = sp;
   }
 }
 
@@ -930,23 +927,13 @@ cudaError_t node_pass(cmg_bnd* h, int l, double theta, Vec3c<double> x, Vec3c<do
   const St3 g3{{v.g3[0], v.g3[1], v.g3[2]}}, b3{{v.b3[0], v.b3[1], v.b3[2]}};
   const int need = (h->N + 31) / 32;
   if (need > 8) return cudaErrorNotSupported;
-  const long threads = (long)v.nodes * 32;
+  const unsigned cta = need == 1 ? 128 : 32 * need;
+  const unsigned grid = (unsigned)(need == 1 ? (v.nodes + 3) / 4 : v.nodes);
   const auto go = [&](auto* k) {
-    return launch_k(k, dim3(ctas_for(threads)), dim3(block_for(threads)), 0, h->stream, v.n, h->N, 1.0 / h->N,
-                    (const double*)v.a9, (const double*)v.m9, g3, b3, (const double*)v.inva, (const double*)v.isigma,
-                    theta, x, f, o);
+    return launch_k(k, dim3(grid), dim3(cta), 0, h->stream, v.n, h->N, 1.0 / h->N, (const double*)v.a9,
+                    (const double*)v.m9, g3, b3, (const double*)v.inva, (const double*)v.isigma, theta, x, f, o);
   };
-  cudaError_t e;
-  if (l == 0)
-    e = need <= 1   ? go(bnd_node_kernel<1, true, JAC>)
-        : need <= 2 ? go(bnd_node_kernel<2, true, JAC>)
-        : need <= 4 ? go(bnd_node_kernel<4, true, JAC>)
-                    : go(bnd_node_kernel<8, true, JAC>);
-  else
-    e = need <= 1   ? go(bnd_node_kernel<1, false, JAC>)
-        : need <= 2 ? go(bnd_node_kernel<2, false, JAC>)
-        : need <= 4 ? go(bnd_node_kernel<4, false, JAC>)
-                    : go(bnd_node_kernel<8, false, JAC>);
+  const cudaError_t e = l == 0 ? go(bnd_node_kernel<true, JAC>) : go(bnd_node_kernel<false, JAC>);
   count_launches(1);
   return e;
 }
