@@ -686,11 +686,8 @@ cmg_status check_cycle(cmg_handle* h, const cmg_cycle* o) {
 cudaError_t sumsq3(cmg_handle* h, int l, const double* y, const double* u, const double* p, double* out,
                    double wy2 = 1.0) {
   const size_t nodes = h->lv[l].nodes, N = (size_t)h->prob.N;
-  cudaError_t e = launch_sumsq(y, nodes * N, h->red, 0, wy2, h->stream);
-  if (e == cudaSuccess) e = launch_sumsq(u, nodes, h->red, 1, 1.0, h->stream);
-  if (e == cudaSuccess) e = launch_sumsq(p, nodes * N, h->red, 1, 1.0, h->stream);
-  if (e == cudaSuccess) e = launch_finish_sum(h->red, kRedBlocks, out, h->stream);
-  return e;
+  const int cnt = launch_sumsq3(y, u, p, nodes * N, nodes, wy2, h->red, h->stream);
+  return cnt < 0 ? cudaErrorLaunchFailure : launch_finish_sum(h->red, cnt, out, h->stream);
 }
 
 cudaError_t fetch(cmg_handle* h, const double* dev, int count) {
@@ -820,8 +817,7 @@ cmg_status cmg_create(const cmg_problem* prob, const double* xi_host, void* stre
       AL(h->lv[l].a9f, 9 * h->lv[l].nodes * N);
       AL(h->lv[l].invaf, h->lv[l].nodes * N);
     }
-  const size_t g = (size_t)P.n + 2;
-  AL(h->kap, g * g * N + g * N);
+  AL(h->kap, field_scratch(P.n, P.N));
   AL(h->xi, (size_t)N * (P.K > 0 ? P.K : 1));
   AL(h->red, (size_t)kRedBlocks * 8 * 16);
   AL(h->dsc, 1024);

@@ -36,6 +36,20 @@ __device__ __forceinline__ vec<T, V> ldv_if(bool ok, const T* p) {
   return ok ? ldv<T, V>(p) : vzero<T, V>();
 }
 
+// (float)v, round to nearest even, on the integer pipe: the conversion
+// instruction is one of the FP64 pipe's, which has two lanes per clock and SM.
+// Values outside the normal FP32 range take the instruction.
+__device__ __forceinline__ float narrow_rn(double v) {
+  const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+  const unsigned mag = hi & 0x7fffffffu;
+  if (mag - 0x38100000u >= 0x0fd00000u && (mag | lo) != 0u) return (float)v;   // below 2^-126 or from 2^127 on
+  // drop 29 bits: add half a unit (less one when the last kept bit is even), then shift
+  const unsigned l2 = lo + 0x0fffffffu + ((lo >> 29) & 1u);
+  const unsigned h2 = mag + (l2 < lo ? 1u : 0u);
+  const unsigned f = (h2 << 3 | l2 >> 29) - (896u << 23);
+  return __uint_as_float((mag | lo) != 0u ? (f | (hi & 0x80000000u)) : (hi & 0x80000000u));
+}
+
 // Programmatic dependent launch: a kernel launched with launch_k may start
 // while its predecessor in the stream drains; it waits here, before touching
 // any memory, until the predecessor has completed and its writes are

@@ -432,8 +432,9 @@ cudaError_t launch_coarse_setup(const CoarseData& C, const double* kx, const dou
                                 double c, double G, double d, double e, cudaStream_t s);
 
 // ---- coefficients (cmg_setup.cu) ----
-// Nodal field on the (n+2)^2 grid including boundary points, then faces,
-// 1/diag and Schur denominators.  kap: scratch [(n+2)^2][N] doubles.
+// Nodal field (1 / kappa) on the (n+2)^2 grid including boundary points, then
+// faces, 1/diag and Schur denominators.  kap: scratch of field_scratch doubles.
+size_t field_scratch(int n, int N);
 // a[node][j] = sum of the node's four faces (FP64).
 cudaError_t launch_diag_sum(int n, int N, const double* kx, const double* ky, double* a, cudaStream_t s);
 cudaError_t launch_level_setup(int n, int N, int K, double amp, const double* xi, double* kap,
@@ -465,9 +466,13 @@ cudaError_t launch_diag32(int n, int N, const float* kx32, const float* ky32, in
                           double* isigma_d, double dce, double G, cudaStream_t s, const float* dw = nullptr);
 
 // ---- vector kernels (cmg_blas.cu) ----
-constexpr int kRedBlocks = 304;    // fixed partial count: deterministic reductions
+constexpr int kRedBlocks = 608;    // fixed partial count: deterministic reductions
 // partial[0..kRedBlocks) (+)= w2 * per-block sums of squares; call finish to combine.
 cudaError_t launch_sumsq(const double* a, size_t n, double* partial, int accumulate, double w2, cudaStream_t s);
+// partials of wy2 ||y||^2 + ||u||^2 + ||p||^2 (ny entries in y and p, nu in u;
+// 16-byte aligned) in one launch; returns their count (<= kRedBlocks * 2) or -1.
+int launch_sumsq3(const double* y, const double* u, const double* p, size_t ny, size_t nu, double wy2,
+                  double* partial, cudaStream_t s);
 cudaError_t launch_finish_sum(const double* partial, int count, double* out, cudaStream_t s);
 // out[i] = sum_k V_i[k] w[k], i < nv; V_i = V + i*stride.  partial: [nv][kRedBlocks]
 cudaError_t launch_mdot(const double* V, size_t stride, int nv, const double* w, size_t n,

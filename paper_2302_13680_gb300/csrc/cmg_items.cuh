@@ -577,16 +577,21 @@ __device__ __forceinline__ float residual_cast_item(const LevelView<double>& L, 
             sq = fmaf(rp.v[k], rp.v[k], sq);
           }
         } else {
-          vec<T, V> offy = vzero<T, V>(), offp = vzero<T, V>();
-          fma_faces<T, V>(offy, kW, yW, kE, yE, kS, yS, kN, yN);
-          fma_faces<T, V>(offp, kW, pW, kE, pE, kS, pS, kN, pN);
+          // 13 FP64 instructions per node-sample: one chain per row from its right side on, and the rounding to FP32 on
+          // the integer pipe (17 with separate sums of the neighbours and converting instructions)
+          vec<T, V> qy, qp;
 #pragma unroll
           for (int k = 0; k < V; ++k) {
             const T a = av.v[k];
-            const T ryk = fy.v[k] - fma(c, y.v[k], fma(a, p.v[k], -offp.v[k]));   // f_y - c y - A p
-            const T rpk = (fp.v[k] - eu) - fma(a, y.v[k], -offy.v[k]);             // f_p - e u - A y
-            ry.v[k] = (float)ryk * sf;   // scaled after rounding: FP32 multiplies instead of FP64
-            rp.v[k] = (float)rpk * sf;
+            qy.v[k] = fma(-a, p.v[k], fma(-c, y.v[k], fy.v[k]));   // f_y - c y - A p
+            qp.v[k] = fma(-a, y.v[k], fp.v[k] - eu);               // f_p - e u - A y
+          }
+          fma_faces<T, V>(qy, kW, pW, kE, pE, kS, pS, kN, pN);
+          fma_faces<T, V>(qp, kW, yW, kE, yE, kS, yS, kN, yN);
+#pragma unroll
+          for (int k = 0; k < V; ++k) {
+            ry.v[k] = narrow_rn(qy.v[k]) * sf;   // scaled after rounding: FP32 multiplies instead of FP64
+            rp.v[k] = narrow_rn(qp.v[k]) * sf;
             sq = fmaf(wy2 * ry.v[k], ry.v[k], sq);
             sq = fmaf(rp.v[k], rp.v[k], sq);
             pacc += p.v[k];

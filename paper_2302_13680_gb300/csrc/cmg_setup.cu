@@ -13,10 +13,12 @@ namespace cmg {
 
 namespace {
 
-// gx[ix][j] = sum_k xi[j][k] sin(k pi x_ix) / k, x_ix = ix h, ix = 0..n+1.
-__global__ void field_x_kernel(int n, int N, int K, const double* __restrict__ xi, double* __restrict__ gx) {
+// gx[ix][j] = sum_k xi[j][k] sin(k pi x_ix) / k, x_ix = ix h, ix = 0..n+1, and
+// after it gy[iy] = amp sin(pi y_iy) (the tail of the scratch, field_scratch).
+__global__ void field_x_kernel(int n, int N, int K, double amp, const double* __restrict__ xi, double* __restrict__ gx) {
   const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (long)(n + 2) * N) return;
+  if (t < n + 2) gx[(size_t)(n + 2) * N + t] = amp * sinpi((double)t / (double)(n + 1));
   const int ix = (int)(t / N), j = (int)(t - (long)ix * N);
   const double x = (double)ix / (double)(n + 1);
   double g = 0.0;
@@ -24,23 +26,47 @@ __global__ void field_x_kernel(int n, int N, int K, const double* __restrict__ x
   gx[t] = g;
 }
 
-// kap[iy][ix][j] = exp(amp * sin(pi y_iy) * gx[ix][j]) on the (n+2)^2 grid.
+// t = i N + j, in 32 bits where it fits (a 64-bit division per thread costs more than the rest of a face).
+__device__ __forceinline__ void split(long t, int N, long& i, int& j) {
+  i = t < 0x7fffffffL ? (long)((int)t / N) : t / N;
+  j = (int)(t - i * N);
+}
+
+// rho[iy][ix][j] = 1 / kappa = exp(-amp sin(pi y_iy) gx[ix][j]) on the (n+2)^2
+// grid: a face's harmonic mean is then 2 / (rho_a + rho_b).
 // sin(pi y) is symmetric about y = 1/2 (rows iy and n+1-iy), so each
 // exponential is evaluated once for both rows (the FP64 exponential is the
 // cost of this kernel on a GPU with a narrow FP64 pipe); the boundary rows
-// have sin(pi y) = 0, kappa = 1.
-__global__ void field_kernel(int n, int N, double amp, const double* __restrict__ gx, double* __restrict__ kap) {
+// have sin(pi y) = 0, kappa = 1.  Bound by the FP64 pipe; sin(pi y) and its
+// division per thread were half of it (n = 1023, N = 256: 11.0 ms).
+__global__ void field_kernel(int n, int N, const double* __restrict__ gx, double* __restrict__ rho) {
   const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
   const int half = (n + 1) / 2;   // rows 0 .. half; n + 1 is even
   const long total = (long)(half + 1) * (n + 2) * N;
   if (t >= total) return;
-  const long node = t / N;
-  const int j = (int)(t - node * N);
-  const int iy = (int)(node / (n + 2)), ix = (int)(node - (long)iy * (n + 2));
-  const double v = iy == 0 ? 1.0 : exp(amp * sinpi((double)iy / (double)(n + 1)) * gx[(size_t)ix * N + j]);
-  kap[((size_t)iy * (n + 2) + ix) * N + j] = v;
+  long node;
+  int j;
+  split(t, N, node, j);
+  const int iy = (int)node / (n + 2), ix = (int)node - iy * (n + 2);
+  const double v = iy == 0 ? 1.0 : exp(-(gx[(size_t)(n + 2) * N + iy] * gx[(size_t)ix * N + j]));
+  rho[((size_t)iy * (n + 2) + ix) * N + j] = v;
   const int mirror = n + 1 - iy;
-  if (mirror != iy) kap[((size_t)mirror * (n + 2) + ix) * N + j] = v;
+  if (mirror != iy) rho[((size_t)mirror * (n + 2) + ix) * N + j] = v;
+}
+
+// 2 / s for s > 0 with three FP64 instructions: r0 = 1/s in FP32 (relative
+// error e below 2^-22), then r0 (1 + e + e^2), the geometric series of 1/s up
+// to e^3 = 2^-66; the result's rounding is the only other error.  Out of the FP32 range: the division.
+__device__ __forceinline__ double two_over(double s) {
+  const float sf = narrow_rn(s);
+  if (!(sf > 1e-36f && sf < 1e36f)) return 2.0 / s;
+  const float rf = __frcp_rn(sf);
+  // rf as FP64 by bits (a normal number)
+  const unsigned b = __float_as_uint(rf);
+  const double r0 = __hiloint2double((int)((b >> 3) + (896u << 20)), (int)(b << 29));
+  const double e = fma(-s, r0, 1.0);
+  const double r = fma(r0, fma(e, e, e), r0);
+  return __hiloint2double(__double2hiint(r) + (1 << 20), __double2loint(r));
 }
 
 __device__ __forceinline__ double harmonic(double a, double b) { return 2.0 * a * b / (a + b); }
@@ -48,29 +74,33 @@ __device__ __forceinline__ double harmonic(double a, double b) { return 2.0 * a 
 // kx[iy][f][j] between grid columns f and f+1 of interior row iy (grid row iy+1);
 // ky[f][ix][j] between grid rows f and f+1 of interior column ix.
 // The FP32 copies have rows of ld32 samples, those past N the padding's kPadFace.
-__global__ void faces_kernel(int n, int N, const double* __restrict__ kap, double* __restrict__ kx64,
+// Bound by the FP64 pipe: 4 instructions per face; 2 a b / (a + b) with the
+// division took 11.5 ms at n = 1023, N = 256.
+__global__ void faces_kernel(int n, int N, const double* __restrict__ rho, double* __restrict__ kx64,
                              double* __restrict__ ky64, float* __restrict__ kx32, float* __restrict__ ky32, int ld32) {
   const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
   const long per = (long)n * (n + 1) * N;
   if (t >= 2 * per) return;
   const size_t g = (size_t)(n + 2);
   if (t < per) {
-    const long face = t / N;
-    const int j = (int)(t - face * N);
-    const int iy = (int)(face / (n + 1)), f = (int)(face - (long)iy * (n + 1));
-    const double v = harmonic(kap[((iy + 1) * g + f) * N + j], kap[((iy + 1) * g + f + 1) * N + j]);
+    long face;
+    int j;
+    split(t, N, face, j);
+    const int iy = (int)face / (n + 1), f = (int)face - iy * (n + 1);
+    const double v = two_over(rho[((iy + 1) * g + f) * N + j] + rho[((iy + 1) * g + f + 1) * N + j]);
     kx64[t] = v;
-    kx32[(size_t)face * ld32 + j] = (float)v;
+    kx32[(size_t)face * ld32 + j] = narrow_rn(v);
     if (j == N - 1)
       for (int q = N; q < ld32; ++q) kx32[(size_t)face * ld32 + q] = kPadFace;
   } else {
     const long tt = t - per;
-    const long face = tt / N;
-    const int j = (int)(tt - face * N);
-    const int f = (int)(face / n), ix = (int)(face - (long)f * n);
-    const double v = harmonic(kap[((size_t)f * g + ix + 1) * N + j], kap[((size_t)(f + 1) * g + ix + 1) * N + j]);
+    long face;
+    int j;
+    split(tt, N, face, j);
+    const int f = (int)face / n, ix = (int)face - f * n;
+    const double v = two_over(rho[((size_t)f * g + ix + 1) * N + j] + rho[((size_t)(f + 1) * g + ix + 1) * N + j]);
     ky64[tt] = v;
-    ky32[(size_t)face * ld32 + j] = (float)v;
+    ky32[(size_t)face * ld32 + j] = narrow_rn(v);
     if (j == N - 1)
       for (int q = N; q < ld32; ++q) ky32[(size_t)face * ld32 + q] = kPadFace;
   }
@@ -229,6 +259,8 @@ __global__ void mean_log_kappa_kernel(int n, int N, int K, double amp, const dou
 
 }  // namespace
 
+size_t field_scratch(int n, int N) { return ((size_t)n + 2) * (n + 2) * N + ((size_t)n + 2) * N + (size_t)n + 2; }
+
 cudaError_t launch_mean_log_kappa(int n, int N, int K, double amp, const double* xi, double* out, cudaStream_t s) {
   mean_log_kappa_kernel<<<blocks_for((long)n * n, 256), 256, 0, s>>>(n, N, K, amp, xi, out);
   count_launches(1);
@@ -249,10 +281,10 @@ cudaError_t launch_coarse_level_setup(int nf, int N, const double* kxf, const do
 cudaError_t launch_level_setup(int n, int N, int K, double amp, const double* xi, double* kap, double* kx64,
                                double* ky64, float* kx32, float* ky32, double* inva, double* isigma, double c,
                                double G, double d, double e, cudaStream_t s) {
-  // gx lives in the tail of kap's scratch: (n+2)*N doubles after the field.
+  // gx and gy live in the tail of the scratch (field_scratch), after the field.
   double* gx = kap + (size_t)(n + 2) * (n + 2) * N;
-  field_x_kernel<<<blocks_for((long)(n + 2) * N, 256), 256, 0, s>>>(n, N, K, xi, gx);
-  field_kernel<<<blocks_for((long)((n + 1) / 2 + 1) * (n + 2) * N, 256), 256, 0, s>>>(n, N, amp, gx, kap);
+  field_x_kernel<<<blocks_for((long)(n + 2) * N, 256), 256, 0, s>>>(n, N, K, amp, xi, gx);
+  field_kernel<<<blocks_for((long)((n + 1) / 2 + 1) * (n + 2) * N, 256), 256, 0, s>>>(n, N, gx, kap);
   faces_kernel<<<blocks_for(2L * n * (n + 1) * N, 256), 256, 0, s>>>(n, N, kap, kx64, ky64, kx32, ky32, N);
   diag_kernel<<<blocks_for((long)n * n * 32, 256), 256, 0, s>>>(n, N, kx64, ky64, inva, isigma, d * c * e, G);
   count_launches(4);
@@ -269,8 +301,8 @@ cudaError_t launch_diag_sum(int n, int N, const double* kx, const double* ky, do
 cudaError_t launch_field_faces(int n, int N, int K, double amp, const double* xi, double* kap, double* kx64,
                                double* ky64, float* kx32, float* ky32, int ld32, cudaStream_t s) {
   double* gx = kap + (size_t)(n + 2) * (n + 2) * N;
-  field_x_kernel<<<blocks_for((long)(n + 2) * N, 256), 256, 0, s>>>(n, N, K, xi, gx);
-  field_kernel<<<blocks_for((long)((n + 1) / 2 + 1) * (n + 2) * N, 256), 256, 0, s>>>(n, N, amp, gx, kap);
+  field_x_kernel<<<blocks_for((long)(n + 2) * N, 256), 256, 0, s>>>(n, N, K, amp, xi, gx);
+  field_kernel<<<blocks_for((long)((n + 1) / 2 + 1) * (n + 2) * N, 256), 256, 0, s>>>(n, N, gx, kap);
   faces_kernel<<<blocks_for(2L * n * (n + 1) * N, 256), 256, 0, s>>>(n, N, kap, kx64, ky64, kx32, ky32, ld32);
   count_launches(3);
   return cudaGetLastError();

@@ -19,6 +19,19 @@ namespace cmg {
 
 namespace {
 
+// On grids whose vectors exceed L2 the launches of a cycle alternate in the
+// direction in which their CTAs walk the grid (colour 0, residual,
+// prolongation, recursion forwards; colour 1 and the restriction backwards):
+// what the preceding launch touched last is read first, from L2, where a
+// fixed order always finds it just evicted.  V(2,2) cycle, forwards -> turned:
+// n = 511, N = 27 859 -> 815 us, n = 255, N = 100 633 -> 605, n = 1023, N = 256
+// 13.37 -> 13.25 ms; within L2 (n = 255, N = 64: 100 MB) it costs 1 %.
+__device__ __forceinline__ unsigned turned_block(int backwards) {
+  return backwards ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+}
+// y, p, f_y, f_p and two faces of an n x n grid against the 126 MB L2.
+bool exceeds_l2(int n, int N, size_t elem) { return (size_t)n * n * N * 6 * elem > (size_t)126 << 20; }
+
 template <typename T, int V, int SPL>
 __global__ void __launch_bounds__(kBlock) residual_kernel(LevelView<T> L, Vec3c<T> x, Vec3c<T> f, Vec3<T> r,
                                                           int lpn, T wy) {
@@ -50,9 +63,9 @@ constexpr int wide_ctas(int k) { return (sizeof(T) == 4 && V * SPL == 16) ? k : 
 
 template <typename T, int V, int SPL>
 __global__ void __launch_bounds__(kBlock, wide_ctas<T, V, SPL>(3))
-    rbgs_half_kernel(LevelView<T> L, Vec3<T> x, Vec3c<T> f, int colour, int lpn) {
+    rbgs_half_kernel(LevelView<T> L, Vec3<T> x, Vec3c<T> f, int colour, int lpn, int turned) {
   pdl_enter();
-  const long g = ((long)blockIdx.x * blockDim.x + threadIdx.x) / lpn;
+  const long g = ((long)turned_block(turned) * blockDim.x + threadIdx.x) / lpn;
   rbgs_item<T, V, SPL, false>(L, x, f, colour, g, threadIdx.x & (lpn - 1), lpn);
 }
 
@@ -85,9 +98,9 @@ __global__ void __launch_bounds__(kBlock) jacobi_update_kernel(LevelView<T> L, V
 
 template <typename T, int V, int SPL>
 __global__ void __launch_bounds__(kBlock) restrict_kernel(int nf, int N, Vec3c<T> r, Vec3<T> cv, Vec3<T> zx,
-                                                          int lpn, int colour0) {
+                                                          int lpn, int colour0, int turned) {
   pdl_enter();
-  const long node = ((long)blockIdx.x * blockDim.x + threadIdx.x) / lpn;
+  const long node = ((long)turned_block(turned) * blockDim.x + threadIdx.x) / lpn;
   restrict_item<T, V, SPL, false>(nf, N, r, cv, zx, node, threadIdx.x & (lpn - 1), lpn, colour0 != 0);
 }
 
@@ -333,7 +346,8 @@ cudaError_t launch_rbgs_half(const LevelView<T>& L, Vec3<T> x, Vec3c<T> f, int c
   }
   const long threads = (colour_count(L.n, colour)) * m.lpn;
   cudaError_t e_ = cudaSuccess;
-  CMG_DISPATCH(T, m, (e_ = launch_k(rbgs_half_kernel<T, V, SPL>, ctas_for(threads), block_for(threads), 0, st, L, x, f, colour, m.lpn)));
+  CMG_DISPATCH(T, m, (e_ = launch_k(rbgs_half_kernel<T, V, SPL>, ctas_for(threads), block_for(threads), 0, st, L, x, f, colour, m.lpn,
+                                   colour && exceeds_l2(L.n, L.N, sizeof(T)) ? 1 : 0)));
   count_launches(1);
   return e_ != cudaSuccess ? e_ : cudaGetLastError();
 }
@@ -378,7 +392,8 @@ cudaError_t launch_restrict(int nf, int N, Vec3c<T> r, Vec3<T> c, cudaStream_t s
   const SampleMap m = choose_map(N, sizeof(T), (long)nc * nc);
   const long threads = ((long)nc * nc) * m.lpn;
   cudaError_t e_ = cudaSuccess;
-  CMG_DISPATCH(T, m, (e_ = launch_k(restrict_kernel<T, V, SPL>, ctas_for(threads), block_for(threads), 0, st, nf, N, r, c, zx, m.lpn, colour0)));
+  CMG_DISPATCH(T, m, (e_ = launch_k(restrict_kernel<T, V, SPL>, ctas_for(threads), block_for(threads), 0, st, nf, N, r, c, zx, m.lpn, colour0,
+                                   exceeds_l2(nf, N, sizeof(T)) ? 1 : 0)));
   count_launches(1);
   return e_ != cudaSuccess ? e_ : cudaGetLastError();
 }
