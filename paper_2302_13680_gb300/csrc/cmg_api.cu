@@ -554,7 +554,8 @@ cudaError_t cycle(cmg_handle* h, const cmg_cycle& o, int l, Vec3<T> x, Vec3c<T> 
       const Lev& f0 = h->lv[0];
       return launch_galerkin_coarse_solve<T>(h->coarse, v.m9, f0.c, f0.d, f0.e, f, x, h->stream);
     }
-    return launch_coarse_solve<T>(coarse_for<T>(h), v.c, v.d, v.e, f, x, h->stream, o.freeze_u, N);
+    return launch_coarse_solve<T>(coarse_for<T>(h), v.c, v.d, v.e, f, x, h->stream, o.freeze_u, N,
+                                  h->L > 1);   // above the coarsest grid at least its restriction came before
   }
   cudaError_t e = cudaSuccess;
   bool fz = false;   // one-launch sweeps on this grid

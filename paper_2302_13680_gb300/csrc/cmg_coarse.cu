@@ -353,16 +353,18 @@ __device__ __forceinline__ void coarse_cta_body(const CoarseSmem<C>& S, int m, i
   }
 }
 
-// Every kernel that lets its successors start early (pdl_enter) leaves the
-// inverses alone, so they are read before the wait for the predecessor.
+// With `early` the inverses are read before the wait for the stream's
+// preceding kernel: the caller knows that it is one of the same cycle (none of
+// which writes them), not a set-up kernel.
 template <typename T, typename C>
 __global__ void __launch_bounds__(kCoarseCtaThreads) coarse_solve_cta(int m, int N, const C* __restrict__ Ainv,
                                                                      const double* __restrict__ Minv, double c,
                                                                      double d, double e, Vec3c<T> f, Vec3<T> x, int ld,
                                                                      int freeze_u, int nside, CtlBox ctl,
-                                                                     const float* __restrict__ dw) {
+                                                                     const float* __restrict__ dw, int early) {
   extern __shared__ __align__(16) double sm[];
   const CoarseSmem<C> S(sm, m, N);
+  if (!early) pdl_wait();
   S.stage(m, N, Ainv, Minv);
   pdl_enter();
   coarse_cta_body<T, C>(S, m, N, c, d, e, f, x, ld, freeze_u, nside, ctl, dw);
@@ -390,7 +392,7 @@ __global__ void cast_ainv_kernel(const double* __restrict__ a, float* __restrict
 
 template <typename T, int MM>
 cudaError_t coarse_solve_mm(const CoarseData& C, double c, double d, double e, Vec3c<T> f, Vec3<T> x,
-                            cudaStream_t s, int freeze_u, int ld) {
+                            cudaStream_t s, int freeze_u, int ld, int early) {
   using Cm = std::conditional_t<sizeof(T) == 4, float, double>;   // precision of the per-sample products
   const Cm* ainv = nullptr;
   if constexpr (sizeof(T) == 4) ainv = C.Ainv32;
@@ -405,7 +407,7 @@ cudaError_t coarse_solve_mm(const CoarseData& C, double c, double d, double e, V
     }
     const cudaError_t ek = launch_k(coarse_solve_cta<T, Cm>, dim3(1), dim3(C.N * C.m > 512 ? 1024 : 512),
                                     coarse_cta_smem<Cm>(C.N, C.m), s, C.m, C.N, ainv, (const double*)C.Minv, c, d, e,
-                                    f, x, ld, freeze_u, C.n, C.ctl, C.dw);
+                                    f, x, ld, freeze_u, C.n, C.ctl, C.dw, early);
     count_launches(1);
     return ek != cudaSuccess ? ek : cudaGetLastError();
   }
@@ -421,11 +423,11 @@ cudaError_t coarse_solve_mm(const CoarseData& C, double c, double d, double e, V
 
 template <typename T>
 cudaError_t launch_coarse_solve(const CoarseData& C, double c, double d, double e, Vec3c<T> f, Vec3<T> x,
-                                cudaStream_t s, int freeze_u, int ld) {
+                                cudaStream_t s, int freeze_u, int ld, int early) {
   if (ld == 0) ld = C.N;
-  if (C.m == 1) return coarse_solve_mm<T, 1>(C, c, d, e, f, x, s, freeze_u, ld);
-  if (C.m == 9) return coarse_solve_mm<T, 9>(C, c, d, e, f, x, s, freeze_u, ld);
-  if (C.m == 49) return coarse_solve_mm<T, 49>(C, c, d, e, f, x, s, freeze_u, ld);
+  if (C.m == 1) return coarse_solve_mm<T, 1>(C, c, d, e, f, x, s, freeze_u, ld, early);
+  if (C.m == 9) return coarse_solve_mm<T, 9>(C, c, d, e, f, x, s, freeze_u, ld, early);
+  if (C.m == 49) return coarse_solve_mm<T, 49>(C, c, d, e, f, x, s, freeze_u, ld, early);
   return cudaErrorInvalidValue;
 }
 
@@ -663,7 +665,7 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(kGalClusterThreads)
   const int j0 = min(N, (int)cl.block_rank() * per), cnt = min(N, j0 + per) - j0, nm = cnt * m;
   double *A = gsm, *fy = A + (size_t)per * mm, *w = fy + per * m, *t = w + per * m, *z = t + per * m;
   for (int i = tid; i < cnt * mm; i += kGalClusterThreads) A[i] = Ainv[(size_t)j0 * mm + i];
-  pdl_enter();   // the inverses are written by set-up kernels only
+  pdl_enter();   // A_j^{-1} is never the preceding kernel's: set-up writes M^{-1} and more after it
   for (int i = tid; i < nm; i += kGalClusterThreads) {   // f.y, f.p are [node r][sample j]
     const int r = i / cnt, q = i - r * cnt;
     fy[q * m + r] = (double)f.y[(size_t)r * N + j0 + q];
@@ -769,8 +771,8 @@ template cudaError_t launch_galerkin_coarse_solve<float>(const CoarseData&, cons
                                                          Vec3c<float>, Vec3<float>, cudaStream_t);
 
 template cudaError_t launch_coarse_solve<double>(const CoarseData&, double, double, double, Vec3c<double>,
-                                                 Vec3<double>, cudaStream_t, int, int);
+                                                 Vec3<double>, cudaStream_t, int, int, int);
 template cudaError_t launch_coarse_solve<float>(const CoarseData&, double, double, double, Vec3c<float>,
-                                                Vec3<float>, cudaStream_t, int, int);
+                                                Vec3<float>, cudaStream_t, int, int, int);
 
 }  // namespace cmg

@@ -427,7 +427,8 @@ cudaError_t launch_batch_anchor_control(const BatchTables& T, cudaStream_t s);
 // ---- coarsest grid (cmg_coarse.cu) ----
 template <typename T>
 cudaError_t launch_coarse_solve(const CoarseData& C, double c, double d, double e,
-                                Vec3c<T> f, Vec3<T> x, cudaStream_t s, int freeze_u = 0, int ld = 0);   // rows of ld (0: N)
+                                Vec3c<T> f, Vec3<T> x, cudaStream_t s, int freeze_u = 0, int ld = 0,   // rows of ld (0: N)
+                                int early = 0);   // the stream's preceding kernel is one of the same cycle
 cudaError_t launch_coarse_setup(const CoarseData& C, const double* kx, const double* ky,
                                 double c, double G, double d, double e, cudaStream_t s);
 

@@ -472,8 +472,11 @@ cmg_status cmg_unet_set(cmg_unet* u, int layer, int which, const float* host) {
   cudaError_t e = cudaMemcpyAsync(dst, host, param_elems(p, which) * 4, cudaMemcpyHostToDevice, u->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(u->stream);
   if (e != cudaSuccess) return cuda_fail(u, e, "parameter write");
-  if (which == CMG_UNET_W) NN(cmg_nn_to_bf16(p.w, p.w16, (long long)p.rows * p.cols, u->stream));
-  return CMG_OK;
+  if (which == CMG_UNET_W) {
+    NN(cmg_nn_to_bf16(p.w, p.w16, (long long)p.rows * p.cols, u->stream));
+    e = cudaStreamSynchronize(u->stream);   // the convolutions read w16 ahead of the stream's preceding kernel
+  }
+  return e == cudaSuccess ? CMG_OK : cuda_fail(u, e, "parameter write");
 }
 
 cmg_status cmg_unet_status(cmg_unet* u, int* host) {
@@ -554,6 +557,8 @@ cmg_status cmg_unet_load(cmg_unet* u, const char* path) {
     }
     NN(cmg_nn_to_bf16(p.w, p.w16, (long long)p.rows * p.cols, u->stream));
   }
+  if (const cudaError_t e = cudaStreamSynchronize(u->stream); e != cudaSuccess)   // as in cmg_unet_set
+    return cuda_fail(u, e, "checkpoint upload");
   u->step = head[2];
   u->in_scale[0] = in_scale[0];
   u->in_scale[1] = in_scale[1];
