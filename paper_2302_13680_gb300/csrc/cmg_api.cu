@@ -609,11 +609,10 @@ cudaError_t cycle(cmg_handle* h, const cmg_cycle& o, int l, Vec3<T> x, Vec3c<T> 
     if (e == cudaSuccess) e = smooth<T>(h, o, l, o.n2 - 2, x, f);
     return e;
   }
-  if (sizeof(T) == 4 && o.smoother == CMG_SMOOTH_RBGS && o.n2 >= 1 && !o.freeze_u &&
-      !(v.spl_target[1] & kTuneUnfused) && !(h->galerkin() && l > 0)) {
-    // FP32: prolongation fused into the first post-smoothing half-sweep
-    // (colour 0); identical results, one pass over x fewer.  (In FP64 the
-    // fused sweep is bound by the FP64 pipe and costs more than the pass.)
+  if (o.smoother == CMG_SMOOTH_RBGS && o.n2 >= 1 && !o.freeze_u &&
+      !(sizeof(T) == 4 && (v.spl_target[1] & kTuneUnfused)) && !(h->galerkin() && l > 0)) {
+    // prolongation fused into the first post-smoothing half-sweep
+    // (colour 0); identical results, one pass over x fewer
     const LevelView<T> L = view<T>(h, l, o.freeze_u, o.ctl32);
     {
       ProfScope ps(h, CMG_KERNEL_PROLONG, l);
@@ -1669,9 +1668,8 @@ cmg_status solve_fgmres(cmg_handle* h, const cmg_cycle& o, double tol, int maxit
       CK(launch_mdot(V, pad, k + 1, w, nt, h->red, d_h1, h->stream));
       CK(launch_maxpy(V, pad, k + 1, d_h1, -1.0, w, nt, h->stream));
       CK(launch_mdot(V, pad, k + 1, w, nt, h->red, d_h2, h->stream));
-      CK(launch_maxpy(V, pad, k + 1, d_h2, -1.0, w, nt, h->stream));
-      CK(launch_sumsq(w, nt, h->red, 0, 1.0, h->stream));
-      CK(launch_finish_sum(h->red, kRedBlocks, d_nrm, h->stream));
+      CK(launch_maxpy(V, pad, k + 1, d_h2, -1.0, w, nt, h->stream, h->red));
+      CK(launch_finish_sum(h->red, kAxpyBlocks, d_nrm, h->stream));
       CK(cudaMemcpyAsync(h->hsc, d_h1, 256 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
       CK(cudaMemcpyAsync(h->hsc + 256, d_h2, 256 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
       CK(cudaMemcpyAsync(h->hsc + 512, d_nrm, sizeof(double), cudaMemcpyDeviceToHost, h->stream));

@@ -68,29 +68,34 @@ __global__ void finish_sum_kernel(const double* __restrict__ partial, int count,
   if (threadIdx.x == 0) *out = s;
 }
 
-// Dots of up to 8 basis vectors with w per pass: w is read once per group.
+// Dots of C basis vectors with w, 16 bytes per load; n even, all vectors
+// 16-byte aligned.  Bound by the FP64 pipe from C = 2 on (one FMA per element
+// and vector at two lanes per clock and SM); C known at compile time and two
+// elements per load keep 9 loads in flight at C = 8 (8.4 M elements, 5 vectors
+// on average: 140 us with single elements and predicated vectors).
 constexpr int kDotGroup = 8;
-__global__ void __launch_bounds__(kRedThreads) mdot_kernel(const double* __restrict__ V, size_t stride, int nv,
+template <int C>
+__global__ void __launch_bounds__(kRedThreads) mdot_kernel(const double* __restrict__ V, size_t stride,
                                                            const double* __restrict__ w, size_t n,
                                                            double* __restrict__ partial) {
   __shared__ double sh[32];
-  const int g0 = blockIdx.y * kDotGroup;
-  const int cnt = min(kDotGroup, nv - g0);
-  double acc[kDotGroup];
+  double acc[C];
 #pragma unroll
-  for (int k = 0; k < kDotGroup; ++k) acc[k] = 0.0;
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const double wi = w[i];
+  for (int k = 0; k < C; ++k) acc[k] = 0.0;
+  const double2* w2 = reinterpret_cast<const double2*>(w);
+#pragma unroll(C > 4 ? 1 : 2)
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n / 2; i += (size_t)gridDim.x * blockDim.x) {
+    const double2 wi = w2[i];
+    double2 v[C];
 #pragma unroll
-    for (int k = 0; k < kDotGroup; ++k)
-      if (k < cnt) acc[k] = fma(V[(size_t)(g0 + k) * stride + i], wi, acc[k]);
+    for (int k = 0; k < C; ++k) v[k] = reinterpret_cast<const double2*>(V + (size_t)k * stride)[i];
+#pragma unroll
+    for (int k = 0; k < C; ++k) acc[k] = fma(v[k].y, wi.y, fma(v[k].x, wi.x, acc[k]));
   }
 #pragma unroll
-  for (int k = 0; k < kDotGroup; ++k) {
-    if (k < cnt) {
-      const double s = block_sum(acc[k], sh);
-      if (threadIdx.x == 0) partial[(size_t)(g0 + k) * gridDim.x + blockIdx.x] = s;
-    }
+  for (int k = 0; k < C; ++k) {
+    const double s = block_sum(acc[k], sh);
+    if (threadIdx.x == 0) partial[(size_t)k * gridDim.x + blockIdx.x] = s;
   }
 }
 
@@ -102,16 +107,36 @@ __global__ void mdot_finish_kernel(const double* __restrict__ partial, int count
   if (threadIdx.x == 0) out[blockIdx.x] = s;
 }
 
-__global__ void __launch_bounds__(kRedThreads) maxpy_kernel(const double* __restrict__ V, size_t stride, int nv,
+// w += sign * sum_{k < C} coef[k] V_k, and the partial sums of ||w||^2 where
+// partial is given (a pass over w less).  Bound by the FP64 pipe as the dots;
+// C at compile time keeps all of a pair's loads in flight (a loop over the
+// vectors, unrolled by four, took 116 us for 7 vectors of 8.4 M).
+constexpr int kAxpyGroup = 16;
+template <int C>
+__global__ void __launch_bounds__(kRedThreads) maxpy_kernel(const double* __restrict__ V, size_t stride,
                                                             const double* __restrict__ coef, double sign,
-                                                            double* __restrict__ w, size_t n) {
-  __shared__ double cs[128];
-  for (int k = threadIdx.x; k < nv; k += blockDim.x) cs[k] = sign * coef[k];
-  __syncthreads();
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    double acc = w[i];
-    for (int k = 0; k < nv; ++k) acc = fma(cs[k], V[(size_t)k * stride + i], acc);
-    w[i] = acc;
+                                                            double* __restrict__ w, size_t n,
+                                                            double* __restrict__ partial) {
+  __shared__ double sh[32];
+  double c[C], sq = 0.0;
+#pragma unroll
+  for (int k = 0; k < C; ++k) c[k] = sign * coef[k];
+#pragma unroll(C > 4 ? 1 : 2)
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n / 2; i += (size_t)gridDim.x * blockDim.x) {
+    double2 acc = reinterpret_cast<const double2*>(w)[i], v[C];
+#pragma unroll
+    for (int k = 0; k < C; ++k) v[k] = reinterpret_cast<const double2*>(V + (size_t)k * stride)[i];
+#pragma unroll
+    for (int k = 0; k < C; ++k) {
+      acc.x = fma(c[k], v[k].x, acc.x);
+      acc.y = fma(c[k], v[k].y, acc.y);
+    }
+    reinterpret_cast<double2*>(w)[i] = acc;
+    if (partial) sq = fma(acc.x, acc.x, fma(acc.y, acc.y, sq));
+  }
+  if (partial) {
+    sq = block_sum(sq, sh);
+    if (threadIdx.x == 0) partial[blockIdx.x] = sq;
   }
 }
 
@@ -174,20 +199,48 @@ cudaError_t launch_finish_sum(const double* partial, int count, double* out, cud
   return cudaGetLastError();
 }
 
+namespace {
+bool pairs(const void* a, const void* b, size_t stride, size_t n) {
+  return n % 2 == 0 && stride % 2 == 0 &&
+         ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b)) & 15) == 0;
+}
+template <int C>
+void dots(int c, const double* V, size_t stride, const double* w, size_t n, double* partial, cudaStream_t s) {
+  if constexpr (C > 1) {
+    if (c < C) return dots<C - 1>(c, V, stride, w, n, partial, s);
+  }
+  mdot_kernel<C><<<kRedBlocks, kRedThreads, 0, s>>>(V, stride, w, n, partial);
+}
+template <int C>
+void axpys(int c, const double* V, size_t stride, const double* coef, double sign, double* w, size_t n,
+           double* partial, cudaStream_t s) {
+  if constexpr (C > 1) {
+    if (c < C) return axpys<C - 1>(c, V, stride, coef, sign, w, n, partial, s);
+  }
+  maxpy_kernel<C><<<kAxpyBlocks, kRedThreads, 0, s>>>(V, stride, coef, sign, w, n, partial);
+}
+}  // namespace
+
 cudaError_t launch_mdot(const double* V, size_t stride, int nv, const double* w, size_t n, double* partial,
                         double* out, cudaStream_t s) {
-  dim3 grid(kRedBlocks, (nv + kDotGroup - 1) / kDotGroup);
-  mdot_kernel<<<grid, kRedThreads, 0, s>>>(V, stride, nv, w, n, partial);
+  if (nv < 1 || !pairs(V, w, stride, n)) return cudaErrorInvalidValue;
+  // groups of equal size, so that none reads w for a vector or two
+  const int groups = (nv + kDotGroup - 1) / kDotGroup, per = (nv + groups - 1) / groups;
+  for (int g = 0; g < nv; g += per)
+    dots<kDotGroup>(std::min(per, nv - g), V + (size_t)g * stride, stride, w, n, partial + (size_t)g * kRedBlocks, s);
   mdot_finish_kernel<<<nv, kRedThreads, 0, s>>>(partial, kRedBlocks, out);
-  count_launches(2);
+  count_launches((nv + per - 1) / per + 1);
   return cudaGetLastError();
 }
 
 cudaError_t launch_maxpy(const double* V, size_t stride, int nv, const double* coef, double sign, double* w,
-                         size_t n, cudaStream_t s) {
-  if (nv > 128) return cudaErrorInvalidValue;
-  maxpy_kernel<<<stream_blocks(n), kRedThreads, 0, s>>>(V, stride, nv, coef, sign, w, n);
-  count_launches(1);
+                         size_t n, cudaStream_t s, double* partial) {
+  if (nv < 1 || nv > 128 || !pairs(V, w, stride, n)) return cudaErrorInvalidValue;
+  const int groups = (nv + kAxpyGroup - 1) / kAxpyGroup, per = (nv + groups - 1) / groups;
+  for (int g = 0; g < nv; g += per)
+    axpys<kAxpyGroup>(std::min(per, nv - g), V + (size_t)g * stride, stride, coef + g, sign, w, n,
+                      g + per >= nv ? partial : nullptr, s);
+  count_launches((nv + per - 1) / per);
   return cudaGetLastError();
 }
 

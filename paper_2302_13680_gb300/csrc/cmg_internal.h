@@ -468,6 +468,7 @@ cudaError_t launch_diag32(int n, int N, const float* kx32, const float* ky32, in
 
 // ---- vector kernels (cmg_blas.cu) ----
 constexpr int kRedBlocks = 608;    // fixed partial count: deterministic reductions
+constexpr int kAxpyBlocks = 1216;  // partial sums of launch_maxpy
 // partial[0..kRedBlocks) (+)= w2 * per-block sums of squares; call finish to combine.
 cudaError_t launch_sumsq(const double* a, size_t n, double* partial, int accumulate, double w2, cudaStream_t s);
 // partials of wy2 ||y||^2 + ||u||^2 + ||p||^2 (ny entries in y and p, nu in u;
@@ -478,9 +479,10 @@ cudaError_t launch_finish_sum(const double* partial, int count, double* out, cud
 // out[i] = sum_k V_i[k] w[k], i < nv; V_i = V + i*stride.  partial: [nv][kRedBlocks]
 cudaError_t launch_mdot(const double* V, size_t stride, int nv, const double* w, size_t n,
                         double* partial, double* out, cudaStream_t s);
-// w += sign * sum_i coef[i] V_i  (coef on device)
+// w += sign * sum_i coef[i] V_i  (coef on device); partial: also kAxpyBlocks partial sums of ||w||^2.
+// Both: n and stride even, vectors 16-byte aligned.
 cudaError_t launch_maxpy(const double* V, size_t stride, int nv, const double* coef, double sign,
-                         double* w, size_t n, cudaStream_t s);
+                         double* w, size_t n, cudaStream_t s, double* partial = nullptr);
 // y = alpha * x (alpha read from device scalar: y = x / *den if inv)
 cudaError_t launch_scale_by(const double* x, const double* den, double* y, size_t n, cudaStream_t s);
 // y += a * x (host scalar)

@@ -61,6 +61,10 @@ __device__ __forceinline__ void fma_faces(vec<T, V>& acc, const vec<T, V>& kW, c
   }
 }
 
+__device__ __forceinline__ double flip_sign(double v) {
+  return __hiloint2double(__double2hiint(v) ^ (int)0x80000000, __double2loint(v));
+}
+
 // 1 / diag(A_j): stored (FP64 path) or from the four faces (FP32 path).
 template <typename T, int V, bool CG>
 __device__ __forceinline__ vec<T, V> inv_diag(const LevelView<T>& L, size_t off, const vec<T, V>& kW,
@@ -113,23 +117,57 @@ __device__ __forceinline__ void residual_item(const LevelView<T>& L, const Vec3c
         const vec<T, V> pS = ldx_if<T, V, CG>(hS, x.p + o - (size_t)n * ld + j);
         const vec<T, V> pN = ldx_if<T, V, CG>(hN, x.p + o + (size_t)n * ld + j);
         vec<T, V> ry, rp;
-        vec<T, V> offy = vzero<T, V>(), offp = vzero<T, V>();
-        fma_faces<T, V>(offy, kW, yW, kE, yE, kS, yS, kN, yN);
-        fma_faces<T, V>(offp, kW, pW, kE, pE, kS, pS, kN, pN);
+        if constexpr (sizeof(T) == 8) {
+          // The FP64 pipe (two lanes per clock and SM) bounds this pass: 13
+          // instructions per node-sample, one chain per row from its right
+          // side on and diag(A_j) read where it is kept (18 with separate sums
+          // of the neighbours; n = 255, N = 64: 169 us then).
+          vec<T, V> av;
+          if (L.a64) {
+            av = ldx<T, V, CG>(L.a64 + o + j);
+          } else {
 #pragma unroll
-        for (int k = 0; k < V; ++k) {
-          const T a = (kW.v[k] + kE.v[k]) + (kS.v[k] + kN.v[k]);
-          // state rows: c y + A p ; adjoint rows: A y + e u
-          ry.v[k] = c * y.v[k] + (a * p.v[k] - offp.v[k]);
-          rp.v[k] = (a * y.v[k] - offy.v[k]) + e * uu;
-          pacc += p.v[k];
-        }
-        if (!apply) {
-          const vec<T, V> fy = ldx<T, V, CG>(f.y + o + j), fp = ldx<T, V, CG>(f.p + o + j);
+            for (int k = 0; k < V; ++k) av.v[k] = (kW.v[k] + kE.v[k]) + (kS.v[k] + kN.v[k]);
+          }
+          vec<T, V> fy = vzero<T, V>(), fp = vzero<T, V>();
+          if (!apply) {
+            fy = ldx<T, V, CG>(f.y + o + j);
+            fp = ldx<T, V, CG>(f.p + o + j);
+          }
 #pragma unroll
           for (int k = 0; k < V; ++k) {
-            ry.v[k] = fy.v[k] - ry.v[k];
-            rp.v[k] = fp.v[k] - rp.v[k];
+            ry.v[k] = fma(-av.v[k], p.v[k], fma(-c, y.v[k], fy.v[k]));   // f_y - c y - A p
+            rp.v[k] = fma(-av.v[k], y.v[k], fma(-e, uu, fp.v[k]));      // f_p - e u - A y
+            pacc += p.v[k];
+          }
+          fma_faces<T, V>(ry, kW, pW, kE, pE, kS, pS, kN, pN);
+          fma_faces<T, V>(rp, kW, yW, kE, yE, kS, yS, kN, yN);
+          if (apply) {   // S x: the signs, on the integer pipe
+#pragma unroll
+            for (int k = 0; k < V; ++k) {
+              ry.v[k] = flip_sign(ry.v[k]);
+              rp.v[k] = flip_sign(rp.v[k]);
+            }
+          }
+        } else {
+          vec<T, V> offy = vzero<T, V>(), offp = vzero<T, V>();
+          fma_faces<T, V>(offy, kW, yW, kE, yE, kS, yS, kN, yN);
+          fma_faces<T, V>(offp, kW, pW, kE, pE, kS, pS, kN, pN);
+#pragma unroll
+          for (int k = 0; k < V; ++k) {
+            const T a = (kW.v[k] + kE.v[k]) + (kS.v[k] + kN.v[k]);
+            // state rows: c y + A p ; adjoint rows: A y + e u
+            ry.v[k] = c * y.v[k] + (a * p.v[k] - offp.v[k]);
+            rp.v[k] = (a * y.v[k] - offy.v[k]) + e * uu;
+            pacc += p.v[k];
+          }
+          if (!apply) {
+            const vec<T, V> fy = ldx<T, V, CG>(f.y + o + j), fp = ldx<T, V, CG>(f.p + o + j);
+#pragma unroll
+            for (int k = 0; k < V; ++k) {
+              ry.v[k] = fy.v[k] - ry.v[k];
+              rp.v[k] = fp.v[k] - rp.v[k];
+            }
           }
         }
         if (wy != T(1)) {
@@ -262,7 +300,13 @@ __device__ __forceinline__ void rbgs_node(const LevelView<T>& L, const Vec3c<T>&
 #pragma unroll
         for (int k = 0; k < V; ++k) {
           const T iak = ia[s].v[k];
-          tacc += (c * iak) * (iak * by[s].v[k]) - iak * bp[s].v[k];
+          if constexpr (sizeof(T) == 8) {
+            // bound by the FP64 pipe: 3 instructions here and 3 below instead of 5 and 4
+            by[s].v[k] *= iak;
+            tacc = fma(iak, fma(c, by[s].v[k], -bp[s].v[k]), tacc);
+          } else {
+            tacc += (c * iak) * (iak * by[s].v[k]) - iak * bp[s].v[k];
+          }
         }
       }
     }
@@ -275,7 +319,7 @@ __device__ __forceinline__ void rbgs_node(const LevelView<T>& L, const Vec3c<T>&
     // u_i = 0
     const double uu = L.freeze_u ? bu : (ctl ? su : 0.0);
     if (lane == 0 && !L.freeze_u) x.u[node] = (T)uu;
-    const T uT = (T)uu, e = (T)L.e;
+    const T uT = (T)uu, e = (T)L.e, eu = e * uT;
 #pragma unroll
     for (int s = 0; s < SPL; ++s) {
       const int j = (lane + s * lpn) * V;
@@ -283,7 +327,8 @@ __device__ __forceinline__ void rbgs_node(const LevelView<T>& L, const Vec3c<T>&
         vec<T, V> yn, pn;
 #pragma unroll
         for (int k = 0; k < V; ++k) {
-          yn.v[k] = ia[s].v[k] * (by[s].v[k] - e * uT);
+          if constexpr (sizeof(T) == 8) yn.v[k] = fma(-eu, ia[s].v[k], by[s].v[k]);
+          else yn.v[k] = ia[s].v[k] * (by[s].v[k] - e * uT);
           pn.v[k] = ia[s].v[k] * (bp[s].v[k] - c * yn.v[k]);
         }
         stv<T, V>(x.y + o + j, yn);

@@ -310,9 +310,18 @@ SampleMap choose_map(int N, int elem_bytes, long items, int spl_target) {
 
 
 
+// Chunks per lane of an FP64 residual over `nodes` nodes: four where two
+// 256-thread CTAs per SM remain (0: choose_map's rule); here they hide the
+// loads better than twice the warps (n = 255, N = 64: 141 against 186 us).
+static int residual_chunks(int N, long nodes) {
+  const long chunks = N % 2 == 0 ? N / 2 : N;
+  return chunks >= 4 && nodes * chunks >= 4 * 2L * 152 * 256 ? 4 : 0;
+}
+
 template <typename T>
 cudaError_t launch_residual(const LevelView<T>& L, Vec3c<T> x, Vec3c<T> f, Vec3<T> r, cudaStream_t st, double wy) {
-  const SampleMap m = choose_map(L.N, sizeof(T), (long)L.n * L.n, L.spl_target);
+  const SampleMap m = choose_map(L.N, sizeof(T), (long)L.n * L.n,
+                                 sizeof(T) == 8 ? residual_chunks(L.N, (long)L.n * L.n) : L.spl_target);
   const long threads = ((long)L.n * L.n) * m.lpn;
   cudaError_t e_ = cudaSuccess;
   CMG_DISPATCH(T, m, (e_ = launch_k(residual_kernel<T, V, SPL>, ctas_for(threads), block_for(threads), 0, st, L, x, f, r, m.lpn, (T)wy)));
@@ -323,7 +332,8 @@ cudaError_t launch_residual(const LevelView<T>& L, Vec3c<T> x, Vec3c<T> f, Vec3<
 template <typename T>
 cudaError_t launch_residual_c0(const LevelView<T>& L, Vec3c<T> x, Vec3c<T> f, Vec3<T> r, cudaStream_t st) {
   const long groups = colour_count(L.n, 0);
-  const SampleMap m = choose_map(L.N, sizeof(T), groups, L.spl_target);
+  const SampleMap m =
+      choose_map(L.N, sizeof(T), groups, sizeof(T) == 8 ? residual_chunks(L.N, groups) : L.spl_target);
   const long threads = (groups) * m.lpn;
   cudaError_t e_ = cudaSuccess;
   CMG_DISPATCH(T, m, (e_ = launch_k(residual_c0_kernel<T, V, SPL>, ctas_for(threads), block_for(threads), 0, st, L, x, f, r, m.lpn)));
@@ -411,10 +421,7 @@ cudaError_t launch_prolong_add(int nf, int N, Vec3c<T> e, Vec3<T> x, cudaStream_
 int launch_residual_cast(const LevelView<double>& L, Vec3c<double> x, Vec3c<double> f, Vec3<float> r, double s,
                          const double* sdev, double wy, double* partial, int max_partials, cudaStream_t st,
                          const double* gate) {
-  // four chunks per lane where two 256-thread CTAs per SM remain: here they hide
-  // the loads better than twice the warps (n = 255, N = 64: 166 against 186 us)
-  const long nodes = (long)L.n * L.n, chunks = L.N % 2 == 0 ? L.N / 2 : L.N;
-  const SampleMap m = choose_map(L.N, 8, nodes, chunks >= 4 && nodes * chunks >= 4 * 2L * 152 * 256 ? 4 : 0);
+  const SampleMap m = choose_map(L.N, 8, (long)L.n * L.n, residual_chunks(L.N, (long)L.n * L.n));
   const unsigned grid = grid_for((long)L.n * L.n, m.lpn);
   if ((int)grid > max_partials) return -1;
   const float wy2 = (float)(wy * wy);
