@@ -539,9 +539,11 @@ bool zero_guess_ok(const cmg_handle* h, const cmg_cycle& o, int l) {
 }
 
 // zg: x is logically zero on entry but its memory has not been cleared
-// (callers pass it only where zero_guess_ok holds).
+// (callers pass it only where zero_guess_ok holds); kZeroDone: the zero-guess
+// colour-0 half-sweep has been made too (by the restriction to this grid).
+enum ZeroGuess { kNoZero = 0, kZeroGuess = 1, kZeroDone = 2 };
 template <typename T>
-cudaError_t cycle(cmg_handle* h, const cmg_cycle& o, int l, Vec3<T> x, Vec3c<T> f, bool zg = false) {
+cudaError_t cycle(cmg_handle* h, const cmg_cycle& o, int l, Vec3<T> x, Vec3c<T> f, int zg = kNoZero) {
   Lev& v = h->lv[l];
   const int N = row<T>(h);
   if (o.tail_n > 0 && v.n <= o.tail_n && !h->galerkin()) {
@@ -568,7 +570,7 @@ cudaError_t cycle(cmg_handle* h, const cmg_cycle& o, int l, Vec3<T> x, Vec3c<T> 
   } else if (zg) {
     // first pre-smoothing sweep from the zero iterate
     const LevelView<T> L = view<T>(h, l, o.freeze_u, o.ctl32);
-    {
+    if (zg != kZeroDone) {
       ProfScope ps(h, CMG_KERNEL_SMOOTH, l);
       e = launch_rbgs_zero<T>(L, x, f, h->stream);
     }
@@ -595,12 +597,18 @@ cudaError_t cycle(cmg_handle* h, const cmg_cycle& o, int l, Vec3<T> x, Vec3c<T> 
   Vec3<T> fc = Work<T>::f(cl), xc = Work<T>::x(cl);
   // the coarse iterate starts at zero: cleared by the restriction unless the
   // coarse cycle's first visit does not read it
-  const bool czg = zero_guess_ok(h, o, l + 1);
+  int czg = zero_guess_ok(h, o, l + 1) ? kZeroGuess : kNoZero;
+  bool cfz = false;
+  if constexpr (sizeof(T) == 4) cfz = fused_on(h, o, l + 1);
+  if (czg && l + 1 < h->L - 1 && !cfz) czg = kZeroDone;
   {
     ProfScope ps(h, CMG_KERNEL_RESTRICT, l);
-    e = launch_restrict<T>(v.n, N, cview(r), fc, h->stream, czg ? Vec3<T>{nullptr, nullptr, nullptr} : xc, c0);
+    e = czg == kZeroDone ? launch_restrict_zero<T>(v.n, view<T>(h, l + 1, o.freeze_u, o.ctl32), cview(r), fc, xc, h->stream, c0)
+                         : launch_restrict<T>(v.n, N, cview(r), fc, h->stream,
+                                              czg ? Vec3<T>{nullptr, nullptr, nullptr} : xc, c0);
   }
-  for (int g = 0; g < o.gamma && e == cudaSuccess; ++g) e = cycle<T>(h, o, l + 1, xc, cview(fc), czg && g == 0);
+  for (int g = 0; g < o.gamma && e == cudaSuccess; ++g)
+    e = cycle<T>(h, o, l + 1, xc, cview(fc), g == 0 ? czg : kNoZero);
   if (e != cudaSuccess) return e;
   if (fz && o.n2 >= 2 && !(v.spl_target[1] & kTuneUnfused)) {
     // the first post-smoothing sweep reads its colour-1 neighbours as x + P e

@@ -228,6 +228,10 @@ cudaError_t launch_rbgs_fused(const LevelView<float>& L, Vec3c<float> xa, Vec3<f
 template <typename T>
 cudaError_t launch_restrict(int nf, int N, Vec3c<T> r, Vec3<T> c, cudaStream_t s,
                             Vec3<T> zx = Vec3<T>{nullptr, nullptr, nullptr}, int colour0 = 0);
+// The same, and the zero-guess colour-0 half-sweep of the coarse grid L on x.
+template <typename T>
+cudaError_t launch_restrict_zero(int nf, const LevelView<T>& L, Vec3c<T> r, Vec3<T> c, Vec3<T> x, cudaStream_t s,
+                                 int colour0);
 template <typename T>
 cudaError_t launch_prolong_add(int nf, int N, Vec3c<T> e, Vec3<T> x, cudaStream_t s, CtlBox ctl = CtlBox{});
 

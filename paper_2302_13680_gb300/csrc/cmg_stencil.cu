@@ -104,6 +104,22 @@ __global__ void __launch_bounds__(kBlock) restrict_kernel(int nf, int N, Vec3c<T
   restrict_item<T, V, SPL, false>(nf, N, r, cv, zx, node, threadIdx.x & (lpn - 1), lpn, colour0 != 0);
 }
 
+// The restriction, and the coarse grid's zero-guess half-sweep at its colour-0
+// nodes (see rbgs_item, ZG) by the lanes that hold their right sides: a launch
+// and a pass over the right sides fewer per grid and cycle.
+template <typename T, int V, int SPL>
+__global__ void __launch_bounds__(kBlock) restrict_zero_kernel(int nf, LevelView<T> L, Vec3c<T> r, Vec3<T> cv,
+                                                               Vec3<T> x, int lpn, int colour0, int turned) {
+  pdl_enter();
+  const long node = ((long)turned_block(turned) * blockDim.x + threadIdx.x) / lpn;
+  const int lane = threadIdx.x & (lpn - 1);
+  restrict_item<T, V, SPL, false>(nf, L.ld, r, cv, Vec3<T>{nullptr, nullptr, nullptr}, node, lane, lpn, colour0 != 0);
+  __syncwarp();   // the control right side was written by the node's first lane
+  const int J = (int)(node / L.n), I = (int)(node - (long)J * L.n);
+  rbgs_node<T, V, SPL, false, false, true>(L, cview(x), x, cview(cv), node < (long)L.n * L.n && ((J + I) & 1) == 0, J, I,
+                                           lane, lpn, Vec3c<T>{nullptr, nullptr, nullptr}, 0);
+}
+
 template <typename T, int V, int SPL>
 __global__ void __launch_bounds__(kBlock) prolong_add_kernel(int nf, int N, Vec3c<T> e, Vec3<T> x, int lpn,
                                                              CtlBox ctl) {
@@ -409,6 +425,19 @@ cudaError_t launch_restrict(int nf, int N, Vec3c<T> r, Vec3<T> c, cudaStream_t s
 }
 
 template <typename T>
+cudaError_t launch_restrict_zero(int nf, const LevelView<T>& L, Vec3c<T> r, Vec3<T> c, Vec3<T> x, cudaStream_t st,
+                                 int colour0) {
+  const long nodes = (long)L.n * L.n;
+  const SampleMap m = choose_map(L.N, sizeof(T), nodes);
+  const long threads = nodes * m.lpn;
+  cudaError_t e_ = cudaSuccess;
+  CMG_DISPATCH(T, m, (e_ = launch_k(restrict_zero_kernel<T, V, SPL>, ctas_for(threads), block_for(threads), 0, st, nf, L, r, c, x,
+                                   m.lpn, colour0, exceeds_l2(nf, L.N, sizeof(T)) ? 1 : 0)));
+  count_launches(1);
+  return e_ != cudaSuccess ? e_ : cudaGetLastError();
+}
+
+template <typename T>
 cudaError_t launch_prolong_add(int nf, int N, Vec3c<T> e, Vec3<T> x, cudaStream_t st, CtlBox ctl) {
   const SampleMap m = choose_map(N, sizeof(T), (long)nf * nf);
   const long threads = ((long)nf * nf) * m.lpn;
@@ -495,6 +524,7 @@ cudaError_t launch_axpy3(double a, const double* adev, Vec3c<float> e, Vec3<doub
   template cudaError_t launch_restrict<T>(int, int, Vec3c<T>, Vec3<T>, cudaStream_t, Vec3<T>, int);         \
   template cudaError_t launch_residual_c0<T>(const LevelView<T>&, Vec3c<T>, Vec3c<T>, Vec3<T>, cudaStream_t);       \
   template cudaError_t launch_rbgs_prolong<T>(const LevelView<T>&, Vec3<T>, Vec3c<T>, Vec3c<T>, int, cudaStream_t);                     \
+  template cudaError_t launch_restrict_zero<T>(int, const LevelView<T>&, Vec3c<T>, Vec3<T>, Vec3<T>, cudaStream_t, int);             \
   template cudaError_t launch_prolong_add<T>(int, int, Vec3c<T>, Vec3<T>, cudaStream_t, CtlBox);
 
 CMG_INST(double)
