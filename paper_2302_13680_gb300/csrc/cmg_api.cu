@@ -600,7 +600,14 @@ cudaError_t cycle(cmg_handle* h, const cmg_cycle& o, int l, Vec3<T> x, Vec3c<T> 
   int czg = zero_guess_ok(h, o, l + 1) ? kZeroGuess : kNoZero;
   bool cfz = false;
   if constexpr (sizeof(T) == 4) cfz = fused_on(h, o, l + 1);
-  if (czg && l + 1 < h->L - 1 && !cfz) czg = kZeroDone;
+  // one launch for both up to some 5 M (FP64: 1 M) coarse node-samples; on
+  // larger grids the lanes of the colour-1 nodes, idle in the half-sweep, cost
+  // more than the launch and the pass (FP32, n = 255, N = 32 coarse: 21.2
+  // against 27.7 us in two launches, n = 127, N = 256 30.2 against 35.1,
+  // n = 255, N = 128 61.3 against 57.6, n = 511, N = 256 551 against 390; FP64, n = 127,
+  // N = 32 26.9 against 28, n = 255, N = 32 82 against 70)
+  const bool small = (long)cl.n * cl.n * N <= (sizeof(T) == 8 ? 1L << 20 : 5L << 20);
+  if (czg && l + 1 < h->L - 1 && !cfz && small) czg = kZeroDone;
   {
     ProfScope ps(h, CMG_KERNEL_RESTRICT, l);
     e = czg == kZeroDone ? launch_restrict_zero<T>(v.n, view<T>(h, l + 1, o.freeze_u, o.ctl32), cview(r), fc, xc, h->stream, c0)

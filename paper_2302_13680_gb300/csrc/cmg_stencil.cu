@@ -427,9 +427,9 @@ cudaError_t launch_restrict(int nf, int N, Vec3c<T> r, Vec3<T> c, cudaStream_t s
 template <typename T>
 cudaError_t launch_restrict_zero(int nf, const LevelView<T>& L, Vec3c<T> r, Vec3<T> c, Vec3<T> x, cudaStream_t st,
                                  int colour0) {
-  const long nodes = (long)L.n * L.n;
-  const SampleMap m = choose_map(L.N, sizeof(T), nodes);
-  const long threads = nodes * m.lpn;
+  // the half-sweep's own map: the samples are summed in the order of launch_rbgs_zero
+  const SampleMap m = choose_map(L.N, sizeof(T), colour_count(L.n, 0), L.spl_target);
+  const long threads = (long)L.n * L.n * m.lpn;
   cudaError_t e_ = cudaSuccess;
   CMG_DISPATCH(T, m, (e_ = launch_k(restrict_zero_kernel<T, V, SPL>, ctas_for(threads), block_for(threads), 0, st, nf, L, r, c, x,
                                    m.lpn, colour0, exceeds_l2(nf, L.N, sizeof(T)) ? 1 : 0)));

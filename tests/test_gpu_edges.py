@@ -151,3 +151,36 @@ def test_coarsest_solve_behind_new_samples(P, fp32):
         H.cycle(opts, b, f)
         assert all(torch.equal(s, t) for s, t in zip(a, b))
     H.close()
+
+
+def test_fgmres_with_many_basis_vectors(P):
+    """A weak preconditioner: the basis passes the group sizes of the dots
+    (8) and the updates (16).  The solution at relative residual 1e-11 is the
+    cycle iteration's within 1e-7 (as for the Galerkin solutions: the control
+    block's sensitivity)."""
+    n, N = 31, 5
+    pr = inputs.make_problem(n=n, N=N, K=3, nu=1e-3, amp=0.5, seed=4, target="modes")
+    H = P.Hierarchy(n, N, pr.xi, pr.nu, pr.amp)
+    f = H.rhs(torch.tensor(pr.yd.reshape(-1), device="cuda"))
+    x, z = H.zeros(0), H.zeros(0)
+    weak = P.CycleOptions(smoother=P.SMOOTH_JACOBI, theta=0.2, n1=1, n2=0)
+    st, _ = H.solve(weak, f, x, method=P.METHOD_FGMRES, tol=1e-11, maxit=200, restart=40)
+    assert st.iters > 17
+    H.solve(P.CycleOptions(), f, z, tol=1e-12, maxit=60)
+    check(x, tuple(t.cpu().numpy() for t in z), 1e-7, "solution")
+    H.close()
+
+
+@pytest.mark.parametrize("n,N", [(255, 324), (255, 328), (127, 264), (127, 268)])
+def test_zero_guess_sweep_with_or_after_the_restriction(P, n, N):
+    """Coarse grids on both sides of the lines between one launch and two (n = 255
+    in FP32, n = 127 in FP64): FP32 against FP64 cycles from zero, 1e-4 (the
+    bound the padded rows' cycles are held to)."""
+    H = P.Hierarchy(n, N, inputs.draw_xi(N, N, 3), 1e-4, 0.5)
+    g = torch.Generator(device="cuda").manual_seed(2)
+    f = tuple(torch.randn(t.shape, generator=g, device="cuda").double() for t in H.zeros(0))
+    x, a = H.zeros(0), H.zeros(0, torch.float32)
+    H.cycle(P.CycleOptions(), x, f)
+    H.cycle(P.CycleOptions(precision=P.FP32), a, tuple(t.float() for t in f))
+    check(a, tuple(t.cpu().numpy() for t in x), 1e-4, "cycle")
+    H.close()
