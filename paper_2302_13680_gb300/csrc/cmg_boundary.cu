@@ -752,6 +752,8 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(kBT)
     t[k * m + r] = f.y[(size_t)r * N + j0 + k];
     q[k * m + r] = f.p[(size_t)r * N + j0 + k];
   }
+  // read before the cluster barriers: x may be f, and x.u is written after them
+  const double fu = tid < n ? f.u[tid] : 0.0;
   const auto product = [&](const double* mat, const double* v) {
     double s = 0.0;
     for (int k = 0; k < m; ++k) s = fma(mat[k], v[k], s);
@@ -785,7 +787,7 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(kBT)
   }
   cl.sync();   // nobody leaves while its sums are read
   if (tid < n) {   // rhs = f_u + B^T sum_j q_j
-    double s = f.u[tid];
+    double s = fu;
     for (int d = -1; d <= 1; ++d)
       if (tid + d >= 0 && tid + d < n) s += b3.w[1 - d] * us[tid + d];   // (B^T)_{k, ix} = B_{ix, k}
     rhs[tid] = s;
