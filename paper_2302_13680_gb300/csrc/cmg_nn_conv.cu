@@ -229,6 +229,9 @@ __global__ void __launch_bounds__(kConvThreads)
   } else if (warp == kProd / 32) {
     // MMA issuer.  A single commit per tile (done) frees the patch and hands the accumulator over.  Descriptors are a
     // low word (address / 16, leading offset) that advances by constants and a fixed high word.
+    // The preceding kernel first: nothing can be issued before it ends, and its time is not the waits' (their poll limit
+    // is for this launch's copies).
+    pdl_wait();
     const uint32_t idesc = instr_desc(128, NP) | (TB ? 1u << 16 : 0u);
     const uint32_t ahi = desc_hi(kIW * 16), bhi = desc_hi(TB ? (C + 1) * 16 : 128);
     const uint32_t blo = desc_lo(sB, TB ? 128 : T::kPitchB);
