@@ -717,7 +717,7 @@ __device__ __forceinline__ float recur_item(const LevelView<float>& L, const Vec
           ry.v[k] = ry.v[k] - (c * y.v[k] + ap);
           rp.v[k] = rp.v[k] - (ay + eb * uu);
           pacc += p.v[k];
-          if (V == 4 && j + k >= L.nr) ry.v[k] = rp.v[k] = 0.f;   // a padding sample: no residual (kPadFace)
+          if (V > 1 && j + k >= L.nr) ry.v[k] = rp.v[k] = 0.f;   // a padding sample: no residual (kPadFace)
           sq = fmaf(wy2 * ry.v[k], ry.v[k], sq);
           sq = fmaf(rp.v[k], rp.v[k], sq);
           dy.v[k] += y.v[k];

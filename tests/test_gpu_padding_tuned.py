@@ -1,0 +1,46 @@
+"""Launch-shape targets on sample counts whose FP32 rows are padded (N >= 9, not
+a multiple of four): the refinement's running norm is that of the real
+samples under every target.
+
+The norm decides when a true residual is taken and the solve ends: with a
+tolerance 1 % above the true residual norm after k cycles (the running norm
+follows the true one to FP32 rounding, 1e-3 at most over the first cycles) the
+solve takes k cycles.  A padding sample's residual left in the running one
+kept it above: up to five cycles more at these sizes."""
+import pytest
+import torch
+
+import inputs
+
+pytestmark = pytest.mark.gpu
+STAGED, WIDE, FUSED, TMA = 16, 32, 128, 256
+
+
+@pytest.fixture(scope="module")
+def P():
+    from paper_2302_13680_gb300 import build
+
+    build.build()
+    import paper_2302_13680_gb300 as P
+
+    return P
+
+
+def problem(P, n, N, nu=1e-2):
+    pr = inputs.make_problem(n=n, N=N, K=4, nu=nu, amp=0.5, seed=N, target="modes")
+    H = P.Hierarchy(n, N, pr.xi, pr.nu, pr.amp)
+    return H, H.rhs(torch.tensor(pr.yd.reshape(-1), device="cuda"))
+
+
+@pytest.mark.parametrize("N", [9, 10, 27, 54, 63])
+@pytest.mark.parametrize("target", [0, 1, WIDE | 1, STAGED | 1, FUSED | 1, TMA | 1],
+                         ids=["default", "1", "wide", "staged", "fused", "tma"])
+def test_running_norm_is_that_of_the_real_samples(P, N, target):
+    H, f = problem(P, 15, N)
+    H.set_tuning(P.FP32, [target] * (H.levels - 1) + [0])
+    opts = P.CycleOptions(precision=P.FP32)
+    for k in (1, 2, 3):
+        st, _ = H.solve(opts, f, H.zeros(0), tol=1e-15, maxit=k, raise_on_fail=False)
+        st, _ = H.solve(opts, f, H.zeros(0), tol=1.01 * st.relres, maxit=40)
+        assert st.iters == k
+    H.close()
