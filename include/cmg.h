@@ -382,7 +382,9 @@ cmg_status cmg_autotune(cmg_handle* h, int precision, int* chosen);
  * cmg_autotune runs): num_levels entries of 0 (size heuristic), 1, 2 or 4,
  * and for CMG_FP32 also CMG_TUNE_STAGED | 1, CMG_TUNE_STAGED | 2 or
  * CMG_TUNE_WIDE | 1 (ignored where N is odd or above 64) or CMG_TUNE_FUSED |
- * 1, 2 or 4 or CMG_TUNE_TMA | 1, 2 or 4, each possibly with CMG_TUNE_UNFUSED; NULL resets all to 0.  Other values return
+ * 1, 2 or 4 or CMG_TUNE_TMA | 1, 2 or 4, each possibly with CMG_TUNE_UNFUSED; NULL resets all to 0.  N is the
+ * problem's sample count, also where the handle pads its FP32 rows: STAGED,
+ * FUSED and TMA are ignored where it is no multiple of 4.  Other values return
  * CMG_ERR_INVALID_ARG. */
 #define CMG_TUNE_STAGED 16
 #define CMG_TUNE_WIDE 32

@@ -1229,7 +1229,11 @@ cmg_status cmg_set_tuning(cmg_handle* h, int precision, const int* spl_targets) 
                   "target must be 0, 1, 2 or 4 (FP32: or CMG_TUNE_STAGED | 1 or 2, or CMG_TUNE_WIDE | 1, or "
                   "CMG_TUNE_FUSED | 1, 2 or 4, or CMG_TUNE_TMA | 1, 2 or 4; any of them | CMG_TUNE_UNFUSED)");
   }
-  for (int l = 0; l < h->L; ++l) h->lv[l].spl_target[k] = spl_targets ? spl_targets[l] : 0;
+  // Flags that the problem's sample count does not allow are ignored: dropped here, where it is known (the FP32 views
+  // show the kernels the padded count).
+  const int N = h->prob.N;
+  const int off = (wide_supported(N) ? 0 : kTuneWide) | (N % 4 == 0 ? 0 : kTuneStaged | kTuneFused | kTuneTma);
+  for (int l = 0; l < h->L; ++l) h->lv[l].spl_target[k] = spl_targets ? spl_targets[l] & ~off : 0;
   h->ir_opts.n1 = -1;   // captured graphs bake the launch shapes: force a re-capture
   return CMG_OK;
 }

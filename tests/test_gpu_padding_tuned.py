@@ -44,3 +44,19 @@ def test_running_norm_is_that_of_the_real_samples(P, N, target):
         st, _ = H.solve(opts, f, H.zeros(0), tol=1.01 * st.relres, maxit=40)
         assert st.iters == k
     H.close()
+
+
+@pytest.mark.parametrize("N", [9, 27, 61, 63])
+@pytest.mark.parametrize("flag", [WIDE, STAGED, FUSED, TMA], ids=["wide", "staged", "fused", "tma"])
+def test_flags_go_by_the_problem_s_sample_count(P, N, flag):
+    """Ignored for an odd count (cmg.h): the same bits as without the flag,
+    where the padded count of 12 to 64 would allow it."""
+    H, f = problem(P, 31, N)
+    out = []
+    for target in (1, flag | 1):
+        H.set_tuning(P.FP32, [target] * (H.levels - 1) + [0])
+        x = H.zeros(0)
+        H.solve(P.CycleOptions(precision=P.FP32), f, x, tol=1e-15, maxit=3, raise_on_fail=False)
+        out.append(x)
+    assert all(torch.equal(a, b) for a, b in zip(*out))
+    H.close()
