@@ -326,18 +326,20 @@ SampleMap choose_map(int N, int elem_bytes, long items, int spl_target) {
 
 
 
-// Chunks per lane of an FP64 residual over `nodes` nodes: four where two
-// 256-thread CTAs per SM remain (0: choose_map's rule); here they hide the
+// Target of a residual over `nodes` nodes: the grid's (cmg_set_tuning,
+// cmg_autotune); without one in FP64, four chunks per lane where two
+// 256-thread CTAs per SM remain, else choose_map's rule: here they hide the
 // loads better than twice the warps (n = 255, N = 64: 141 against 186 us).
-static int residual_chunks(int N, long nodes) {
+static int residual_target(int N, int elem_bytes, long nodes, int spl_target) {
+  if (elem_bytes == 4 || (spl_target & 15) > 0) return spl_target;
   const long chunks = N % 2 == 0 ? N / 2 : N;
   return chunks >= 4 && nodes * chunks >= 4 * 2L * 152 * 256 ? 4 : 0;
 }
 
 template <typename T>
 cudaError_t launch_residual(const LevelView<T>& L, Vec3c<T> x, Vec3c<T> f, Vec3<T> r, cudaStream_t st, double wy) {
-  const SampleMap m = choose_map(L.N, sizeof(T), (long)L.n * L.n,
-                                 sizeof(T) == 8 ? residual_chunks(L.N, (long)L.n * L.n) : L.spl_target);
+  const long nodes = (long)L.n * L.n;
+  const SampleMap m = choose_map(L.N, sizeof(T), nodes, residual_target(L.N, sizeof(T), nodes, L.spl_target));
   const long threads = ((long)L.n * L.n) * m.lpn;
   cudaError_t e_ = cudaSuccess;
   CMG_DISPATCH(T, m, (e_ = launch_k(residual_kernel<T, V, SPL>, ctas_for(threads), block_for(threads), 0, st, L, x, f, r, m.lpn, (T)wy)));
@@ -348,8 +350,7 @@ cudaError_t launch_residual(const LevelView<T>& L, Vec3c<T> x, Vec3c<T> f, Vec3<
 template <typename T>
 cudaError_t launch_residual_c0(const LevelView<T>& L, Vec3c<T> x, Vec3c<T> f, Vec3<T> r, cudaStream_t st) {
   const long groups = colour_count(L.n, 0);
-  const SampleMap m =
-      choose_map(L.N, sizeof(T), groups, sizeof(T) == 8 ? residual_chunks(L.N, groups) : L.spl_target);
+  const SampleMap m = choose_map(L.N, sizeof(T), groups, residual_target(L.N, sizeof(T), groups, L.spl_target));
   const long threads = (groups) * m.lpn;
   cudaError_t e_ = cudaSuccess;
   CMG_DISPATCH(T, m, (e_ = launch_k(residual_c0_kernel<T, V, SPL>, ctas_for(threads), block_for(threads), 0, st, L, x, f, r, m.lpn)));
@@ -450,7 +451,7 @@ cudaError_t launch_prolong_add(int nf, int N, Vec3c<T> e, Vec3<T> x, cudaStream_
 int launch_residual_cast(const LevelView<double>& L, Vec3c<double> x, Vec3c<double> f, Vec3<float> r, double s,
                          const double* sdev, double wy, double* partial, int max_partials, cudaStream_t st,
                          const double* gate) {
-  const SampleMap m = choose_map(L.N, 8, (long)L.n * L.n, residual_chunks(L.N, (long)L.n * L.n));
+  const SampleMap m = choose_map(L.N, 8, (long)L.n * L.n, residual_target(L.N, 8, (long)L.n * L.n, 0));
   const unsigned grid = grid_for((long)L.n * L.n, m.lpn);
   if ((int)grid > max_partials) return -1;
   const float wy2 = (float)(wy * wy);
