@@ -370,12 +370,14 @@ cmg_status cmg_batch_solve(cmg_batch* b, const cmg_cycle* opts, double tol, int 
  * shared memory (CMG_TUNE_STAGED | 1 or 2 chunks), and for CMG_FP32 with N
  * even and at most 64 the layout with two samples per lane and N/2 lanes
  * (rounded up to a power of two) per node (CMG_TUNE_WIDE | 1), which applies
- * to every node kernel of that grid.  Each candidate is timed
- * with CUDA events on a few red+black sweeps on the handle's own
- * work vectors, three times in turn, and the one with the fastest median
- * time is kept in the handle.  chosen (host, may
- * be NULL) receives the target per grid (num_levels entries; the coarsest
- * is not tuned: 0).  Synchronises.  Numerical results do not depend on the
+ * to every node kernel of that grid; CMG_FP32 targets also with
+ * CMG_TUNE_UNFUSED.  Each candidate, the size rule (0) among them, is timed
+ * with CUDA events on a V(2,2) cycle's launches on that grid (sweeps, residual,
+ * prolongation) on the handle's own work vectors, three times in turn, and
+ * the one with the fastest median time is kept in the handle; the size rule
+ * where none is 1 % faster (as 1, 2 or 4 where that is the same shapes, else
+ * 0).  chosen (host, may be NULL) receives the target per grid (num_levels
+ * entries; the coarsest is not tuned: 0).  Synchronises.  Numerical results do not depend on the
  * choice except for the order of the sample sums (rounding). */
 cmg_status cmg_autotune(cmg_handle* h, int precision, int* chosen);
 /* Set the per-grid targets directly (e.g. from a cache of earlier

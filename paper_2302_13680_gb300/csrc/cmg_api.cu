@@ -10,6 +10,7 @@
 #include <vector>
 
 #include <algorithm>
+#include <array>
 #include <atomic>
 
 #include "cmg_common.cuh"
@@ -1059,69 +1060,46 @@ long long cmg_kernel_launches(void) { return cmg::g_launches.load(); }
 
 namespace {
 
-// Time `reps` red+black half-sweep pairs on grid l with chunk target t.
+// Time `reps` V(2,2) cycles' launches on grid l that go by its target t: the
+// half-sweep from zero and three sweeps less that one, the colour-0 residual,
+// and the prolongation into the first post-smoothing half-sweep or, with
+// kTuneUnfused, as a pass of its own.  On the handle's own vectors, cleared by
+// the caller.
 template <typename T>
-cmg_status time_sweeps(cmg_handle* h, int l, int t, int reps, float* ms) {
-  Lev& v = h->lv[l];
-  const int k = sizeof(T) == 8 ? 0 : 1;
-  const int saved = v.spl_target[k];
+cmg_status time_target(cmg_handle* h, int l, int t, int reps, float* ms) {
+  Lev &v = h->lv[l], &c = h->lv[l + 1];
+  const int k = sizeof(T) == 8 ? 0 : 1, saved = v.spl_target[k];
   v.spl_target[k] = t;
   const LevelView<T> L = view<T>(h, l);
-  Vec3<T> x = Work<T>::x(v), f = Work<T>::f(v);
-  cudaEvent_t e0, e1;
-  CK(cudaEventCreate(&e0));
-  CK(cudaEventCreate(&e1));
-  cudaError_t e = cudaSuccess;
-  for (int w = 0; w < 2 && e == cudaSuccess; ++w) e = launch_rbgs_half<T>(L, x, cview(f), w & 1, h->stream);
-  if (e == cudaSuccess) e = cudaEventRecord(e0, h->stream);
-  for (int r = 0; r < reps && e == cudaSuccess; ++r) {
-    e = launch_rbgs_half<T>(L, x, cview(f), 0, h->stream);
-    if (e == cudaSuccess) e = launch_rbgs_half<T>(L, x, cview(f), 1, h->stream);
-  }
-  if (e == cudaSuccess) e = cudaEventRecord(e1, h->stream);
-  if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-  if (e == cudaSuccess) e = cudaEventElapsedTime(ms, e0, e1);
-  (void)cudaEventDestroy(e0);
-  (void)cudaEventDestroy(e1);
   v.spl_target[k] = saved;
-  if (e != cudaSuccess) return cuda_fail(h, e, "autotune timing");
-  return CMG_OK;
-}
-
-// Time `reps` first post-smoothing steps on FP32 grid l (chunk target t):
-// the prolongation-fused colour-0 half-sweep + the colour-1 half-sweep, or
-// (unfused) the prolongation pass + both plain half-sweeps.
-cmg_status time_prolong(cmg_handle* h, int l, int t, int reps, bool unfused, float* ms) {
-  Lev& v = h->lv[l];
-  Lev& c = h->lv[l + 1];
-  const int saved = v.spl_target[1];
-  v.spl_target[1] = t;
-  const LevelView<float> L = view<float>(h, l);
-  Vec3<float> x = Work<float>::x(v), f = Work<float>::f(v), e = Work<float>::x(c);
-  CK(zero_vec<float>(h, l + 1, e));
-  cudaEvent_t e0, e1;
-  CK(cudaEventCreate(&e0));
-  CK(cudaEventCreate(&e1));
-  cudaError_t err = cudaSuccess;
-  for (int r = -1; r < reps && err == cudaSuccess; ++r) {   // r = -1: warm-up
-    if (r == 0) err = cudaEventRecord(e0, h->stream);
-    if (err != cudaSuccess) break;
-    if (unfused) {
-      err = launch_prolong_add<float>(v.n, h->ld32, cview(e), x, h->stream, v.ctl);
-      if (err == cudaSuccess) err = launch_rbgs_half<float>(L, x, cview(f), 0, h->stream);
+  const Vec3<T> x = Work<T>::x(v), f = Work<T>::f(v), r = Work<T>::r(v), e = Work<T>::x(c);
+  cudaEvent_t ev[2] = {nullptr, nullptr};
+  cudaError_t err = cudaEventCreate(&ev[0]);
+  if (err == cudaSuccess) err = cudaEventCreate(&ev[1]);
+  const auto go = [&](cudaError_t q) {
+    if (err == cudaSuccess) err = q;
+  };
+  for (int i = -1; i < reps && err == cudaSuccess; ++i) {   // i = -1: warm-up
+    if (i == 0) go(cudaEventRecord(ev[0], h->stream));
+    go(launch_rbgs_zero<T>(L, x, cview(f), h->stream));
+    go(launch_rbgs_half<T>(L, x, cview(f), 1, h->stream));
+    for (int colour = 0; colour < 2; ++colour) go(launch_rbgs_half<T>(L, x, cview(f), colour, h->stream));
+    go(launch_residual_c0<T>(L, cview(x), cview(f), r, h->stream));
+    if (t & kTuneUnfused) {
+      go(launch_prolong_add<T>(v.n, row<T>(h), cview(e), x, h->stream, v.ctl));
+      go(launch_rbgs_half<T>(L, x, cview(f), 0, h->stream));
     } else {
-      err = launch_rbgs_prolong<float>(L, x, cview(f), cview(e), c.n, h->stream);
+      go(launch_rbgs_prolong<T>(L, x, cview(f), cview(e), c.n, h->stream));
     }
-    if (err == cudaSuccess) err = launch_rbgs_half<float>(L, x, cview(f), 1, h->stream);
+    go(launch_rbgs_half<T>(L, x, cview(f), 1, h->stream));
+    for (int colour = 0; colour < 2; ++colour) go(launch_rbgs_half<T>(L, x, cview(f), colour, h->stream));
   }
-  if (err == cudaSuccess) err = cudaEventRecord(e1, h->stream);
-  if (err == cudaSuccess) err = cudaEventSynchronize(e1);
-  if (err == cudaSuccess) err = cudaEventElapsedTime(ms, e0, e1);
-  (void)cudaEventDestroy(e0);
-  (void)cudaEventDestroy(e1);
-  v.spl_target[1] = saved;
-  if (err != cudaSuccess) return cuda_fail(h, err, "autotune timing");
-  return CMG_OK;
+  go(cudaEventRecord(ev[1], h->stream));
+  if (err == cudaSuccess) err = cudaEventSynchronize(ev[1]);
+  if (err == cudaSuccess) err = cudaEventElapsedTime(ms, ev[0], ev[1]);
+  for (cudaEvent_t q : ev)
+    if (q) (void)cudaEventDestroy(q);
+  return err == cudaSuccess ? CMG_OK : cuda_fail(h, err, "autotune timing");
 }
 
 template <typename T>
@@ -1137,50 +1115,42 @@ cmg_status autotune_levels(cmg_handle* h, int* chosen) {
     }
     CK(zero_vec<T>(h, l, Work<T>::x(v)));
     CK(zero_vec<T>(h, l, Work<T>::f(v)));
-    const int reps = v.n >= 255 ? 8 : 16;
-    // direct-load sweeps with 1, 2, 4 chunks per lane; FP32 also the staged
-    // sweep with 1 or 2 (kTuneStaged) and the two-sample layout (kTuneWide).
-    // Three rounds over all candidates in turn; each candidate is judged by
-    // its median round (one timing per candidate was at the mercy of clock
-    // ramps and L2 state).
-    int cand[6] = {1, 2, 4, 0, 0, 0}, nc = 3;
-    if (sizeof(T) == 4 && staged_supported(h->prob.N, 1)) {
-      cand[nc++] = kTuneStaged | 1;
-      cand[nc++] = kTuneStaged | 2;
+    CK(zero_vec<T>(h, l + 1, Work<T>::x(h->lv[l + 1])));
+    const int reps = v.n >= 255 ? 2 : 6;
+    // The size rule, then 1, 2, 4 chunks per lane; FP32 also the staged sweep
+    // with 1 or 2 (kTuneStaged) and the two-sample layout (kTuneWide), and all
+    // of them with the prolongation as its own pass.  Three rounds over all
+    // candidates in turn; each candidate is judged by its median round (one
+    // timing per candidate was at the mercy of clock ramps and L2 state), on
+    // everything that its target decides: judged on plain sweeps alone, four
+    // chunks won at n = 1023, N = 256, which the fused prolongation then had to
+    // take too, and the cycle lost 10 % to the size rule.  That rule is left
+    // only for a gain of 1 %.
+    std::vector<int> cand = {0, 1, 2, 4};
+    if (sizeof(T) == 4) {
+      if (staged_supported(h->prob.N, 1)) cand.insert(cand.end(), {kTuneStaged | 1, kTuneStaged | 2});
+      if (wide_supported(h->prob.N)) cand.push_back(kTuneWide | 1);
+      for (size_t i = 0, m = cand.size(); i < m; ++i) cand.push_back(cand[i] | kTuneUnfused);
     }
-    if (sizeof(T) == 4 && wide_supported(h->prob.N)) cand[nc++] = kTuneWide | 1;
     constexpr int kRounds = 3;
-    float t_ms[kRounds][6] = {};
+    std::vector<std::array<float, kRounds>> t_ms(cand.size());
     for (int r = 0; r < kRounds; ++r)
-      for (int ci = 0; ci < nc; ++ci) {
-        const cmg_status s = time_sweeps<T>(h, l, cand[ci], reps, &t_ms[r][ci]);
+      for (size_t i = 0; i < cand.size(); ++i) {
+        const cmg_status s = time_target<T>(h, l, cand[i], reps, &t_ms[i][r]);
         if (s != CMG_OK) return s;
       }
-    float best = 1e30f;
+    const auto median = [&](size_t i) {
+      std::sort(t_ms[i].begin(), t_ms[i].end());
+      return t_ms[i][kRounds / 2];
+    };
     int best_t = 0;
-    for (int ci = 0; ci < nc; ++ci) {
-      float a = t_ms[0][ci], b = t_ms[1][ci], c = t_ms[2][ci];
-      const float med = std::max(std::min(a, b), std::min(std::max(a, b), c));
-      if (med < best) {
-        best = med;
-        best_t = cand[ci];
+    float best = 0.99f * median(0);
+    for (size_t i = 1; i < cand.size(); ++i)
+      if (const float m = median(i); m < best) {
+        best = m;
+        best_t = cand[i];
       }
-    }
-    // FP32: the prolongation fused into the first post-smoothing half-sweep
-    // or as its own pass (on large grids the fused sweep's extra coarse
-    // loads can cost more than the pass)
-    if (sizeof(T) == 4 && !h->galerkin()) {
-      float tf[kRounds] = {}, tu[kRounds] = {};
-      for (int r = 0; r < kRounds; ++r) {
-        cmg_status s = time_prolong(h, l, best_t, reps, false, &tf[r]);
-        if (s == CMG_OK) s = time_prolong(h, l, best_t, reps, true, &tu[r]);
-        if (s != CMG_OK) return s;
-      }
-      const auto med = [](const float* a) {
-        return std::max(std::min(a[0], a[1]), std::min(std::max(a[0], a[1]), a[2]));
-      };
-      if (med(tu) < med(tf)) best_t |= kTuneUnfused;
-    }
+    if ((best_t & ~kTuneUnfused) == 0) best_t |= size_rule_target(v.n, row<T>(h), sizeof(T));
     v.spl_target[k] = best_t;
     if (chosen) chosen[l] = best_t;
   }

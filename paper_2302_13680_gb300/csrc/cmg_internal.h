@@ -111,6 +111,9 @@ constexpr long kMinLanes2 = 20000;
 constexpr long kMinLanes4 = 400000;
 constexpr long kMinLanes1 = 40000;
 SampleMap choose_map(int N, int elem_bytes, long items, int spl_target = 0);
+// The explicit target (1, 2 or 4) with the shapes that target 0 gives the
+// red-black cycle's launches on an n x n grid, 0 where they differ among themselves.
+int size_rule_target(int n, int N, int elem_bytes);
 
 // Coarsest-grid factors (FP64).
 struct CoarseData {

@@ -336,6 +336,30 @@ static int residual_target(int N, int elem_bytes, long nodes, int spl_target) {
   return chunks >= 4 && nodes * chunks >= 4 * 2L * 152 * 256 ? 4 : 0;
 }
 
+// Map of the prolongation-fused half-sweep: 16 samples per lane take 128
+// registers there (the coarse loads), so eight unless the target asks for more.
+static SampleMap prolong_map(int N, int elem_bytes, long groups, int spl_target) {
+  const SampleMap m = choose_map(N, elem_bytes, groups, spl_target);
+  return m.V * m.spl > 8 && (spl_target & 15) == 0 ? choose_map(N, elem_bytes, groups, spl_target | 2) : m;
+}
+
+int size_rule_target(int n, int N, int elem_bytes) {
+  const auto same = [](const SampleMap& a, const SampleMap& b) { return a.lpn == b.lpn && a.V == b.V && a.spl == b.spl; };
+  const long c0 = colour_count(n, 0), c1 = colour_count(n, 1), all = (long)n * n;
+  for (int t : {1, 2, 4}) {
+    const auto residual = [&](long items) {
+      return same(choose_map(N, elem_bytes, items, residual_target(N, elem_bytes, items, 0)),
+                  choose_map(N, elem_bytes, items, t));
+    };
+    if (same(choose_map(N, elem_bytes, c0, 0), choose_map(N, elem_bytes, c0, t)) &&
+        same(choose_map(N, elem_bytes, c1, 0), choose_map(N, elem_bytes, c1, t)) &&
+        same(prolong_map(N, elem_bytes, c0, 0), prolong_map(N, elem_bytes, c0, t)) && residual(c0) &&
+        (elem_bytes == 4 || residual(all)))
+      return t;
+  }
+  return 0;
+}
+
 template <typename T>
 cudaError_t launch_residual(const LevelView<T>& L, Vec3c<T> x, Vec3c<T> f, Vec3<T> r, cudaStream_t st, double wy) {
   const long nodes = (long)L.n * L.n;
@@ -393,9 +417,7 @@ cudaError_t launch_rbgs_zero(const LevelView<T>& L, Vec3<T> x, Vec3c<T> f, cudaS
 template <typename T>
 cudaError_t launch_rbgs_prolong(const LevelView<T>& L, Vec3<T> x, Vec3c<T> f, Vec3c<T> e, int nc, cudaStream_t st) {
   const long groups = colour_count(L.n, 0);
-  SampleMap m = choose_map(L.N, sizeof(T), groups, L.spl_target);
-  // 16 samples per lane take 128 registers here (the coarse loads): eight then
-  if (m.V * m.spl > 8 && (L.spl_target & 15) == 0) m = choose_map(L.N, sizeof(T), groups, L.spl_target | 2);
+  const SampleMap m = prolong_map(L.N, sizeof(T), groups, L.spl_target);
   const long threads = (groups) * m.lpn;
   cudaError_t e_ = cudaSuccess;
   CMG_DISPATCH(T, m, (e_ = launch_k(rbgs_prolong_kernel<T, V, SPL>, ctas_for(threads), block_for(threads), 0, st, L, x, f, e, nc, m.lpn)));

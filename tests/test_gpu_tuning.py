@@ -51,3 +51,32 @@ def test_fp64_residual_takes_the_grid_s_target(P, N, target):
     ref = lane_sum(x[2].cpu().numpy(), *sample_map(N, 8, n * n, target))
     assert np.array_equal(r[1].cpu().numpy(), -ref / (n + 1) ** 2)
     H.close()
+
+
+@pytest.mark.parametrize("n,N,fp32", [(511, 256, True), (255, 64, True), (255, 64, False), (127, 54, True)])
+def test_autotuned_cycle_is_not_slower_than_the_default(P, n, N, fp32):
+    """The size rule is one of the tuner's candidates and all are judged on the
+    cycle's launches, so a tuned V(2,2) cycle takes at most the default's time:
+    medians of nine alternating measurements, 4 % for their spread (1 to 2 %)."""
+    H = P.Hierarchy(n, N, inputs.draw_xi(1, N, 8), 1e-5, 1.0)
+    prec, dt = (P.FP32, torch.float32) if fp32 else (P.FP64, torch.float64)
+    chosen = H.autotune(prec)
+    opts, x = P.CycleOptions(precision=prec), H.zeros(0, dt)
+    f = tuple(torch.randn_like(t) for t in x)
+    ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+    times = {True: [], False: []}
+    for i in range(20):
+        H.set_tuning(prec, chosen if i % 2 else None)
+        H.cycle(opts, x, f)
+        ev[0].record()
+        for _ in range(5):
+            H.cycle(opts, x, f)
+        ev[1].record()
+        ev[1].synchronize()
+        if i > 1:
+            times[bool(i % 2)].append(ev[0].elapsed_time(ev[1]))
+        for t in x:
+            t.zero_()
+    H.close()
+    assert chosen[-1] == 0 and all((t & ~64) in (0, 1, 2, 4, 17, 18, 33) for t in chosen)
+    assert np.median(times[True]) <= 1.04 * np.median(times[False]), (chosen, times)
