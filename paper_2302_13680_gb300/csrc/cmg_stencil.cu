@@ -300,17 +300,28 @@ SampleMap choose_map(int N, int elem_bytes, long items, int spl_target) {
   const int chunks = (N + m.V - 1) / m.V;
   // Chunks per lane by what the launch has to offer (kMinLanes*): 16 samples
   // per lane only where that still leaves a dozen waves of CTAs, 8 from a few CTAs per
-  // SM on; and at least two (four) lanes per node, else a warp's loads fall
+  // SM on; and at least two (four) lanes per node, else a warp's 16-byte loads fall
   // apart into single sectors.  FP64 takes two chunks at most: with four, the
   // registers leave the FP64 pipe too few warps (n = 255, N = 64: 96 against 81
   // us per half-sweep).  FP32 half-sweeps, 4 -> 2 chunks: n = 255, N = 64 20.8 -> 18.9 us,
   // n = 511, N = 16 50.9 -> 25.9 us; 1 -> 2: n = 127, N = 64 7.2 -> 5.5 us.
+  // Rows of a few single samples have no 16-byte loads to keep whole: up to four in a lane
+  // (FP32 sweep at n = 1023, two -> four: N = 3 64 -> 53 us, one: 107; N = 9 247 -> 172), in
+  // FP64 where that leaves fewer lanes idle (N = 5 266 -> 227, N = 9 541 -> 439, but N = 7 270 -> 302).
   int target = 1;
   if (items > 0) {
     const long lanes = items * chunks;
-    if (lanes >= 2 * kMinLanes2 && chunks >= 4) target = 2;
-    if (m.V == 1 ? lanes >= 4 * kMinLanes1 && chunks >= 16 : elem_bytes == 4 && lanes >= 4 * kMinLanes4 && chunks >= 16)
+    const auto slots = [chunks](int t) {   // lanes times the chunks that any of them takes
+      int l = 1;
+      while (l < (chunks + t - 1) / t && l < 32) l <<= 1;
+      return l * ((chunks + l - 1) / l);
+    };
+    if (lanes >= 2 * kMinLanes2 && chunks >= (m.V == 1 ? 2 : 3)) target = 2;
+    if (m.V == 1) {
+      if (lanes >= 4 * kMinLanes1 && chunks >= 2 && (chunks >= 16 || elem_bytes == 4 || slots(4) < slots(2))) target = 4;
+    } else if (elem_bytes == 4 && lanes >= 4 * kMinLanes4 && chunks >= 16) {
       target = 4;
+    }
   }
   if ((spl_target & 15) > 0) target = spl_target & 15;   // the staged and wide flags are not part of it
   const int want = (chunks + target - 1) / target;   // lanes needed at `target` chunks each
@@ -327,13 +338,14 @@ SampleMap choose_map(int N, int elem_bytes, long items, int spl_target) {
 
 
 // Target of a residual over `nodes` nodes: the grid's (cmg_set_tuning,
-// cmg_autotune); without one in FP64, four chunks per lane where two
-// 256-thread CTAs per SM remain, else choose_map's rule: here they hide the
-// loads better than twice the warps (n = 255, N = 64: 141 against 186 us).
+// cmg_autotune); without one in FP64, four chunks per lane (all of them where
+// there are fewer) where two 256-thread CTAs per SM remain, else choose_map's
+// rule: here they hide the loads better than twice the warps (n = 255, N = 64:
+// 141 against 186 us; n = 1023, N = 3 119 against 165, N = 6 215 against 292).
 static int residual_target(int N, int elem_bytes, long nodes, int spl_target) {
   if (elem_bytes == 4 || (spl_target & 15) > 0) return spl_target;
   const long chunks = N % 2 == 0 ? N / 2 : N;
-  return chunks >= 4 && nodes * chunks >= 4 * 2L * 152 * 256 ? 4 : 0;
+  return chunks >= 2 && nodes * chunks >= 4 * 2L * 152 * 256 ? 4 : 0;
 }
 
 // Map of the prolongation-fused half-sweep: 16 samples per lane take 128
