@@ -98,17 +98,22 @@ __device__ __forceinline__ void residual_item(const LevelView<T>& L, const Vec3c
   const bool ctl = L.ctl.inside(iy, ix);
   if (valid) {
     const size_t o = (size_t)node * ld;
-    const size_t lk = (size_t)L.ldk;
-    const T* kWp = L.kx + ((size_t)iy * (n + 1) + ix) * lk;
-    const T* kSp = L.ky + ((size_t)iy * n + ix) * lk;
+    // Faces by 32-bit index in the single-sample FP32 form, whose rows may differ in length from the vectors' (a caller's
+    // on padded faces): with 64-bit offsets of their own it took 327 us at n = 511, N = 125 (238 now, 257 when the rows
+    // were alike).  A handle of 2^32 faces does not fit the GPU.
+    constexpr bool kIdx = sizeof(T) == 4 && V == 1;
+    using Face = std::conditional_t<kIdx, unsigned, size_t>;
+    const Face lk = (Face)L.ldk, fx = ((Face)iy * (n + 1) + ix) * lk, fy0 = ((Face)iy * n + ix) * lk;
+    const T *kWp = L.kx + (kIdx ? 0 : fx), *kSp = L.ky + (kIdx ? 0 : fy0);
+    const Face kw = kIdx ? fx : 0, ks = kIdx ? fy0 : 0;
     const bool hW = ix > 0, hE = ix < n - 1, hS = iy > 0, hN = iy < n - 1;
     const T uu = ctl ? ld1<T, CG>(x.u + node) : T(0);
 #pragma unroll
     for (int s = 0; s < SPL; ++s) {
       const int j = (lane + s * lpn) * V;
       if (j < N) {
-        const vec<T, V> kW = ldx<T, V, CG>(kWp + j), kE = ldx<T, V, CG>(kWp + lk + j);
-        const vec<T, V> kS = ldx<T, V, CG>(kSp + j), kN = ldx<T, V, CG>(kSp + (size_t)n * lk + j);
+        const vec<T, V> kW = ldx<T, V, CG>(kWp + (kw + j)), kE = ldx<T, V, CG>(kWp + (kw + lk + j));
+        const vec<T, V> kS = ldx<T, V, CG>(kSp + (ks + j)), kN = ldx<T, V, CG>(kSp + (ks + n * lk + j));
         const vec<T, V> y = ldx<T, V, CG>(x.y + o + j), p = ldx<T, V, CG>(x.p + o + j);
         const vec<T, V> yW = ldx_if<T, V, CG>(hW, x.y + o - ld + j), yE = ldx_if<T, V, CG>(hE, x.y + o + ld + j);
         const vec<T, V> yS = ldx_if<T, V, CG>(hS, x.y + o - (size_t)n * ld + j);

@@ -60,9 +60,15 @@ __global__ void __launch_bounds__(kBlock) residual_c0_kernel(LevelView<T> L, Vec
 // (a few spilled registers cost less).
 template <typename T, int V, int SPL>
 constexpr int wide_ctas(int k) { return (sizeof(T) == 4 && V * SPL == 16) ? k : 1; }
+// The half-sweep on single samples too: 78 registers otherwise (three CTAs
+// per SM, n = 511, N = 125: 448 against 362 us), none spilled at 64.
+template <typename T, int V, int SPL>
+constexpr int half_ctas() {
+  return sizeof(T) == 4 && V == 1 && SPL > 1 ? (SPL == 8 ? 3 : 4) : wide_ctas<T, V, SPL>(3);
+}
 
 template <typename T, int V, int SPL>
-__global__ void __launch_bounds__(kBlock, wide_ctas<T, V, SPL>(3))
+__global__ void __launch_bounds__(kBlock, half_ctas<T, V, SPL>())
     rbgs_half_kernel(LevelView<T> L, Vec3<T> x, Vec3c<T> f, int colour, int lpn, int turned) {
   pdl_enter();
   const long g = ((long)turned_block(turned) * blockDim.x + threadIdx.x) / lpn;
