@@ -186,6 +186,10 @@ LevelView<float> view<float>(const cmg_handle* h, int l, int freeze_u, int ctl32
           ctl32 ? 1 : 0};
 }
 
+// Samples in a row of the handle's own vectors (raw: as a caller's).
+template <typename T>
+int row(const cmg_handle* h, bool raw = false) { return sizeof(T) == 4 && !raw ? h->ld32 : h->prob.N; }
+
 // The coarsest-grid data for a cycle of precision T; its per-node factor on d
 // is passed only while the factors are in use (else the kernels skip it).
 template <typename T>
@@ -467,10 +471,6 @@ cudaError_t smooth(cmg_handle* h, const cmg_cycle& o, int l, int sweeps, Vec3<T>
   return cudaSuccess;
 }
 
-// Samples in a row of the handle's own vectors.
-template <typename T>
-int row(const cmg_handle* h) { return sizeof(T) == 4 ? h->ld32 : h->prob.N; }
-
 // x = 0 (FP32: one of the handle's own vectors).
 template <typename T>
 cudaError_t zero_vec(cmg_handle* h, int l, Vec3<T> x) {
@@ -487,14 +487,15 @@ cudaError_t zero_vec(cmg_handle* h, int l, Vec3<T> x) {
 // The coarse-grid part of the cycle from grid l down as one cluster launch
 // (cmg_tail.cuh).  Returns cudaErrorNotSupported when not applicable.
 template <typename T>
-cudaError_t tail_cycle(cmg_handle* h, const cmg_cycle& o, int l, Vec3<T> x, Vec3c<T> f) {
+cudaError_t tail_cycle(cmg_handle* h, const cmg_cycle& o, int l, Vec3<T> x, Vec3c<T> f, bool raw) {
   const int nlev = h->L - l;
-  if (nlev > kTailMax || !tail_supported(row<T>(h), sizeof(T), h->coarse.m)) return cudaErrorNotSupported;
+  const int N = row<T>(h, raw);
+  if (nlev > kTailMax || !tail_supported(N, sizeof(T), h->coarse.m)) return cudaErrorNotSupported;
   TailParams<T> P{};
   P.nlev = nlev;
   for (int k = 0; k < nlev; ++k) {
     Lev& v = h->lv[l + k];
-    P.lev[k].L = view<T>(h, l + k, o.freeze_u, o.ctl32);
+    P.lev[k].L = view<T>(h, l + k, o.freeze_u, o.ctl32, raw);
     P.lev[k].r = Work<T>::r(v);
     if (k == 0) {
       P.lev[k].x = x;
@@ -510,8 +511,8 @@ cudaError_t tail_cycle(cmg_handle* h, const cmg_cycle& o, int l, Vec3<T> x, Vec3
   P.gamma = o.gamma;
   P.theta = o.theta;
   P.freeze_u = o.freeze_u;
-  P.lpn = choose_map(row<T>(h), sizeof(T), 0).lpn;
-  P.cld = row<T>(h);
+  P.lpn = choose_map(N, sizeof(T), 0).lpn;
+  P.cld = N;
   const CoarseData& cd = sizeof(T) == 4 ? h->c32() : h->coarse;
   P.cm = cd.m;
   P.cN = cd.N;
@@ -544,11 +545,11 @@ bool zero_guess_ok(const cmg_handle* h, const cmg_cycle& o, int l) {
 // colour-0 half-sweep has been made too (by the restriction to this grid).
 enum ZeroGuess { kNoZero = 0, kZeroGuess = 1, kZeroDone = 2 };
 template <typename T>
-cudaError_t cycle(cmg_handle* h, const cmg_cycle& o, int l, Vec3<T> x, Vec3c<T> f, int zg = kNoZero) {
+cudaError_t cycle(cmg_handle* h, const cmg_cycle& o, int l, Vec3<T> x, Vec3c<T> f, int zg = kNoZero, bool raw = false) {
   Lev& v = h->lv[l];
-  const int N = row<T>(h);
+  const int N = row<T>(h, raw);
   if (o.tail_n > 0 && v.n <= o.tail_n && !h->galerkin()) {
-    const cudaError_t e = tail_cycle<T>(h, o, l, x, f);
+    const cudaError_t e = tail_cycle<T>(h, o, l, x, f, raw);
     if (e != cudaErrorNotSupported) return e;
   }
   if (l == h->L - 1) {
@@ -567,10 +568,10 @@ cudaError_t cycle(cmg_handle* h, const cmg_cycle& o, int l, Vec3<T> x, Vec3c<T> 
     // the first pre-smoothing sweep from the zero iterate and the next one,
     // one launch each
     if constexpr (sizeof(T) == 4) e = fused_pair(h, o, l, x, f, kFusedZero);
-    if (e == cudaSuccess) e = smooth<T>(h, o, l, o.n1 - 2, x, f);
+    if (e == cudaSuccess) e = smooth<T>(h, o, l, o.n1 - 2, x, f, raw);
   } else if (zg) {
     // first pre-smoothing sweep from the zero iterate
-    const LevelView<T> L = view<T>(h, l, o.freeze_u, o.ctl32);
+    const LevelView<T> L = view<T>(h, l, o.freeze_u, o.ctl32, raw);
     if (zg != kZeroDone) {
       ProfScope ps(h, CMG_KERNEL_SMOOTH, l);
       e = launch_rbgs_zero<T>(L, x, f, h->stream);
@@ -579,9 +580,9 @@ cudaError_t cycle(cmg_handle* h, const cmg_cycle& o, int l, Vec3<T> x, Vec3c<T> 
       ProfScope ps(h, CMG_KERNEL_SMOOTH, l);
       e = launch_rbgs_half<T>(L, x, f, 1, h->stream);
     }
-    if (e == cudaSuccess) e = smooth<T>(h, o, l, o.n1 - 1, x, f);
+    if (e == cudaSuccess) e = smooth<T>(h, o, l, o.n1 - 1, x, f, raw);
   } else {
-    e = smooth<T>(h, o, l, o.n1, x, f);
+    e = smooth<T>(h, o, l, o.n1, x, f, raw);
   }
   if (e != cudaSuccess) return e;
   Vec3<T> r = Work<T>::r(v);
@@ -590,8 +591,8 @@ cudaError_t cycle(cmg_handle* h, const cmg_cycle& o, int l, Vec3<T> x, Vec3c<T> 
   const int c0 = (o.smoother == CMG_SMOOTH_RBGS && o.n1 >= 1 && !o.freeze_u && !(h->galerkin() && l > 0)) ? 1 : 0;
   {
     ProfScope ps(h, CMG_KERNEL_RESIDUAL, l);
-    e = c0 ? launch_residual_c0<T>(view<T>(h, l), cview(x), f, r, h->stream)
-           : level_residual<T>(h, l, cview(x), f, r);
+    e = c0 ? launch_residual_c0<T>(view<T>(h, l, 0, 0, raw), cview(x), f, r, h->stream)
+           : level_residual<T>(h, l, cview(x), f, r, raw);
   }
   if (e != cudaSuccess) return e;
   Lev& cl = h->lv[l + 1];
@@ -611,25 +612,25 @@ cudaError_t cycle(cmg_handle* h, const cmg_cycle& o, int l, Vec3<T> x, Vec3c<T> 
   if (czg && l + 1 < h->L - 1 && !cfz && small) czg = kZeroDone;
   {
     ProfScope ps(h, CMG_KERNEL_RESTRICT, l);
-    e = czg == kZeroDone ? launch_restrict_zero<T>(v.n, view<T>(h, l + 1, o.freeze_u, o.ctl32), cview(r), fc, xc, h->stream, c0)
+    e = czg == kZeroDone ? launch_restrict_zero<T>(v.n, view<T>(h, l + 1, o.freeze_u, o.ctl32, raw), cview(r), fc, xc, h->stream, c0)
                          : launch_restrict<T>(v.n, N, cview(r), fc, h->stream,
                                               czg ? Vec3<T>{nullptr, nullptr, nullptr} : xc, c0);
   }
   for (int g = 0; g < o.gamma && e == cudaSuccess; ++g)
-    e = cycle<T>(h, o, l + 1, xc, cview(fc), g == 0 ? czg : kNoZero);
+    e = cycle<T>(h, o, l + 1, xc, cview(fc), g == 0 ? czg : kNoZero, raw);
   if (e != cudaSuccess) return e;
   if (fz && o.n2 >= 2 && !(v.spl_target[1] & kTuneUnfused)) {
     // the first post-smoothing sweep reads its colour-1 neighbours as x + P e
     // (see below), then the next sweep, one launch each
     if constexpr (sizeof(T) == 4) e = fused_pair(h, o, l, x, f, kFusedProlong, cview(xc), cl.n);
-    if (e == cudaSuccess) e = smooth<T>(h, o, l, o.n2 - 2, x, f);
+    if (e == cudaSuccess) e = smooth<T>(h, o, l, o.n2 - 2, x, f, raw);
     return e;
   }
   if (o.smoother == CMG_SMOOTH_RBGS && o.n2 >= 1 && !o.freeze_u &&
       !(sizeof(T) == 4 && (v.spl_target[1] & kTuneUnfused)) && !(h->galerkin() && l > 0)) {
     // prolongation fused into the first post-smoothing half-sweep
     // (colour 0); identical results, one pass over x fewer
-    const LevelView<T> L = view<T>(h, l, o.freeze_u, o.ctl32);
+    const LevelView<T> L = view<T>(h, l, o.freeze_u, o.ctl32, raw);
     {
       ProfScope ps(h, CMG_KERNEL_PROLONG, l);
       e = launch_rbgs_prolong<T>(L, x, f, cview(xc), cl.n, h->stream);
@@ -638,24 +639,33 @@ cudaError_t cycle(cmg_handle* h, const cmg_cycle& o, int l, Vec3<T> x, Vec3c<T> 
       ProfScope ps(h, CMG_KERNEL_SMOOTH, l);
       e = launch_rbgs_half<T>(L, x, f, 1, h->stream);
     }
-    if (e == cudaSuccess) e = smooth<T>(h, o, l, o.n2 - 1, x, f);
+    if (e == cudaSuccess) e = smooth<T>(h, o, l, o.n2 - 1, x, f, raw);
     return e;
   }
   {
     ProfScope ps(h, CMG_KERNEL_PROLONG, l);
     e = launch_prolong_add<T>(v.n, N, cview(xc), x, h->stream, v.ctl);
   }
-  if (e == cudaSuccess) e = smooth<T>(h, o, l, o.n2, x, f);
+  if (e == cudaSuccess) e = smooth<T>(h, o, l, o.n2, x, f, raw);
   return e;
 }
 
 // One cycle on a caller's vectors.  FP32 vectors whose rows are shorter than
 // the handle's padded ones go through the finest grid's own (two copies each
-// way, some 10 % of the cycle; scalar loads on the finest grid cost 40 %).
+// way, some 10 % of the cycle; scalar loads on the finest grid cost up to 40 %),
+// except where the launches bound the cycle: there it runs on rows of N
+// throughout.  V(2,2), copies against rows of N: n = 7, N = 9 51 and 34 us (34 without
+// padding anywhere), n = 31, N = 27 110 and 83, n = 63, N = 50 148 and 137, n = 15, N = 65 87 and
+// 79, n = 255, N = 27 317 and 309; beyond the lines n = 127, N = 33 206 and 210,
+// n = 15, N = 125 90 and 97, n = 255, N = 15 257 and 259.
+inline bool rows_of_n(size_t nodes, int N) {
+  return nodes * N <= (N < 32 ? 1800000u : N < 64 ? 250000u : 15000u);
+}
 template <typename T>
 cudaError_t cycle_on(cmg_handle* h, const cmg_cycle& o, Vec3<T> x, Vec3c<T> f) {
   if constexpr (sizeof(T) == 4) {
     const int N = h->prob.N, ld = h->ld32;
+    if (ld != N && rows_of_n(h->lv[0].nodes, N)) return cycle<float>(h, o, 0, x, f, kNoZero, true);
     if (ld != N) {
       Lev& v = h->lv[0];
       const Vec3<float> xi = Work<float>::x(v), fi = Work<float>::f(v);

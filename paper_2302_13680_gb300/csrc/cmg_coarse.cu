@@ -173,6 +173,16 @@ __global__ void __launch_bounds__(kCoarseThreads) coarse_solve_a(int m, int N, c
   }
 }
 
+// The padding samples of a coarsest iterate (rows of ld): the memory may have
+// held rows of another length.
+template <typename T>
+__device__ __forceinline__ void clear_padding(const Vec3<T>& x, int m, int N, int ld, int t, int nt) {
+  for (int i = t; i < m * (ld - N); i += nt) {
+    const size_t q = (size_t)(i / (ld - N)) * ld + N + i % (ld - N);
+    x.y[q] = x.p[q] = T(0);
+  }
+}
+
 // Control solve (every CTA redundantly, fixed order) and back substitution.
 template <typename T, int MM>
 __global__ void __launch_bounds__(kCoarseThreads) coarse_solve_b(int m, int N, int nblk,
@@ -199,6 +209,7 @@ __global__ void __launch_bounds__(kCoarseThreads) coarse_solve_b(int m, int N, i
     if (blockIdx.x == 0) u[r] = (T)s;
   }
   __syncthreads();
+  if (blockIdx.x == 0) clear_padding(Vec3<T>{y, u, p}, m, N, ld, threadIdx.x, blockDim.x);
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= N) return;
   const double* A = Ainv + (size_t)j * m * m;
@@ -351,6 +362,7 @@ __device__ __forceinline__ void coarse_cta_body(const CoarseSmem<C>& S, int m, i
     for (int k = 0; k < m; ++k) t += Ar[k] * by[j * m + k];
     x.p[(size_t)r * ld + j] = (T)(w[i] - cc * t);
   }
+  clear_padding(x, m, N, ld, tid, nt);
 }
 
 // With `early` the inverses are read before the wait for the stream's

@@ -127,6 +127,10 @@ __device__ void coarse_cta(const TailParams<T>& P, const Vec3<T>& x, const Vec3<
       }
     }
   }
+  for (int i = threadIdx.x; i < m * (P.cld - N); i += blockDim.x) {   // padding samples (clear_padding, cmg_coarse.cu)
+    const size_t q = (size_t)(i / (P.cld - N)) * P.cld + N + i % (P.cld - N);
+    x.y[q] = x.p[q] = T(0);
+  }
 }
 
 // Loop of one phase: the warp's groups step through [0, count) with the
