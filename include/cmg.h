@@ -517,8 +517,8 @@ cmg_status cmg_nn_set_wait_limit(long long polls);
  * aligned), bias FP32 [Cout] or NULL, Y [B H W][Cout] BF16, all device
  * pointers.  No im2col matrix in memory; the result equals cmg_nn_im2col
  * followed by cmg_nn_gemm_bf16 bit for bit.  C = 8, 32 and 64 run on each
- * tile's input patch in shared memory; the other C read X through a TMA im2col
- * map.  Covers C a multiple of 32 (per K step of
+ * tile's input patch in shared memory, but for thin and small images, which like
+ * the other C read X through a TMA im2col map.  Covers C a multiple of 32 (per K step of
  * 64, one tensor-map load of 64 channels of a tap, or two of 32) and C = 8,
  * 16, 24 (one load per 8 channels of a tap); returns CMG_ERR_UNSUPPORTED,
  * with nothing enqueued, for other C, Cout > 64, where no tensor map can be

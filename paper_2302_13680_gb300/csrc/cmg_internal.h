@@ -585,6 +585,8 @@ cudaError_t launch_conv3x3_bf16(const void* X, int B, int H, int W, int C, const
 cudaError_t launch_conv3x3_patch(const void* X, int B, int H, int W, int C, const void* Wt, int Cout,
                                  const float* bias, int relu, int turned, void* Y16, int* status, cudaStream_t s,
                                  int early = 0);
+// Whether that kernel is the faster one for a layer it covers, against the im2col tensor map.
+bool conv3x3_patch_pays(int B, int H, int W, int C, int Cout);
 // Weight gradient of the 3x3 layer C -> Cout (C = 8, 32, 64, Cout = 32, 64) as
 // per-slice partial sums part[slices][Cout][9 C] (at most wgrad_max_slices
 // of them), added by launch_finish_layer.

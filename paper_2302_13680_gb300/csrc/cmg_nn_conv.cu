@@ -726,6 +726,25 @@ cudaError_t launch_conv3x3_wgrad(const void* X, const void* dZ, int B, int H, in
   return cudaErrorNotSupported;
 }
 
+// Times (us) by the tiles that an SM works off, fitted to 30 image shapes per
+// channel pair on a GB300, batches included: a patch tile costs a third (C =
+// 64) to an eighth (C = 8) of an im2col tile, but its 8 x 16 pixels end at the
+// image's edge while im2col tiles run on over rows and images, and C = 64
+// starts by loading 74 KB of weights.  So thin and small images stay with im2col
+// (C = Cout = 64: 64 images of 1 x 4096 343 against 59, 4096 of 4 x 4 51 against 21,
+// 8 of 40^2 10.8 against 8.4; the network's levels are on the patches' side,
+// 8 of 128^2 21 against 32).
+bool conv3x3_patch_pays(int B, int H, int W, int C, int Cout) {
+  using namespace nn;
+  const long sms = sm_count() > 0 ? sm_count() : 1;
+  const long tiles = (long)B * ((W + kPW - 1) / kPW) * ((H + kPH - 1) / kPH), dense = ((long)B * H * W + 127) / 128;
+  const double rp = (double)((tiles + sms - 1) / sms), ri = (double)((dense + sms - 1) / sms);
+  const bool narrow = Cout <= 32;
+  if (C == 8) return 3.9 + (narrow ? 0.38 : 0.48) * rp <= 4.8 + 3.0 * ri;
+  if (C == 32) return std::min(4.5 + (narrow ? 1.3 : 1.4) * rp, 10.0 + 0.68 * rp) <= 4.6 + 3.6 * ri;
+  return (2 * tiles <= sms ? 8.0 : 9.0 + 1.7 * rp) <= 4.2 + 4.1 * ri;
+}
+
 cudaError_t launch_conv3x3_patch(const void* X, int B, int H, int W, int C, const void* Wt, int Cout,
                                  const float* bias, int relu, int turned, void* Y16, int* status, cudaStream_t s, int early) {
   using namespace nn;

@@ -766,13 +766,17 @@ cudaError_t launch_conv3x3_bf16(const void* X, int B, int H, int W, int C, const
   if (!cpp || Cout < 1 || Cout > 64 || P < 1 || P > 0x7fffffffL || 9L * C > 0x7fffffffL)
     return cudaErrorNotSupported;
   // the network's channel counts: the patch kernel, which reads each pixel 1.4
-  // times instead of nine
-  const cudaError_t pe = launch_conv3x3_patch(X, B, H, W, C, Wt, Cout, bias, relu, 0, Y16, status, s);
-  if (pe != cudaErrorNotSupported) return pe;
+  // times instead of nine, where the image shape fills its tiles
+  const auto patch = [&] { return launch_conv3x3_patch(X, B, H, W, C, Wt, Cout, bias, relu, 0, Y16, status, s); };
+  const bool covered = C == 8 || C == 32 || C == 64;
+  if (covered && conv3x3_patch_pays(B, H, W, C, Cout)) {
+    const cudaError_t pe = patch();
+    if (pe != cudaErrorNotSupported) return pe;
+  }
   const int K = 9 * C;
   CUtensorMap mA, mB;
   if (!nn::im2col_map(&mA, X, B, H, W, C, cpp) || !nn::operand_map(&mB, Wt, K, Cout, K, 1, 64))
-    return cudaErrorNotSupported;
+    return covered ? patch() : cudaErrorNotSupported;
   const int vec16 = (Cout % 8 == 0) && ((reinterpret_cast<uintptr_t>(Y16) & 15) == 0);
   const nn::ConvGeom geo{H, W, C / 8, 9 * (C / 8)};
   __nv_bfloat16* y16 = static_cast<__nv_bfloat16*>(Y16);

@@ -1,10 +1,13 @@
 """Times of public calls whose launch rule or code went wrong once, against a
 device copy of the bytes the call's form moves, in the same process: medians of
 nine, the limit nearer to the faulty time than to the present one."""
+import ctypes
+
 import pytest
 import torch
 
 import inputs
+from test_gpu_nn_conv import data, lib, ptr  # noqa: F401  (module fixture)
 
 pytestmark = pytest.mark.gpu
 
@@ -52,3 +55,30 @@ def test_single_sample_rows_on_padded_faces(P):
     H.close()
     assert residual <= 1.9 * copy_micros(32 * n * n * N)
     assert sweep <= 2.2 * copy_micros(40 * n * n * N)
+
+
+@pytest.mark.parametrize("C", [8, 32, 64])
+@pytest.mark.parametrize("B,H,W", [(64, 1, 4096), (4096, 4, 4), (300, 17, 9)])
+def test_convolution_of_thin_and_small_images(lib, B, H, W, C):  # noqa: F811
+    """No slower than 96 channels in the same image shape, which always read
+    through the im2col map and do half as much work again or more (on tiles that
+    the image leaves mostly empty C = 64 took 343 us, 96 channels 75), and the
+    bits of im2col + GEMM on either route."""
+    Cout, px = 64, B * H * W
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    s = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+
+    def conv(X, Wt, bias, out):
+        assert lib.cmg_nn_conv3x3_bf16(ptr(X), B, H, W, X.shape[3], ptr(Wt), Cout, ptr(bias), 1, ptr(out), ptr(status),
+                                       s) == 0
+
+    few, many = (tuple(t.cuda() for t in data(B, H, W, c, Cout, seed=c + H)) for c in (C, 96))
+    Y, Y2 = (torch.empty(px, Cout, dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    thin, wide = micros(lambda: conv(*few, Y)), micros(lambda: conv(*many, Y2))
+    col = torch.empty(px, 9 * C, dtype=torch.bfloat16, device="cuda")
+    assert lib.cmg_nn_im2col(ptr(few[0]), ptr(col), B, H, W, C, 0, s) == 0
+    assert lib.cmg_nn_gemm_bf16(ptr(col), 9 * C, ptr(few[1]), 9 * C, px, Cout, 9 * C, ptr(few[2]), 1, None, ptr(Y2), Cout,
+                                ptr(status), s) == 0
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0 and torch.equal(Y, Y2)
+    assert thin <= wide, (thin, wide)
