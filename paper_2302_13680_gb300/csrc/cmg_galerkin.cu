@@ -606,9 +606,16 @@ cudaError_t launch_gs4_sweep(int n, int N, const T* a9, const Stencil9& M, doubl
       const int cy = col >> 1, cx = col & 1;
       const long groups = (long)((n - cx + 1) / 2) * ((n - cy + 1) / 2);
       if (groups == 0) continue;
+      // FP64 with eight samples per lane (136 registers): a launch of between half and one CTA of 256 threads per SM keeps
+      // them whole, one per SM; halves pile up on some SMs, whose FP64 pipes then end last (n = 63, N = 130: sweep 145
+      // and 102 us, FP64 V(2,2) cycle at n = 127 2190 and 2024).  With fewer samples the halves make the faster cycle
+      // (N = 33 895 and 960).
+      const long threads = groups * lpn;
+      const unsigned cta =
+          sizeof(T) == 8 && R == 8 && threads > 152L * 128 && threads <= 152L * 256 ? kGBlock : block_for(threads);
+      const unsigned ctas = (unsigned)((threads + cta - 1) / cta);
 #define CMG_GS4(RR, LL)                                                                                         \
-  err = launch_k(gs4_colour_reg_kernel<T, RR, LL>, ctas_for(groups * LL), block_for(groups * LL), 0, s, n, N, cy, cx, a9, \
-                 M, mt, G, d, e, inva, isigma, x, f)
+  err = launch_k(gs4_colour_reg_kernel<T, RR, LL>, ctas, cta, 0, s, n, N, cy, cx, a9, M, mt, G, d, e, inva, isigma, x, f)
       if (lpn == 16) {
         if (R == 1) CMG_GS4(1, 16);
         else if (R == 2) CMG_GS4(2, 16);

@@ -82,3 +82,16 @@ def test_convolution_of_thin_and_small_images(lib, B, H, W, C):  # noqa: F811
     torch.cuda.synchronize()
     assert int(status.item()) == 0 and torch.equal(Y, Y2)
     assert thin <= wide, (thin, wide)
+
+
+def test_fp64_four_colour_sweep_of_many_samples(P):
+    """Galerkin grid of 63^2 nodes: 130 samples against 64, 2.03 times the work
+    (measured 1.45 times the time; 2.05 where some SMs got three CTAs of the
+    launch and others one)."""
+    times = []
+    for N in (64, 130):
+        H = P.Hierarchy(127, N, inputs.draw_xi(1, N, 4), 1e-4, 0.5, coarse="galerkin")
+        x, f = H.zeros(1), tuple(torch.randn_like(t) for t in H.zeros(1))
+        times.append(micros(lambda: H.smooth(1, P.CycleOptions(), 1, x, f), calls=10))
+        H.close()
+    assert times[1] <= 1.8 * times[0], times
