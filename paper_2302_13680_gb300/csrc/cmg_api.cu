@@ -867,7 +867,7 @@ cmg_status cmg_create(const cmg_problem* prob, const double* xi_host, void* stre
   AL(h->coarse.Ainv32, N * h->coarse.m * h->coarse.m);
   AL(h->coarse.Minv, (size_t)h->coarse.m * h->coarse.m);
   AL(h->coarse.wz, std::max(2 * N * h->coarse.m, (size_t)h->coarse.m * h->coarse.m));
-  AL(h->coarse.partial, (size_t)h->coarse.blocks * h->coarse.m);
+  AL(h->coarse.partial, ((size_t)h->coarse.blocks + 1) * h->coarse.m);
   if (P.coarse_coeff != CMG_COARSE_NODAL) {
     h->coarse32.n = h->coarse.n;
     h->coarse32.m = h->coarse.m;
@@ -879,7 +879,7 @@ cmg_status cmg_create(const cmg_problem* prob, const double* xi_host, void* stre
     AL(h->coarse32.Ainv32, N * h->coarse.m * h->coarse.m);
     AL(h->coarse32.Minv, (size_t)h->coarse.m * h->coarse.m);
     AL(h->coarse32.wz, std::max(2 * N * h->coarse.m, (size_t)h->coarse.m * h->coarse.m));
-    AL(h->coarse32.partial, (size_t)h->coarse.blocks * h->coarse.m);
+    AL(h->coarse32.partial, ((size_t)h->coarse.blocks + 1) * h->coarse.m);
     AL(h->cface64, 2 * (size_t)cn * (cn + 1) * N);
   }
 #undef AL

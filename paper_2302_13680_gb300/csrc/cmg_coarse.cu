@@ -119,12 +119,16 @@ __global__ void invert_kernel(int m, const double* __restrict__ M, double* __res
 constexpr int kCoarseThreads = 32;   // one warp per CTA: samples spread over SMs
 
 // Per sample j: w = A_j^{-1} f_y,j, z = A_j^{-1} f_p,j, v = A_j^{-1} z;
-// per-warp partial sums of q = w - c v for the control right side.
+// per-warp partial sums of q = w - c v for the control right side, and after
+// them f_u: coarse_solve_b's CTAs all read it while one of them writes u, which
+// may be the same array.
 template <typename T, int MM>
 __global__ void __launch_bounds__(kCoarseThreads) coarse_solve_a(int m, int N, const double* __restrict__ Ainv,
                                                                 double c, const T* __restrict__ fy,
-                                                                const T* __restrict__ fp, int ld, double* __restrict__ wz,
-                                                                double* __restrict__ partial) {
+                                                                const T* __restrict__ fu, const T* __restrict__ fp, int ld,
+                                                                double* __restrict__ wz, double* __restrict__ partial) {
+  if (blockIdx.x == 0)
+    for (int r = threadIdx.x; r < m; r += blockDim.x) partial[(size_t)gridDim.x * m + r] = (double)fu[r];
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   const bool valid = j < N;
   double q[MM];
@@ -188,8 +192,7 @@ template <typename T, int MM>
 __global__ void __launch_bounds__(kCoarseThreads) coarse_solve_b(int m, int N, int nblk,
                                                                 const double* __restrict__ Ainv,
                                                                 const double* __restrict__ Minv, double c, double d,
-                                                                double e, const T* __restrict__ fu,
-                                                                const double* __restrict__ wz,
+                                                                double e, const double* __restrict__ wz,
                                                                 const double* __restrict__ partial, T* __restrict__ y,
                                                                 T* __restrict__ u, T* __restrict__ p, int ld, int freeze_u,
                                                                 int n, CtlBox ctl, const float* __restrict__ dw) {
@@ -198,7 +201,7 @@ __global__ void __launch_bounds__(kCoarseThreads) coarse_solve_b(int m, int N, i
     double s = 0.0;
     for (int b = 0; b < nblk; ++b) s += partial[(size_t)b * m + r];
     const double dr = dw ? d * (double)dw[r] : d;
-    rhs[r] = ctl.inside(r / n, r % n) ? (double)fu[r] - dr * s : 0.0;   // control rows only at control nodes
+    rhs[r] = ctl.inside(r / n, r % n) ? partial[(size_t)nblk * m + r] - dr * s : 0.0;   // control rows only at control nodes
   }
   __syncthreads();
   for (int r = threadIdx.x; r < m; r += blockDim.x) {
@@ -424,8 +427,8 @@ cudaError_t coarse_solve_mm(const CoarseData& C, double c, double d, double e, V
     return ek != cudaSuccess ? ek : cudaGetLastError();
   }
   const int nblk = (C.N + kCoarseThreads - 1) / kCoarseThreads;
-  coarse_solve_a<T, MM><<<nblk, kCoarseThreads, 0, s>>>(C.m, C.N, C.Ainv, c, f.y, f.p, ld, C.wz, C.partial);
-  coarse_solve_b<T, MM><<<nblk, kCoarseThreads, 0, s>>>(C.m, C.N, nblk, C.Ainv, C.Minv, c, d, e, f.u, C.wz,
+  coarse_solve_a<T, MM><<<nblk, kCoarseThreads, 0, s>>>(C.m, C.N, C.Ainv, c, f.y, f.u, f.p, ld, C.wz, C.partial);
+  coarse_solve_b<T, MM><<<nblk, kCoarseThreads, 0, s>>>(C.m, C.N, nblk, C.Ainv, C.Minv, c, d, e, C.wz,
                                                          C.partial, x.y, x.u, x.p, ld, freeze_u, C.n, C.ctl, C.dw);
   count_launches(2);
   return cudaGetLastError();

@@ -124,7 +124,7 @@ struct CoarseData {
   float* Ainv32;     // [N][m][m] FP32 copy for the FP32 cycle's coarse solve (may be null)
   double* Minv;      // [m][m]   inverse of the control Schur system
   double* wz;        // scratch [2][N][m] (A_j^{-1} f_y,j and A_j^{-1} f_p,j)
-  double* partial;   // scratch [blocks][m]
+  double* partial;   // scratch [blocks + 1][m]: partial sums, then f_u
   int blocks;
 };
 

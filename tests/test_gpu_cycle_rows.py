@@ -90,3 +90,19 @@ def test_padded_solve_after_a_cycle_on_rows_of_n(P, coarsest_n, tail_n):
     for x in sols[1:]:
         assert all(torch.equal(a, b) for a, b in zip(x, sols[0]))
     H.close()
+
+
+@pytest.mark.parametrize("N", [9, 27, 125, 130])
+@pytest.mark.parametrize("method", ["cycle", "fgmres"])
+def test_refined_solution_block_by_block(P, N, method):
+    """FP32 cycles on padded rows inside FP64 refinement or FGMRES, to 1e-11:
+    every block within 1e-8 of the FP64 solution."""
+    pr = inputs.make_problem(n=31, N=N, K=4, nu=1e-4, amp=0.5, seed=N, target="modes")
+    H = P.Hierarchy(31, N, pr.xi, pr.nu, pr.amp)
+    f = H.rhs(torch.tensor(pr.yd.reshape(-1), device="cuda"))
+    x, ref = H.zeros(0), H.zeros(0)
+    H.solve(P.CycleOptions(), f, ref, tol=1e-11)
+    H.solve(P.CycleOptions(precision=P.FP32), f, x, method=P.METHOD_FGMRES if method == "fgmres" else P.METHOD_CYCLE,
+            tol=1e-11)
+    close(x, ref, 1e-8)
+    H.close()
