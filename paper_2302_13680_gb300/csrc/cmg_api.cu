@@ -84,6 +84,7 @@ struct cmg_handle {
   bool g32_ready = false;      // Galerkin handles: the FP32 copies of the coarse planes are current
   CoarseData& c32() { return prob.coarse_coeff == CMG_COARSE_NODAL ? coarse : coarse32; }
   bool galerkin() const { return prob.coarse_coeff == CMG_COARSE_GALERKIN; }
+  bool galerkin_asked = false;   // also on a single grid, which has no coarse operators (cmg_create): the refusals
   int ld32 = 0;                // sample stride of the FP32 arrays (padded_samples; N unless averaged coarse grids)
   double* xi = nullptr;       // [N][K] device
   double* kap = nullptr;      // setup scratch
@@ -698,9 +699,9 @@ cmg_status check_cycle(cmg_handle* h, const cmg_cycle* o) {
   if (o->ctl32 != 0 && o->ctl32 != 1) return fail(h, CMG_ERR_INVALID_ARG, "ctl32 must be 0 or 1");
   if (o->smoother == CMG_SMOOTH_JACOBI && !(o->theta > 0.0 && o->theta <= 1.0))
     return fail(h, CMG_ERR_INVALID_ARG, "theta must be in (0, 1]");
-  if (h && h->galerkin() && o->freeze_u)
+  if (h && h->galerkin_asked && o->freeze_u)
     return fail(h, CMG_ERR_UNSUPPORTED, "Galerkin coarse operators: the control is updated in every sweep");
-  if (h && h->galerkin() && o->precision != CMG_FP64 && o->ctl32)
+  if (h && h->galerkin_asked && o->precision != CMG_FP64 && o->ctl32)
     return fail(h, CMG_ERR_UNSUPPORTED, "Galerkin coarse operators: the control row is FP64");
   return CMG_OK;
 }
@@ -753,7 +754,7 @@ cmg_status cmg_create(const cmg_problem* prob, const double* xi_host, void* stre
   if (!out) return CMG_ERR_INVALID_ARG;
   *out = nullptr;
   if (!prob) return CMG_ERR_INVALID_ARG;
-  const cmg_problem P = *prob;
+  cmg_problem P = *prob;
   const auto pow2m1 = [](int v) { return v >= 1 && ((v + 1) & v) == 0; };
   if (!pow2m1(P.n) || P.n < 3 || P.n > 4095) return CMG_ERR_INVALID_ARG;
   if (!(P.coarsest_n == 1 || P.coarsest_n == 3 || P.coarsest_n == 7) || P.coarsest_n > P.n) return CMG_ERR_INVALID_ARG;
@@ -797,6 +798,10 @@ cmg_status cmg_create(const cmg_problem* prob, const double* xi_host, void* stre
     n = (n - 1) / 2;
   }
   h->L = L;
+  // a single grid has no coarse operators, whose planes the Galerkin coarsest solve reads: its direct solve is the
+  // finest operator's, as with the other rules
+  h->galerkin_asked = P.coarse_coeff == CMG_COARSE_GALERKIN;
+  if (h->galerkin_asked && L == 1) P.coarse_coeff = h->prob.coarse_coeff = CMG_COARSE_AVERAGED;
   h->lv[0].m9.w[4] = 1.0;   // fine mass: the identity (times c, G, d, e)
   if (P.coarse_coeff == CMG_COARSE_GALERKIN) {
     const Lev& f0 = h->lv[0];
@@ -1771,7 +1776,7 @@ extern "C" cmg_status cmg_ssn_solve(cmg_handle* h, const cmg_cycle* opts, int me
       !std::isfinite(b) || !std::isfinite(beta))
     return fail(h, CMG_ERR_INVALID_ARG, "need a < 0 < b, beta >= 0, tol > 0, inner_tol > 0, maxit >= 0");
   if (opts->freeze_u) return fail(h, CMG_ERR_INVALID_ARG, "the Newton systems need the control update");
-  if (h->galerkin()) return fail(h, CMG_ERR_UNSUPPORTED, "semismooth Newton: rediscretised coarse grids only");
+  if (h->galerkin_asked) return fail(h, CMG_ERR_UNSUPPORTED, "semismooth Newton: rediscretised coarse grids only");
   if (method != CMG_METHOD_CYCLE && method != CMG_METHOD_FGMRES) return fail(h, CMG_ERR_INVALID_ARG, "unknown method");
   cmg_ssn_stats local{};
   cmg_ssn_stats* st = stats ? stats : &local;
