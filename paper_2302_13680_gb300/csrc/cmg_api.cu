@@ -10,7 +10,6 @@
 #include <vector>
 
 #include <algorithm>
-#include <array>
 #include <atomic>
 
 #include "cmg_common.cuh"
@@ -1141,27 +1140,30 @@ cmg_status autotune_levels(cmg_handle* h, int* chosen) {
     // chunks won at n = 1023, N = 256, which the fused prolongation then had to
     // take too, and the cycle lost 10 % to the size rule.  That rule is left
     // only for a gain of 1 %.
-    std::vector<int> cand = {0, 1, 2, 4};
-    if (sizeof(T) == 4) {
-      if (staged_supported(h->prob.N, 1)) cand.insert(cand.end(), {kTuneStaged | 1, kTuneStaged | 2});
-      if (wide_supported(h->prob.N)) cand.push_back(kTuneWide | 1);
-      for (size_t i = 0, m = cand.size(); i < m; ++i) cand.push_back(cand[i] | kTuneUnfused);
-    }
     constexpr int kRounds = 3;
-    std::vector<std::array<float, kRounds>> t_ms(cand.size());
+    int cand[14] = {0, 1, 2, 4}, nc = 4;
+    if (sizeof(T) == 4) {
+      if (staged_supported(h->prob.N, 1)) {
+        cand[nc++] = kTuneStaged | 1;
+        cand[nc++] = kTuneStaged | 2;
+      }
+      if (wide_supported(h->prob.N)) cand[nc++] = kTuneWide | 1;
+      for (int i = 0, m = nc; i < m; ++i) cand[nc++] = cand[i] | kTuneUnfused;
+    }
+    float t_ms[14][kRounds] = {};
     for (int r = 0; r < kRounds; ++r)
-      for (size_t i = 0; i < cand.size(); ++i) {
+      for (int i = 0; i < nc; ++i) {
         const cmg_status s = time_target<T>(h, l, cand[i], reps, &t_ms[i][r]);
         if (s != CMG_OK) return s;
       }
-    const auto median = [&](size_t i) {
-      std::sort(t_ms[i].begin(), t_ms[i].end());
-      return t_ms[i][kRounds / 2];
+    const auto median = [](float(&t)[kRounds]) {
+      std::sort(t, t + kRounds);
+      return t[kRounds / 2];
     };
     int best_t = 0;
-    float best = 0.99f * median(0);
-    for (size_t i = 1; i < cand.size(); ++i)
-      if (const float m = median(i); m < best) {
+    float best = 0.99f * median(t_ms[0]);
+    for (int i = 1; i < nc; ++i)
+      if (const float m = median(t_ms[i]); m < best) {
         best = m;
         best_t = cand[i];
       }
