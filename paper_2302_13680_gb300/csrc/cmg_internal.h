@@ -81,8 +81,9 @@ struct LevelView {
 // from the rest by 1/kPadFace (y, p of about h^2 u / kPadFace, some 1e-15 of a
 // real sample's, below half an FP32 unit of every sum over samples), and the
 // refinement keeps their residual at zero and out of its norm (recur_item).
-// N = 125 against 128 samples, scalar loads: half-sweep at n = 255 55 against
-// 41 us, V(2,2) cycle at n = 127 363 against 254 us.
+// N = 125, rows of N against padded ones: half-sweep at n = 255 55 against 41 us,
+// V(2,2) cycle on a caller's vectors at n = 31 141 against 120 us, copies
+// included (N = 250 212 against 153; small counts and grids: rows_of_n).
 constexpr float kPadFace = 1e15f;
 constexpr int kPadFrom = 8;
 inline int padded_samples(int N) { return N >= kPadFrom ? (N + 3) & ~3 : N; }

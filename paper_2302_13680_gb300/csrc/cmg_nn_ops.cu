@@ -1,10 +1,13 @@
-// Layer kernels of the warm-start network (everything except the GEMM):
-// im2col packing for 3x3 convolutions (and its transpose for weight
-// gradients), the col2im gather of data gradients, ReLU / 2x2 average
-// pooling / nearest upsampling and their gradients, BF16 casts and
-// transposes, split-K and column reductions, the masked MSE loss, AdamW, and
-// the conversions between solver grids (n x n, FP64) and the network's
-// 256 x 256 BF16 images.
+// Layer kernels of the warm-start network besides the convolutions, the head
+// (cmg_nn_conv.cu) and the GEMM: 2x2 average pooling, nearest upsampling with the
+// additive skip, the one-pass gradient of a layer's activation (resampling,
+// skip, ReLU and head gradients with the bias sums), the sums of the weight
+// gradient's slices, the masked MSE loss, AdamW, BF16 casts, and the
+// conversions between solver grids (n x n, FP64) and the network's S x S BF16
+// images.  Also the same layers one at a time (im2col and col2im, transposes,
+// flip3x3, ReLU / pooling / upsampling gradients, add, outer, column and slice
+// sums): entry points of the C ABI that the network itself does not use; the
+// gradients are tested against the chain they make.
 //
 // Activations are NHWC BF16 ([B][H][W][C], C a multiple of 8 so a 16-byte
 // chunk holds 8 channels of one pixel); convolution weights are
