@@ -62,7 +62,7 @@ def test_single_sample_rows_on_padded_faces(P):
 def test_convolution_of_thin_and_small_images(lib, B, H, W, C):  # noqa: F811
     """No slower than 96 channels in the same image shape, which always read
     through the im2col map and do half as much work again or more (on tiles that
-    the image leaves mostly empty C = 64 took 343 us, 96 channels 75), and the
+    the image leaves mostly empty C = 64 took 343 us, 96 channels 134), and the
     bits of im2col + GEMM on either route."""
     Cout, px = 64, B * H * W
     status = torch.zeros(1, dtype=torch.int32, device="cuda")
